@@ -2,15 +2,18 @@
 // one column step of R query rows owned by one lane (Sec. 2.2 Eqs. 1-3), or,
 // with split lanes, the lane's two halves of R/2 rows a column apart.
 //
-// int32 form: Algorithm 1's statements, one cell per lane op.
+// int32 form: one cell per lane op.
 // packed form: two cells per 32-bit word, each 16-bit half a signed cell value.
-// On sm_103 the integer ALU pipe (which executes every max, PRMT and IADD)
-// issues a warp instruction every second cycle, and the FMA pipe is a second
-// pipe of the same width that executes the per-half 16x2 adds (__vadd2 /
-// __vsub2).  So a word update spends its 5 maxima on the ALU pipe (the zero
-// floor of Eq. 1 is free in __vimax_s16x2_relu) and its 4 additions on the FMA
-// pipe.  Per-half adds never carry into the other half; a half whose running
-// score exceeds 32767 - max(SM) may have wrapped and is recomputed in int32.
+// On sm_103 the integer ALU pipe (which executes every maximum and PRMT)
+// issues a warp instruction every second cycle, whether a maximum has two
+// inputs, three, or an addition fused to it; the FMA pipe is a second pipe
+// that executes the per-half 16x2 adds (__vadd2 / __vsub2) and the byte dot
+// products, also every second cycle.  So a cell's cost is its instructions on
+// the ALU pipe: 3.5 (one three-input maximum for H, the zero floor of Eq. 1
+// free in it, an add-maximum each for E and F, half a three-input maximum for
+// the running best).  Per-half adds never carry into the other half; a half
+// whose running score exceeds 32767 - max(SM) may have wrapped and is
+// recomputed in int32.
 #pragma once
 
 #include <cstdint>
@@ -102,8 +105,6 @@ __host__ __device__ constexpr uint32_t sel_sext(int i) {
   return (uint32_t)i | ((uint32_t)(i | 8) << 4) | ((uint32_t)(i | 8) << 8) | ((uint32_t)(i | 8) << 12);
 }
 __host__ __device__ constexpr uint32_t sel_one(int i) { return 0x4440u | (uint32_t)i; }
-// the low 16-bit half of a, sign-extended to 32 bits
-__host__ __device__ constexpr uint32_t sel_sext16() { return 0x9910u; }
 
 // R 32-bit profile entries of one residue in the wide layout (R/4 16-byte
 // groups, `gstride` bytes apart: the lanes' groups interleaved)
@@ -164,32 +165,34 @@ __device__ __forceinline__ uint32_t word_of(const uint4 &v, int i) {
 // N rows [R0, R0 + N) of one column, 32-bit words of two 16-bit cells
 // (Eqs. 1-3 per half).  hd0 is H of the row above R0 at the previous column,
 // p the rows' substitution words; E (per row, this column) and f (passed down
-// the column) are updated in place, S keeps the running best.  Per word five
-// maxima, the zero floor riding on the one with F, and four per-half
-// additions, H - Go shared by the E and F updates.  The terms that do not
-// depend on the row above, max(H_diag + SM, E), are formed for all N rows
-// first: the previous column's H is then dead before any row is rewritten
-// (no register copies), and only max(., F), the subtraction and the F update
-// remain on the chain down the rows.  (Computing the next F from
-// max(hd + p, E, 0) - Go instead of H - Go, which is equal because Ge <= Go,
-// shortens that chain further but costs a fifth addition and measured
-// slower.)
+// the column) are updated in place, S keeps the running best.
+//
+// Per word: H = max(H_diag + SM, E, F, 0) is one three-input maximum with the
+// zero floor, the E and F updates one add-maximum each, and the running best
+// one three-input maximum per two rows: 3.5 instructions on the ALU pipe
+// (each a warp instruction every second cycle, three-input or not); H_diag +
+// SM and H - Go (shared by E and F) are per-half adds on the FMA pipe.  All
+// H_diag + SM are formed first: the previous column's H is then dead before
+// any row is rewritten (forming them row by row costs a register copy each).
+// Two-input maxima throughout (5 on the ALU pipe) took 10.3 cycles per word
+// and SM sub-partition in a loop over 24 rows and four warps, this order 9.1
+// (the ALU pipe 79 % busy; register operands, up to three per instruction,
+// are the rest), and the same formed row by row 10.2-10.6.
 template <int R0, int N, int R>
 __device__ __forceinline__ void word_rows(uint32_t hd0, const uint32_t (&p)[N], uint32_t (&E)[R],
                                           uint32_t (&Hl)[R], uint32_t &f, uint32_t &S, const Consts &cs) {
-  static_assert(R0 + N <= R, "rows in range");
-  uint32_t tt[N];
-  tt[0] = __vmaxs2(__vadd2(hd0, p[0]), E[R0]);
+  static_assert(R0 + N <= R && N % 2 == 0, "rows in range, whole pairs of rows");
+  uint32_t x[N];
 #pragma unroll
-  for (int r = 1; r < N; ++r) tt[r] = __vmaxs2(__vadd2(Hl[R0 + r - 1], p[r]), E[R0 + r]);
+  for (int r = N - 1; r >= 0; --r) x[r] = __vadd2(r > 0 ? Hl[R0 + r - 1] : hd0, p[r]);
 #pragma unroll
   for (int r = 0; r < N; ++r) {
-    const uint32_t h = __vimax_s16x2_relu(tt[r], f);  // max(H_diag + SM, E, F, 0)
-    S = __vmaxs2(S, h);
+    const uint32_t h = __vimax3_s16x2_relu(x[r], E[R0 + r], f);  // max(H_diag + SM, E, F, 0)
     const uint32_t hgo = __vsub2(h, cs.goW);
     E[R0 + r] = __vmaxs2(__vsub2(E[R0 + r], cs.geW), hgo);
     f = __vmaxs2(__vsub2(f, cs.geW), hgo);
     Hl[R0 + r] = h;
+    if (r & 1) S = __vimax3_s16x2(S, Hl[R0 + r - 1], h);
   }
 }
 
@@ -199,108 +202,88 @@ __device__ __forceinline__ void word_rows(uint32_t hd0, const uint32_t (&p)[N], 
 // depend on the row above; since Ge <= Go, the F passed down is
 // max(F - Ge, H - Go) = max(F - Ge, U - Go, F - Go) = max(F - Ge, U - Go), so
 // the only operation on the chain is that max-add, and H = max(U, F), the
-// running best and E' = max(E - Ge, H - Go) hang off it.  Same five maxima
-// per word as word_rows, one more addition (U - Go beside H - Go).
+// running best and E' = max(E - Ge, H - Go) hang off it.  One more maximum
+// and one more addition per word than word_rows.
 template <int R0, int N, int R>
 __device__ __forceinline__ void word_rows_short(uint32_t hd0, const uint32_t (&p)[N], uint32_t (&E)[R],
                                                 uint32_t (&Hl)[R], uint32_t &f, uint32_t &S, const Consts &cs) {
-  static_assert(R0 + N <= R, "rows in range");
+  static_assert(R0 + N <= R && N % 2 == 0, "rows in range, whole pairs of rows");
   uint32_t u[N];
-  u[0] = __vimax_s16x2_relu(__vadd2(hd0, p[0]), E[R0]);  // max(H_diag + SM, E, 0)
 #pragma unroll
-  for (int r = 1; r < N; ++r) u[r] = __vimax_s16x2_relu(__vadd2(Hl[R0 + r - 1], p[r]), E[R0 + r]);
+  for (int r = N - 1; r >= 0; --r)
+    u[r] = __vimax_s16x2_relu(__vadd2(r > 0 ? Hl[R0 + r - 1] : hd0, p[r]), E[R0 + r]);  // max(H_diag + SM, E, 0)
 #pragma unroll
   for (int r = 0; r < N; ++r) {
     const uint32_t h = __vmaxs2(u[r], f);  // H = max(U, F)
     f = __vmaxs2(__vsub2(f, cs.geW), __vsub2(u[r], cs.goW));
-    S = __vmaxs2(S, h);
     E[R0 + r] = __vmaxs2(__vsub2(E[R0 + r], cs.geW), __vsub2(h, cs.goW));
     Hl[R0 + r] = h;
+    if (r & 1) S = __vimax3_s16x2(S, Hl[R0 + r - 1], h);
   }
 }
 
 template <int FORM>
 using Word = typename std::conditional<FORM != kFormInt32, uint32_t, int32_t>::type;
 
-// N rows [R0, R0 + N) of one column in int32, Algorithm 1 statement by
-// statement.  hul is H of the row above R0 at the previous column, (hu, fu) H
-// and F of that row at this column (replaced by those of row R0 + N - 1); pb
-// the rows' profile bytes, four per word; E and Hl hold the previous column's
-// E and H per row and are updated in place; S keeps the running best.
-// sm_of(r): the substitution score of row R0 + r (one sign extension on the
-// ALU pipe from a profile byte, or from the low half of a 32-bit entry).
-template <int R0, int N, int R, class SmOf>
-__device__ __forceinline__ void int_rows_of(int32_t hul, SmOf sm_of, int32_t (&E)[R], int32_t (&Hl)[R], int32_t &hu,
-                                            int32_t &fu, int32_t &S, const Consts &cs) {
-  static_assert(R0 + N <= R, "rows in range");
+// The rows of word_rows in int32 cells (Algorithm 1, one cell per lane op).
+// add(r, h): h plus the substitution score of row R0 + r.
+// Per cell 3.5 instructions on the ALU pipe like a word of word_rows; the
+// score is added by a byte dot product (FMA pipe), which sign-extends it on
+// the way.  Statement by statement with two-input maxima and a byte
+// extraction on the ALU pipe: 11.3 cycles per cell and SM sub-partition in a
+// loop over 24 rows and four warps; three-input maxima 9.45; with the dot
+// product 7.9 (the ALU pipe 89 % busy).
+template <int R0, int N, int R, class Add>
+__device__ __forceinline__ void int_rows_of(int32_t hd0, Add add, int32_t (&E)[R], int32_t (&Hl)[R], int32_t &f,
+                                            int32_t &S, const Consts &cs) {
+  static_assert(R0 + N <= R && N % 2 == 0, "rows in range, whole pairs of rows");
+  int32_t x[N];
+#pragma unroll
+  for (int r = N - 1; r >= 0; --r) x[r] = add(r, r > 0 ? Hl[R0 + r - 1] : hd0);
 #pragma unroll
   for (int r = 0; r < N; ++r) {
-    const int32_t sm = sm_of(r);
-    const int32_t e1 = E[R0 + r] - cs.ge;
-    const int32_t e2 = Hl[R0 + r] - cs.go;
-    const int32_t e = max(e1, e2);
-    const int32_t f1 = fu - cs.ge;
-    const int32_t f2 = hu - cs.go;
-    const int32_t f = max(f1, f2);
-    int32_t h = hul + sm;
-    h = max(h, e);
-    h = max(h, f);
-    h = max(h, 0);
-    S = max(S, h);
-    hul = Hl[R0 + r];
+    const int32_t h = __vimax3_s32_relu(x[r], E[R0 + r], f);  // max(H_diag + SM, E, F, 0)
+    const int32_t hgo = h - cs.go;
+    E[R0 + r] = max(E[R0 + r] - cs.ge, hgo);
+    f = max(f - cs.ge, hgo);
     Hl[R0 + r] = h;
-    E[R0 + r] = e;
-    hu = h;
-    fu = f;
+    if (r & 1) S = __vimax3_s32(S, Hl[R0 + r - 1], h);
   }
 }
 
-template <int R0, int N, int R>
-__device__ __forceinline__ void int_rows(int32_t hul, const uint32_t (&pb)[N / 4], int32_t (&E)[R], int32_t (&Hl)[R],
-                                         int32_t &hu, int32_t &fu, int32_t &S, const Consts &cs) {
-  static_assert(N % 4 == 0, "whole profile words");
-  int_rows_of<R0, N, R>(hul, [&](int r) { return (int32_t)prmt(pb[r >> 2], 0u, sel_sext(r & 3)); }, E, Hl, hu, fu, S,
-                        cs);
-}
-
-// int_rows with the one-operation F chain of word_rows_short, for the int32
-// units of the 16-bit path's small-batch jobs (pairs that could pass the
-// 16-bit range): the F of the row below is max(F - Ge, U - Go) with
-// U = max(H_diag + SM, E, 0), equal to Eq. 3's max(F - Ge, H - Go) because
-// H = max(U, F) and Ge <= Go; U does not depend on the row above, so the
-// chain down the rows is one subtraction and one maximum per row.  Same
-// interface and operation count as int_rows (the plain int32 form keeps
-// Algorithm 1's statement order).
-template <int R0, int N, int R>
-__device__ __forceinline__ void int_rows_short(int32_t hul, const uint32_t (&pb)[N / 4], int32_t (&E)[R],
-                                               int32_t (&Hl)[R], int32_t &hu, int32_t &fu, int32_t &S,
-                                               const Consts &cs) {
-  static_assert(R0 + N <= R && N % 4 == 0, "rows in range, whole profile words");
-  int32_t f = max(fu - cs.ge, hu - cs.go);  // the first row's F from the (H, F) above (Eq. 3)
+// int_rows_of with the one-operation F chain of word_rows_short, for the
+// int32 units of the 16-bit path's small-batch jobs (pairs that could pass
+// the 16-bit range).
+template <int R0, int N, int R, class Add>
+__device__ __forceinline__ void int_rows_short_of(int32_t hd0, Add add, int32_t (&E)[R], int32_t (&Hl)[R], int32_t &f,
+                                                  int32_t &S, const Consts &cs) {
+  static_assert(R0 + N <= R && N % 2 == 0, "rows in range, whole pairs of rows");
+  int32_t u[N];
+#pragma unroll
+  for (int r = N - 1; r >= 0; --r) u[r] = __vimax_s32_relu(add(r, r > 0 ? Hl[R0 + r - 1] : hd0), E[R0 + r]);
 #pragma unroll
   for (int r = 0; r < N; ++r) {
-    const int32_t sm = (int32_t)prmt(pb[r >> 2], 0u, sel_sext(r & 3));
-    const int32_t e = max(E[R0 + r] - cs.ge, Hl[R0 + r] - cs.go);
-    const int32_t u = max(max(hul + sm, e), 0);
-    const int32_t h = max(u, f);
-    S = max(S, h);
-    hul = Hl[R0 + r];
+    const int32_t h = max(u[r], f);
+    f = max(f - cs.ge, u[r] - cs.go);
+    E[R0 + r] = max(E[R0 + r] - cs.ge, h - cs.go);
     Hl[R0 + r] = h;
-    E[R0 + r] = e;
-    if (r + 1 < N) {
-      f = max(f - cs.ge, u - cs.go);
-    } else {
-      hu = h;
-      fu = f;
-    }
+    if (r & 1) S = __vimax3_s32(S, Hl[R0 + r - 1], h);
   }
 }
+
+// h plus profile byte r (signed) of pb: the dot product with a one in that byte
+template <int W>
+__device__ __forceinline__ int32_t add_byte(const uint32_t (&pb)[W], int r, int32_t h) {
+  return __dp4a((int32_t)pb[r >> 2], 1 << (8 * (r & 3)), h);
+}
+// h plus the low 16-bit half (signed) of w
+__device__ __forceinline__ int32_t add_low16(uint32_t w, int32_t h) { return __dp2a_lo((int32_t)w, 1, h); }
 
 // Per-lane DP state of R rows.
 template <int R, int FORM>
 struct LaneState {
   Word<FORM> Hl[R];  // H of each row at the previous column
-  Word<FORM> E[R];   // packed: E of each row at the current column; int32: E at the previous column
+  Word<FORM> E[R];   // E of each row at the current column
   Word<FORM> hdiag;  // H of the row above this lane's first row, previous column
 };
 
@@ -324,9 +307,9 @@ __device__ __forceinline__ void lane_reset(LaneState<R, FORM> &st, const Consts 
 // half); prow points at this lane's first 16-byte group of four words; its
 // R/4 groups are `gstride` bytes apart (lanes interleaved, so the
 // 32 lanes of a warp read 32 consecutive 16-byte groups: no bank conflict).
-// Outputs the (H, F) pair for the row below: int32 passes (H, F) of the last
-// row; packed passes (H of the last row, F of the row below it).
-// SHORTF: rows by word_rows_short / int_rows_short, the one-operation chain.
+// Outputs the (H, F) pair for the row below: H of the last row, F of the row
+// below it.
+// SHORTF: rows by word_rows_short / int_rows_short_of, the one-operation chain.
 // WIDE (two-sequence and int32 forms): the profile holds 32-bit entries, the
 // score in the low 16-bit half (zero-extended), in the query-pair form's
 // group layout; the two sequences' entries are paired by one multiply-add
@@ -371,25 +354,23 @@ __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_
     S = (W)s;
     outH = st.Hl[R - 1];
     outF = (W)f;
-  } else if constexpr (WIDE) {
-    static_assert(!SHORTF, "the wide int32 rows follow Algorithm 1");
-    uint32_t pw[R];
-    load_groups<R>(prow + (res & 0xffu) * stride, gstride, pw);
-    int32_t hu = inH, fu = inF, s = S;
-    int_rows_of<0, R, R>(st.hdiag, [&](int r) { return (int32_t)prmt(pw[r], 0u, sel_sext16()); }, st.E, st.Hl, hu,
-                         fu, s, cs);
-    S = (W)s;
-    outH = (W)hu;
-    outF = (W)fu;
   } else {
-    uint32_t pa[R / 4];
-    load_prof<R>(prow + (res & 0xffu) * stride, pa);
-    int32_t hu = inH, fu = inF, s = S;
-    if constexpr (SHORTF) int_rows_short<0, R>(st.hdiag, pa, st.E, st.Hl, hu, fu, s, cs);
-    else int_rows<0, R>(st.hdiag, pa, st.E, st.Hl, hu, fu, s, cs);
+    int32_t f = inF, s = S;
+    if constexpr (WIDE) {
+      static_assert(!SHORTF, "no wide profiles in the small-batch kernels");
+      uint32_t pw[R];
+      load_groups<R>(prow + (res & 0xffu) * stride, gstride, pw);
+      int_rows_of<0, R, R>(st.hdiag, [&](int r, int32_t h) { return add_low16(pw[r], h); }, st.E, st.Hl, f, s, cs);
+    } else {
+      uint32_t pa[R / 4];
+      load_prof<R>(prow + (res & 0xffu) * stride, pa);
+      const auto add = [&](int r, int32_t h) { return add_byte(pa, r, h); };
+      if constexpr (SHORTF) int_rows_short_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
+      else int_rows_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
+    }
     S = (W)s;
-    outH = (W)hu;
-    outF = (W)fu;
+    outH = st.Hl[R - 1];
+    outF = (W)f;
   }
   st.hdiag = inH;
 }
@@ -459,35 +440,31 @@ __device__ __forceinline__ void column_step_split(LaneState<R, FORM> &st, uint32
   st.hdiag = inH;
 }
 
-// int32 form with split lanes (the pair-band kernel): rows [0, R/2) at column
-// c, rows [R/2, R) at column c - 1.  The upper half's last row (H, F) of the
-// step before (midH, midF) and its H of the step before that (hdiagB) feed
-// the lower half; the lane passes on the lower half's last row, of column
-// c - 1.  resA / resB: the residue code of column c / c - 1.
+// int32 form with split lanes (the pair-band and intra-task kernels): as
+// column_step_split, with byte profiles.
 template <int R>
-__device__ __forceinline__ void column_step_split_int(LaneState<R, kFormInt32> &st, int32_t &hdiagB, int32_t &midH,
-                                                      int32_t &midF, const uint8_t *prow, int stride, uint32_t resA,
-                                                      uint32_t resB, int32_t inH, int32_t inF, const Consts &cs,
-                                                      int32_t &S, int32_t &S2, int32_t &outH, int32_t &outF) {
+__device__ __forceinline__ void column_step_split_int(LaneState<R, kFormInt32> &st, int32_t &hdiagB, int32_t &midF,
+                                                      const uint8_t *prow, int stride, uint32_t resA, uint32_t resB,
+                                                      int32_t inH, int32_t inF, const Consts &cs, int32_t &S,
+                                                      int32_t &S2, int32_t &outH, int32_t &outF) {
   static_assert(R % 8 == 0, "halves of whole profile words");
   constexpr int H2 = R / 2;
   uint32_t pa[H2 / 4], pb[H2 / 4];
   load_prof_at<H2, 0>(prow + (resA & 0xffu) * stride, pa);
   load_prof_at<H2, H2>(prow + (resB & 0xffu) * stride, pb);
+  const int32_t diagB_next = st.Hl[H2 - 1];  // H of the upper half's last row at column c - 1
   // lower half first in program order (its inputs are ready), then the upper
-  int32_t hu = midH, fu = midF, s2 = S2;
-  int_rows<H2, H2>(hdiagB, pb, st.E, st.Hl, hu, fu, s2, cs);
-  outH = hu;
-  outF = fu;
+  int32_t f = midF, s2 = S2;
+  int_rows_of<H2, H2, R>(hdiagB, [&](int r, int32_t h) { return add_byte(pb, r, h); }, st.E, st.Hl, f, s2, cs);
+  outH = st.Hl[R - 1];
+  outF = f;
   S2 = s2;
-  hdiagB = midH;
-  hu = inH;
-  fu = inF;
+  f = inF;
   int32_t s = S;
-  int_rows<0, H2>(st.hdiag, pa, st.E, st.Hl, hu, fu, s, cs);
+  int_rows_of<0, H2, R>(st.hdiag, [&](int r, int32_t h) { return add_byte(pa, r, h); }, st.E, st.Hl, f, s, cs);
   S = s;
-  midH = hu;
-  midF = fu;
+  midF = f;
+  hdiagB = diagB_next;
   st.hdiag = inH;
 }
 

@@ -397,9 +397,9 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
   lane_reset(st, cs);
   W outH = H0, outF = F0, S = (W)0;
   uint32_t outRes = kPadRes;
-  // split lanes: the lower half's residue, diagonal H, incoming H (int32) and F, best
+  // split lanes: the lower half's residue, diagonal H and incoming F, best
   uint32_t prevRes = kPadRes;
-  W hdiagB = H0, midH = H0, midF = F0, S2 = (W)0;
+  W hdiagB = H0, midF = F0, S2 = (W)0;
   uint8_t *rres = ring;                              // [slot][16 B] query residue codes
   uint2 *rgb = reinterpret_cast<uint2 *>(ring + 64);  // [slot][16] (H, F) of the band above
   bool failed = false;
@@ -501,14 +501,13 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
           outH = (W)oh;
           outF = (W)of;
         } else if constexpr (SPLIT) {
-          int32_t s1 = (int32_t)S, s2 = (int32_t)S2, hb = (int32_t)hdiagB, mh = (int32_t)midH, mf = (int32_t)midF;
+          int32_t s1 = (int32_t)S, s2 = (int32_t)S2, hb = (int32_t)hdiagB, mf = (int32_t)midF;
           int32_t oh, of;
-          column_step_split_int<R>(st, hb, mh, mf, prow, kTrackStride<R>, inRes, prevRes, (int32_t)inH, (int32_t)inF,
+          column_step_split_int<R>(st, hb, mf, prow, kTrackStride<R>, inRes, prevRes, (int32_t)inH, (int32_t)inF,
                                    cs, s1, s2, oh, of);
           S = (W)s1;
           S2 = (W)s2;
           hdiagB = (W)hb;
-          midH = (W)mh;
           midF = (W)mf;
           outH = (W)oh;
           outF = (W)of;

@@ -76,9 +76,9 @@ __device__ __forceinline__ void sweep_chunk(IntraShared *sh, const uint8_t *pbuf
   lane_reset(st, cs);
   W outH = H0, outF = F0;
   uint32_t outRes = kPadPair;
-  // split lanes: the lower half's residue, diagonal H, incoming H and F, best
+  // split lanes: the lower half's residue, diagonal H and incoming F, best
   uint32_t prevRes = kPadPair;
-  W hdiagB = H0, midH = H0, midF = F0, S2 = (W)0;
+  W hdiagB = H0, midF = F0, S2 = (W)0;
   const uint8_t *prow = pbuf + g * R;
   const bool first = warp == 0, last = warp == Wq - 1;
   // warp 0 reads residues and (after the first chunk) the boundary strip one
@@ -166,14 +166,13 @@ __device__ __forceinline__ void sweep_chunk(IntraShared *sh, const uint8_t *pbuf
           outH = (W)oh;
           outF = (W)of;
         } else {
-          int32_t s = (int32_t)S, s2 = (int32_t)S2, hb = (int32_t)hdiagB, mh = (int32_t)midH, mf = (int32_t)midF;
+          int32_t s = (int32_t)S, s2 = (int32_t)S2, hb = (int32_t)hdiagB, mf = (int32_t)midF;
           int32_t oh, of;
-          column_step_split_int<R>(st, hb, mh, mf, prow, chunk_stride, inRes, prevRes, (int32_t)inH, (int32_t)inF,
+          column_step_split_int<R>(st, hb, mf, prow, chunk_stride, inRes, prevRes, (int32_t)inH, (int32_t)inF,
                                    cs, s, s2, oh, of);
           S = (W)s;
           S2 = (W)s2;
           hdiagB = (W)hb;
-          midH = (W)mh;
           midF = (W)mf;
           outH = (W)oh;
           outF = (W)of;

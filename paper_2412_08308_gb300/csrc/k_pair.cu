@@ -25,8 +25,9 @@
 // zeros (generation bit 0, which no band of generation 0 writes).  The reader
 // hands consumed columns back through a counter (release/acquire), so a band
 // never overwrites an entry that the band below has not read.  H lies in
-// [0, 2^31 - Go) (the host bounds the scores) and F in [-Go, H] (H takes the
-// maximum with F; H >= 0 bounds F below by -Go), so both fields fit 31 bits.
+// [0, 2^31 - Go) (the host bounds the scores) and F, that of the row below, in
+// [-Go, H] (max(F - Ge, H - Go) with F <= H and H >= 0), so both fields fit 31
+// bits.
 #include "devutil.cuh"
 #include "dp_common.cuh"
 #include "internal.h"
@@ -75,9 +76,9 @@ __device__ __forceinline__ bool band_pass(const uint8_t *__restrict__ pch, const
   lane_reset(st, cs);
   W outH = 0, outF = 0;
   uint32_t outRes = kPadPair;
-  // split lanes: the lower half's residue, diagonal H, incoming H and F, best
+  // split lanes: the lower half's residue, diagonal H and incoming F, best
   uint32_t prevRes = kPadPair;
-  int32_t hdiagB = 0, midH = 0, midF = 0, S2 = 0;
+  int32_t hdiagB = 0, midF = 0, S2 = 0;
   const int src = lane > 0 ? lane - 1 : lane;
   const bool lead = lane == 0;
   const bool tail = lane == 31 && next;
@@ -206,7 +207,7 @@ __device__ __forceinline__ bool band_pass(const uint8_t *__restrict__ pch, const
           inF = (W)v.y;
         }
         if constexpr (kBandSplit<R>) {
-          column_step_split_int<R>(st, hdiagB, midH, midF, prow, stride, inRes, prevRes, inH, inF, cs, S, S2, outH,
+          column_step_split_int<R>(st, hdiagB, midF, prow, stride, inRes, prevRes, inH, inF, cs, S, S2, outH,
                                    outF);
           outRes = prevRes;
           prevRes = inRes;
