@@ -106,18 +106,6 @@ __host__ __device__ constexpr uint32_t sel_sext(int i) {
 }
 __host__ __device__ constexpr uint32_t sel_one(int i) { return 0x4440u | (uint32_t)i; }
 
-// R 32-bit profile entries of one residue in the wide layout (R/4 16-byte
-// groups, `gstride` bytes apart: the lanes' groups interleaved)
-template <int N>
-__device__ __forceinline__ void load_groups(const uint8_t *p, int gstride, uint32_t (&w)[N]) {
-  static_assert(N % 4 == 0, "whole groups");
-#pragma unroll
-  for (int i = 0; i < N / 4; ++i) {
-    const uint4 v = *reinterpret_cast<const uint4 *>(p + i * gstride);
-    w[4 * i + 0] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
-  }
-}
-
 template <int R>
 __device__ __forceinline__ void load_prof(const uint8_t *p, uint32_t (&w)[R / 4]) {
   static_assert(R % 4 == 0, "rows per lane must be a multiple of 4");
@@ -276,8 +264,7 @@ template <int W>
 __device__ __forceinline__ int32_t add_byte(const uint32_t (&pb)[W], int r, int32_t h) {
   return __dp4a((int32_t)pb[r >> 2], 1 << (8 * (r & 3)), h);
 }
-// h plus the low 16-bit half (signed) of w
-__device__ __forceinline__ int32_t add_low16(uint32_t w, int32_t h) { return __dp2a_lo((int32_t)w, 1, h); }
+
 
 // Per-lane DP state of R rows.
 template <int R, int FORM>
@@ -310,11 +297,7 @@ __device__ __forceinline__ void lane_reset(LaneState<R, FORM> &st, const Consts 
 // Outputs the (H, F) pair for the row below: H of the last row, F of the row
 // below it.
 // SHORTF: rows by word_rows_short / int_rows_short_of, the one-operation chain.
-// WIDE (two-sequence and int32 forms): the profile holds 32-bit entries, the
-// score in the low 16-bit half (zero-extended), in the query-pair form's
-// group layout; the two sequences' entries are paired by one multiply-add
-// (FMA pipe) instead of a byte shuffle (ALU pipe).
-template <int R, int FORM, bool SHORTF = false, bool WIDE = false>
+template <int R, int FORM, bool SHORTF = false>
 __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_t *prow, int stride,
                                             uint32_t res, Word<FORM> inH, Word<FORM> inF, const Consts &cs,
                                             Word<FORM> &S, Word<FORM> &outH, Word<FORM> &outF, int gstride = 0) {
@@ -335,19 +318,11 @@ __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_
     outF = (W)f;
   } else if constexpr (FORM == kFormPacked) {
     uint32_t pw[R];
-    if constexpr (WIDE) {
-      uint32_t pa[R], pb[R];
-      load_groups<R>(prow + (res & 0xffu) * stride, gstride, pa);
-      load_groups<R>(prow + (res >> 16) * stride, gstride, pb);
+    uint32_t pa[R / 4], pb[R / 4];
+    load_prof<R>(prow + (res & 0xffu) * stride, pa);
+    load_prof<R>(prow + (res >> 16) * stride, pb);
 #pragma unroll
-      for (int r = 0; r < R; ++r) pw[r] = pb[r] * 0x10000u + pa[r];  // (SM_a, SM_b)
-    } else {
-      uint32_t pa[R / 4], pb[R / 4];
-      load_prof<R>(prow + (res & 0xffu) * stride, pa);
-      load_prof<R>(prow + (res >> 16) * stride, pb);
-#pragma unroll
-      for (int r = 0; r < R; ++r) pw[r] = prmt(pa[r >> 2], pb[r >> 2], sel_pair(r & 3));  // (SM_a, SM_b), signed halves
-    }
+    for (int r = 0; r < R; ++r) pw[r] = prmt(pa[r >> 2], pb[r >> 2], sel_pair(r & 3));  // (SM_a, SM_b), signed halves
     uint32_t f = (uint32_t)inF, s = (uint32_t)S;
     if constexpr (SHORTF) word_rows_short<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
     else word_rows<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
@@ -356,18 +331,11 @@ __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_
     outF = (W)f;
   } else {
     int32_t f = inF, s = S;
-    if constexpr (WIDE) {
-      static_assert(!SHORTF, "no wide profiles in the small-batch kernels");
-      uint32_t pw[R];
-      load_groups<R>(prow + (res & 0xffu) * stride, gstride, pw);
-      int_rows_of<0, R, R>(st.hdiag, [&](int r, int32_t h) { return add_low16(pw[r], h); }, st.E, st.Hl, f, s, cs);
-    } else {
-      uint32_t pa[R / 4];
-      load_prof<R>(prow + (res & 0xffu) * stride, pa);
-      const auto add = [&](int r, int32_t h) { return add_byte(pa, r, h); };
-      if constexpr (SHORTF) int_rows_short_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
-      else int_rows_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
-    }
+    uint32_t pa[R / 4];
+    load_prof<R>(prow + (res & 0xffu) * stride, pa);
+    const auto add = [&](int r, int32_t h) { return add_byte(pa, r, h); };
+    if constexpr (SHORTF) int_rows_short_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
+    else int_rows_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
     S = (W)s;
     outH = st.Hl[R - 1];
     outF = (W)f;
@@ -382,7 +350,7 @@ __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_
 // the lane passes on the lower half's bottom row, of column c - 1, so lane
 // k + 1 works two columns behind lane k.  resA / resB: the residue code(s) of
 // column c / c - 1.  S and S2 keep the halves' running best.
-template <int R, int FORM, bool WIDE = false>
+template <int R, int FORM>
 __device__ __forceinline__ void column_step_split(LaneState<R, FORM> &st, uint32_t &hdiagB, uint32_t &midF,
                                                   const uint8_t *prow, int stride, uint32_t resA, uint32_t resB,
                                                   uint32_t inH, uint32_t inF, const Consts &cs, uint32_t &S,
@@ -399,20 +367,12 @@ __device__ __forceinline__ void column_step_split(LaneState<R, FORM> &st, uint32
       const uint4 w = *reinterpret_cast<const uint4 *>(prow + resB * stride + (H2 / 4 + i) * gstride);
       pb[4 * i + 0] = w.x; pb[4 * i + 1] = w.y; pb[4 * i + 2] = w.z; pb[4 * i + 3] = w.w;
     }
-  } else if constexpr (WIDE) {
-    // two database sequences, 32-bit entries: each word pairs them by one multiply-add
-    uint32_t a0[H2], a1[H2], b0[H2], b1[H2];
-    load_groups<H2>(prow + (resA & 0xffu) * stride, gstride, a0);
-    load_groups<H2>(prow + (resA >> 16) * stride, gstride, a1);
-    load_groups<H2>(prow + (resB & 0xffu) * stride + (H2 / 4) * gstride, gstride, b0);
-    load_groups<H2>(prow + (resB >> 16) * stride + (H2 / 4) * gstride, gstride, b1);
-#pragma unroll
-    for (int r = 0; r < H2; ++r) {
-      pa[r] = a1[r] * 0x10000u + a0[r];
-      pb[r] = b1[r] * 0x10000u + b0[r];
-    }
   } else {
-    // two database sequences: each word pairs their profile bytes (PRMT)
+    // two database sequences: each word pairs their profile bytes by a byte
+    // shuffle (ALU pipe).  32-bit entries paired by a multiply-add on the FMA
+    // pipe take two shared-memory wavefronts per word, of the one per cycle
+    // that an SM has for its four sub-partitions, and measured slower: 4,974
+    // against 5,242 GCUPS, one 400-residue query x 200,000 proteins.
     uint32_t a0[H2 / 4], a1[H2 / 4], b0[H2 / 4], b1[H2 / 4];
     load_prof_at<H2, 0>(prow + (resA & 0xffu) * stride, a0);
     load_prof_at<H2, 0>(prow + (resA >> 16) * stride, a1);
