@@ -56,10 +56,8 @@ int cuda_fail(cudaError_t e, const char *what) {
 
 inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
-// transposed jobs: rows per lane, and each lane's rows as two half-chains a
-// column apart or not
+// transposed jobs: rows per lane
 constexpr int kTrackRows = 16;
-constexpr bool kTrackSplit = false;
 
 int sm_count(int dev) {
   int n = 0;
@@ -71,21 +69,21 @@ int sm_count(int dev) {
 // shape, so each is asked of the runtime once per process (the query, and the
 // shared-memory attribute it sets, cost tens of microseconds per plan).
 // kind: 0 inter-task (a = R, b = form), 1 band-stream (a = R), 2 transposed
-// (a = R, b = split).  Failures (0) are not kept.
-int cached_occupancy(int kind, int a, int b, int threads, size_t smem) {
+// (a = R); gaps: GapSet.  Failures (0) are not kept.
+int cached_occupancy(int kind, int a, int b, int gaps, int threads, size_t smem) {
   static std::mutex mu;
-  static std::map<std::tuple<int, int, int, int, int, size_t>, int> memo;
+  static std::map<std::tuple<int, int, int, int, int, int, size_t>, int> memo;
   int dev = 0;
   cudaGetDevice(&dev);
-  const auto key = std::make_tuple(dev, kind, a, b, threads, smem);
+  const auto key = std::make_tuple(dev, kind, a, b, gaps, threads, smem);
   {
     std::lock_guard<std::mutex> lock(mu);
     auto it = memo.find(key);
     if (it != memo.end()) return it->second;
   }
-  const int n = kind == 0 ? inter_max_ctas_per_sm(a, b, threads, smem)
-                : kind == 1 ? band_max_ctas_per_sm(a)
-                            : track_max_ctas_per_sm(a, b != 0);
+  const int n = kind == 0 ? inter_max_ctas_per_sm(a, b, gaps, threads, smem)
+                : kind == 1 ? band_max_ctas_per_sm(a, gaps)
+                            : track_max_ctas_per_sm(a, gaps);
   if (n > 0) {
     std::lock_guard<std::mutex> lock(mu);
     memo[key] = n;
@@ -697,6 +695,7 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   sc.pad = std::min(0, smin);
   sc.maxp = std::max(0, smax);
   sc.thresh = 32767 - sc.maxp;
+  const int gaps = gap_set(sc);
 
   const int sms = sm_count(db->device);
   const int64_t n = db->n;
@@ -832,14 +831,14 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
       any_band |= band_q[q] != 0;
       any_track |= track_q[q] != 0;
     }
-    const int bmax = any_band ? cached_occupancy(1, bR, 0, 0, 0) : 1;
+    const int bmax = any_band ? cached_occupancy(1, bR, 0, gaps, 0, 0) : 1;
     int bocc = bmax;
     // transposed jobs beside band-stream jobs take 8-row lanes: twice the
     // bands, each half the work per step, which fill in around the
     // band-stream pipelines (homolog workload 2.29 -> 2.14 ms, A/B medians);
     // alone (one short query) 16-row lanes are faster (0.081 against 0.084 ms)
     const int tRows = any_band ? 8 : kTrackRows;
-    int tocc = any_track ? cached_occupancy(2, tRows, kTrackSplit ? 1 : 0, 0, 0) : 1;
+    int tocc = any_track ? cached_occupancy(2, tRows, 0, gaps, 0, 0) : 1;
     int64_t ring = 0, band = 0, tring = 0, tband = 0, n_tlanes = 0;
     if (bocc > 0 && tocc > 0) {
       // band jobs: each band query against every unit
@@ -1003,7 +1002,7 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
         const int64_t bands16 =
             (!any_band && tRows == 16) ? (lay ? lay->bands : track_bands(bins, 16)) * n_track_q : 0;
         if (bands16 > subparts && bands16 <= subparts * tocc) {
-          const int occ24 = cached_occupancy(2, 24, 0, 0, 0);
+          const int occ24 = cached_occupancy(2, 24, 0, gaps, 0, 0);
           const sw_db::TrackLayout *lay24 = nullptr;
           int64_t bands24 = 0;
           if (occ24 > 0) {
@@ -1389,9 +1388,9 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
     delete Q;
     return fail(SW_EINVAL, "sw_queries_prepare: profile chunk too large for shared memory");
   }
-  const int occ = cached_occupancy(0, R, packed ? kFormPacked : kFormInt32, threads, Q->smem);
-  const int occ32 = cached_occupancy(0, R, kFormInt32, threads, Q->smem);
-  const int occp = Q->n_ptasks ? cached_occupancy(0, R, kFormQPair, threads, Q->psmem) : 1;
+  const int occ = cached_occupancy(0, R, packed ? kFormPacked : kFormInt32, gaps, threads, Q->smem);
+  const int occ32 = cached_occupancy(0, R, kFormInt32, gaps, threads, Q->smem);
+  const int occp = Q->n_ptasks ? cached_occupancy(0, R, kFormQPair, gaps, threads, Q->psmem) : 1;
   if (occ <= 0 || occ32 <= 0 || occp <= 0) {
     delete Q;
     return fail(SW_ECUDA, "sw_queries_prepare: cannot configure the inter-task kernel");
@@ -1707,7 +1706,7 @@ int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev
     ta.ring_entries = Q->track_ring_bytes / 8;
     ta.out_size = Q->nq * db->n;
     ta.qt_bytes = Q->qt_bytes;
-    SW_CUDA(launch_track(ta, Q->tR, kTrackSplit, Q->tgrid, s), "band-stream kernel (transposed jobs)");
+    SW_CUDA(launch_track(ta, Q->tR, Q->tgrid, s), "band-stream kernel (transposed jobs)");
   }
   if (Q->timing && !band_timing && (Q->n_tasks || Q->n_ptasks)) SW_CUDA(cudaEventRecord(Q->ev0, s), "event");
   if (Q->n_ptasks) {  // query pairs, one short database sequence per chain

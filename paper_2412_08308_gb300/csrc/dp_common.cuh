@@ -72,15 +72,18 @@ struct Consts {
   int32_t go, ge;
 };
 
+template <int GAPS = kGapsAny>
 __device__ __forceinline__ Consts make_consts(const Scoring &sc) {
+  const int32_t go = GAPS == kGapsProtein ? kProteinGo : GAPS == kGapsDna ? kDnaGo : sc.go;
+  const int32_t ge = GAPS == kGapsProtein ? kProteinGe : GAPS == kGapsDna ? kDnaGe : sc.ge;
   Consts c;
-  c.goW = (uint32_t)sc.go * 0x10001u;
-  c.geW = (uint32_t)sc.ge * 0x10001u;
-  const uint32_t ngo = (uint32_t)(-sc.go) & 0xffffu;  // E, F start at -Go (any value <= 0 works)
+  c.goW = (uint32_t)go * 0x10001u;
+  c.geW = (uint32_t)ge * 0x10001u;
+  const uint32_t ngo = (uint32_t)(-go) & 0xffffu;  // E, F start at -Go (any value <= 0 works)
   c.F0W = ngo | (ngo << 16);
   c.E0W = c.F0W;
-  c.go = sc.go;
-  c.ge = sc.ge;
+  c.go = go;
+  c.ge = ge;
   return c;
 }
 
@@ -163,16 +166,19 @@ __device__ __forceinline__ uint32_t word_of(const uint4 &v, int i) {
 // H_diag + SM are formed first: the previous column's H is then dead before
 // any row is rewritten (forming them row by row costs a register copy each).
 // Two-input maxima throughout (5 on the ALU pipe) took 10.3 cycles per word
-// and SM sub-partition in a loop over 24 rows and four warps, this order 9.1
-// (the ALU pipe 79 % busy; register operands, up to three per instruction,
-// are the rest), and the same formed row by row 10.2-10.6.
+// and SM sub-partition in a loop over 24 rows and four warps, this 9.1 (the
+// ALU pipe 79 % busy; register operands, up to three per instruction, are the
+// rest; 8.4-8.7 with the penalties as immediates), and the same formed row by
+// row 10.2-10.6.  The running best is taken after the rows, as two chains:
+// inside the row loop the two-sequence form took 71.5 ms instead of 67.0 (20
+// queries x 40,000 proteins), query pairs the same.
 template <int R0, int N, int R>
 __device__ __forceinline__ void word_rows(uint32_t hd0, const uint32_t (&p)[N], uint32_t (&E)[R],
                                           uint32_t (&Hl)[R], uint32_t &f, uint32_t &S, const Consts &cs) {
   static_assert(R0 + N <= R && N % 2 == 0, "rows in range, whole pairs of rows");
   uint32_t x[N];
 #pragma unroll
-  for (int r = N - 1; r >= 0; --r) x[r] = __vadd2(r > 0 ? Hl[R0 + r - 1] : hd0, p[r]);
+  for (int r = 0; r < N; ++r) x[r] = __vadd2(r > 0 ? Hl[R0 + r - 1] : hd0, p[r]);
 #pragma unroll
   for (int r = 0; r < N; ++r) {
     const uint32_t h = __vimax3_s16x2_relu(x[r], E[R0 + r], f);  // max(H_diag + SM, E, F, 0)
@@ -180,8 +186,16 @@ __device__ __forceinline__ void word_rows(uint32_t hd0, const uint32_t (&p)[N], 
     E[R0 + r] = __vmaxs2(__vsub2(E[R0 + r], cs.geW), hgo);
     f = __vmaxs2(__vsub2(f, cs.geW), hgo);
     Hl[R0 + r] = h;
-    if (r & 1) S = __vimax3_s16x2(S, Hl[R0 + r - 1], h);
   }
+  constexpr int N2 = N / 2;
+  uint32_t a = Hl[R0], b = Hl[R0 + N2];
+#pragma unroll
+  for (int r = 1; r + 1 < N2; r += 2) {
+    a = __vimax3_s16x2(a, Hl[R0 + r], Hl[R0 + r + 1]);
+    b = __vimax3_s16x2(b, Hl[R0 + N2 + r], Hl[R0 + N2 + r + 1]);
+  }
+  if constexpr (N2 % 2 == 0) a = __vimax3_s16x2(a, Hl[R0 + N2 - 1], Hl[R0 + N - 1]);
+  S = __vimax3_s16x2(S, a, b);
 }
 
 // word_rows with a one-operation chain down the rows, for kernels bound by

@@ -25,6 +25,23 @@ struct Scoring {
   int32_t thresh;  // a packed 16-bit lane may have wrapped only if its score S > thresh
 };
 
+// Gap penalties compiled into a kernel.  A register operand that becomes an
+// immediate takes one read off each E and F update and off H - Go, and the
+// register file's read ports are what keeps the 16-bit forms from their ALU
+// rate: 20 queries x 40,000 proteins 67.8 -> 64.8 ms (two-sequence form), 2
+// queries x 500,000 23.1 -> 21.6 ms (query pairs), DNA pair 1M x 1M 401 -> 376
+// ms; the int32 inter-task form gains nothing and has no such variant.  Only
+// the two pairs of penalties that the interface defaults to and the paper
+// uses (Sec. 4.1) get kernels of their own; all others take kGapsAny.
+enum GapSet : int { kGapsAny = 0, kGapsProtein = 1, kGapsDna = 2 };
+constexpr int32_t kProteinGo = 12, kProteinGe = 2;  // 10 + 2k
+constexpr int32_t kDnaGo = 7, kDnaGe = 2;           // 5 + 2k
+inline int gap_set(const Scoring &sc) {
+  if (sc.go == kProteinGo && sc.ge == kProteinGe) return kGapsProtein;
+  if (sc.go == kDnaGo && sc.ge == kDnaGe) return kGapsDna;
+  return kGapsAny;
+}
+
 // Per-query descriptor for the dynamic-programming kernels, or (query-track
 // plans of the query-pair form) per plan.
 struct QDesc {
@@ -133,7 +150,7 @@ struct PairBandArgs {
   Scoring sc;
 };
 size_t pair_smem_bytes(int pbuf_bytes, int warps);
-int pair_max_ctas_per_sm(int R, int threads, size_t smem);
+int pair_max_ctas_per_sm(int R, int gaps, int threads, size_t smem);  // gaps: GapSet, here and below
 cudaError_t launch_pair(const PairBandArgs &a, int R, int grid, int threads, size_t smem, cudaStream_t s);
 
 // Band-stream kernel (k_band.cu): in small batches, a long query's rows (or a
@@ -216,17 +233,16 @@ struct TrackArgs {
   // buffer sizes, tested by the checked build (-DSW_CHECK) before every access
   int64_t n_lanes, ring_entries, out_size, qt_bytes;
 };
-// R: rows per lane of the transposed jobs (8 or 16: bands of 256 or 512 database rows);
-// split: each lane's rows as two half-chains a column apart (see column_step_split)
+// R: rows per lane of the transposed jobs (8, 16 or 24: bands of 256, 512 or 768 database rows)
 bool track_supported_R(int R);
-int track_max_ctas_per_sm(int R, bool split);  // plan time: raises the shared-memory limit; 0 on failure
+int track_max_ctas_per_sm(int R, int gaps);  // plan time: raises the shared-memory limit; 0 on failure
 int track_threads();
-cudaError_t launch_track(const TrackArgs &a, int R, bool split, int grid, cudaStream_t s);
+cudaError_t launch_track(const TrackArgs &a, int R, int grid, cudaStream_t s);
 
 int band_threads();
 bool band_supported_R(int R);  // rows per lane: 8 or 16 (bands of 256 or 512 query rows)
 size_t band_smem_bytes(int R);
-int band_max_ctas_per_sm(int R);  // plan time: raises the shared-memory limit; 0 on failure
+int band_max_ctas_per_sm(int R, int gaps);  // plan time: raises the shared-memory limit; 0 on failure
 // one_per_sm: reserve shared memory so that the launch places at most one CTA per SM
 cudaError_t launch_band(const BandArgs &a, int R, int grid, bool one_per_sm, cudaStream_t s);
 
@@ -272,7 +288,7 @@ cudaError_t launch_inter(const InterArgs &a, int R, int form, int grid, int thre
                          cudaStream_t s);
 // Raises the instantiation's shared-memory limit (plan time only) and returns resident CTAs per SM
 // (0 on failure).
-int inter_max_ctas_per_sm(int R, int form, int threads, size_t smem);
+int inter_max_ctas_per_sm(int R, int form, int gaps, int threads, size_t smem);
 
 // intra-task kernel (k_intra.cu): one CTA of intra_threads() per (query, unit) task;
 // QDesc::L = 32 * warps of the chain.

@@ -240,7 +240,7 @@ __device__ __forceinline__ bool band_unit(const BandArgs &a, const uint8_t *__re
   return !failed;
 }
 
-template <int R>
+template <int R, int GAPS>
 __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(const BandArgs a) {
   constexpr int RH = R / 2;  // rows per lane of kBandInt32Half jobs
   extern __shared__ __align__(128) uint8_t smem[];
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(cons
   uint8_t *ring = prof + kProfBytes<R>;
   for (int i = threadIdx.x; i < kAlphabet * kAlphabet; i += blockDim.x) sm[i] = a.submat[i];
   __syncthreads();
-  const Consts cs = make_consts(a.sc);
+  const Consts cs = make_consts<GAPS>(a.sc);
 
   for (;;) {
     int g = 0;
@@ -369,10 +369,9 @@ __device__ __forceinline__ void build_track_profile(uint8_t *prof, const int8_t 
 
 // One band of a row track over all columns of its query.  keepH / addF: the
 // lane's restart masks (a half whose rows start a sequence takes the matrix
-// top boundary (0, F0) instead of the row above).  SPLIT: the lane's rows as
-// two half-chains a column apart (column_step_split).  Returns false when a
-// wait expired.
-template <int R, int FORM, bool SPLIT>
+// top boundary (0, F0) instead of the row above).  Returns false when a wait
+// expired.
+template <int R, int FORM>
 __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__restrict__ prof, uint8_t *ring,
                                            const int lane, const uint8_t *resQ, const int npad,
                                            const unsigned long long *ring_in, unsigned long long *ring_out,
@@ -380,10 +379,9 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
                                            Word<FORM> &Sout) {
   using W = Word<FORM>;
   constexpr bool PACKED = FORM != kFormInt32;
-  constexpr int LAG = SPLIT ? 2 * 32 - 1 : 32 - 1;
   const W H0 = (W)0;
   const W F0 = PACKED ? (W)cs.F0W : (W)0;
-  const int nblk = (npad + LAG + kColBlock - 1) / kColBlock;
+  const int nblk = (npad + kLag + kColBlock - 1) / kColBlock;
   const int nreal = npad / kColBlock;
   const bool prev = ring_in != nullptr, next = ring_out != nullptr;
   const bool lead = lane == 0;
@@ -397,9 +395,6 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
   lane_reset(st, cs);
   W outH = H0, outF = F0, S = (W)0;
   uint32_t outRes = kPadRes;
-  // split lanes: the lower half's residue, diagonal H and incoming F, best
-  uint32_t prevRes = kPadRes;
-  W hdiagB = H0, midF = F0, S2 = (W)0;
   uint8_t *rres = ring;                              // [slot][16 B] query residue codes
   uint2 *rgb = reinterpret_cast<uint2 *>(ring + 64);  // [slot][16] (H, F) of the band above
   bool failed = false;
@@ -490,38 +485,10 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
             inRes = kPadRes;
           }
         }
-        if constexpr (SPLIT && PACKED) {
-          uint32_t s1 = (uint32_t)S, s2 = (uint32_t)S2, hb = (uint32_t)hdiagB, mf = (uint32_t)midF, oh, of;
-          column_step_split<R, FORM>(st, hb, mf, prow, kTrackStride<R>, inRes, prevRes, (uint32_t)inH, (uint32_t)inF,
-                                     cs, s1, s2, oh, of, 0);
-          S = (W)s1;
-          S2 = (W)s2;
-          hdiagB = (W)hb;
-          midF = (W)mf;
-          outH = (W)oh;
-          outF = (W)of;
-        } else if constexpr (SPLIT) {
-          int32_t s1 = (int32_t)S, s2 = (int32_t)S2, hb = (int32_t)hdiagB, mf = (int32_t)midF;
-          int32_t oh, of;
-          column_step_split_int<R>(st, hb, mf, prow, kTrackStride<R>, inRes, prevRes, (int32_t)inH, (int32_t)inF,
-                                   cs, s1, s2, oh, of);
-          S = (W)s1;
-          S2 = (W)s2;
-          hdiagB = (W)hb;
-          midF = (W)mf;
-          outH = (W)oh;
-          outF = (W)of;
-        } else {
-          column_step<R, FORM, PACKED>(st, prow, kTrackStride<R>, inRes, inH, inF, cs, S, outH, outF, 0);
-        }
-        if constexpr (SPLIT) {
-          outRes = prevRes;
-          prevRes = inRes;
-        } else {
-          outRes = inRes;
-        }
+        column_step<R, FORM, PACKED>(st, prow, kTrackStride<R>, inRes, inH, inF, cs, S, outH, outF, 0);
+        outRes = inRes;
         if (tail) {
-          const int j = t - LAG;
+          const int j = t - kLag;
           if (j >= 0 && j < npad && in_range(ring_out - a.rings + j, a.ring_entries, a.status)) {
             const uint32_t lo = (uint32_t)outH | 0x80000000u;
             st_relaxed_u64(ring_out + j, ((unsigned long long)(uint32_t)outF << 32) | lo);
@@ -542,7 +509,7 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
     }
   }
   if (lead) cp_async_wait<0>();
-  Sout = SPLIT ? score_max<FORM>(S, S2) : S;
+  Sout = S;
   return !failed;
 }
 
@@ -564,7 +531,7 @@ __device__ __forceinline__ void track_scores(const TrackArgs &a, int32_t q, int3
   }
 }
 
-template <int R, bool SPLIT>
+template <int R, int GAPS>
 __global__ void __launch_bounds__(kTrackThreads, R == 8 ? 4 : R == 16 ? 2 : 1) band_track_kernel(const TrackArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   int8_t *sm = reinterpret_cast<int8_t *>(smem);
@@ -573,7 +540,7 @@ __global__ void __launch_bounds__(kTrackThreads, R == 8 ? 4 : R == 16 ? 2 : 1) b
   uint8_t *ring = prof + kTrackProfBytes<R>;
   for (int i = threadIdx.x; i < kAlphabet * kAlphabet; i += blockDim.x) sm[i] = a.submat[i];
   __syncthreads();
-  const Consts cs = make_consts(a.sc);
+  const Consts cs = make_consts<GAPS>(a.sc);
   const TrackLane idle{-1, 0, -1, 0};
   // a lane continues the sequence of the row above (in at least one used half)
   auto continues = [](const TrackLane &L, bool packed) {
@@ -611,7 +578,7 @@ __global__ void __launch_bounds__(kTrackThreads, R == 8 ? 4 : R == 16 ? 2 : 1) b
       __syncwarp();
       const uint32_t mask = (ra0 ? 0x0000ffffu : 0u) | (rb0 ? 0xffff0000u : 0u);
       uint32_t S = 0u;
-      ok = track_pass<R, kFormPacked, SPLIT>(a, prof, ring, lane, resQ, npad, ring_in, ring_out, ~mask, cs.F0W & mask,
+      ok = track_pass<R, kFormPacked>(a, prof, ring, lane, resQ, npad, ring_in, ring_out, ~mask, cs.F0W & mask,
                                           cs, S);
       track_scores(a, job.q, L.pa, (int32_t)(S & 0xffffu), lane);
       track_scores(a, job.q, L.pb, (int32_t)(S >> 16), lane);
@@ -619,7 +586,7 @@ __global__ void __launch_bounds__(kTrackThreads, R == 8 ? 4 : R == 16 ? 2 : 1) b
       build_track_profile<R, false>(prof, sm, a.db, L, lane, a.sc.pad, a.status);
       __syncwarp();
       int32_t S = 0;
-      ok = track_pass<R, kFormInt32, SPLIT>(a, prof, ring, lane, resQ, npad, ring_in, ring_out, ra0 ? 0 : -1, 0, cs, S);
+      ok = track_pass<R, kFormInt32>(a, prof, ring, lane, resQ, npad, ring_in, ring_out, ra0 ? 0 : -1, 0, cs, S);
       track_scores(a, job.q, L.pa, S, lane);
     }
     __syncwarp();
@@ -646,18 +613,28 @@ size_t one_cta_smem() {
   return want <= (size_t)per_block ? want : 0;
 }
 
-template <int R>
-int occupancy_of() {
-  // the limit admits the one-CTA-per-SM reservation as well
-  const size_t limit = std::max(smem_of<R>(), one_cta_smem());
-  if (cudaFuncSetAttribute(band_stream_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
+// The kernels with the protein penalties compiled in (see GapSet), or general.
+using BandKernel = void (*)(const BandArgs);
+BandKernel band_kernel(int R, int gaps) {
+  const bool p = gaps == kGapsProtein;
+  if (R == 8) return p ? band_stream_kernel<8, kGapsProtein> : band_stream_kernel<8, kGapsAny>;
+  if (R == 16) return p ? band_stream_kernel<16, kGapsProtein> : band_stream_kernel<16, kGapsAny>;
+  return nullptr;
+}
+using TrackKernel = void (*)(const TrackArgs);
+TrackKernel track_kernel(int R, int gaps) {
+  const bool p = gaps == kGapsProtein;
+  if (R == 8) return p ? band_track_kernel<8, kGapsProtein> : band_track_kernel<8, kGapsAny>;
+  if (R == 16) return p ? band_track_kernel<16, kGapsProtein> : band_track_kernel<16, kGapsAny>;
+  if (R == 24) return p ? band_track_kernel<24, kGapsProtein> : band_track_kernel<24, kGapsAny>;
+  return nullptr;
+}
+
+template <class Kernel>
+int occupancy_of(Kernel kern, int threads, size_t smem, size_t limit) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, band_stream_kernel<R>, kBandStreamThreads,
-                                                    smem_of<R>()) != cudaSuccess) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -666,22 +643,7 @@ int occupancy_of() {
 
 template <int R>
 size_t track_smem() { return kSubmatBytes + (size_t)(kTrackThreads / 32) * kTrackWarpBytes<R>; }
-
-template <int R, bool SPLIT>
-int track_occupancy() {
-  if (cudaFuncSetAttribute(band_track_kernel<R, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)track_smem<R>()) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, band_track_kernel<R, SPLIT>, kTrackThreads,
-                                                    track_smem<R>()) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return n;
-}
+size_t track_smem_of(int R) { return R == 8 ? track_smem<8>() : R == 16 ? track_smem<16>() : track_smem<24>(); }
 
 }  // namespace
 
@@ -689,38 +651,36 @@ int track_threads() { return kTrackThreads; }
 
 bool track_supported_R(int R) { return R == 8 || R == 16 || R == 24; }
 
-int track_max_ctas_per_sm(int R, bool split) {
-  if (R == 8) return split ? track_occupancy<8, true>() : track_occupancy<8, false>();
-  if (R == 16) return split ? track_occupancy<16, true>() : track_occupancy<16, false>();
-  if (R == 24 && !split) return track_occupancy<24, false>();
-  return 0;
+int track_max_ctas_per_sm(int R, int gaps) {
+  const TrackKernel kern = track_kernel(R, gaps);
+  return kern ? occupancy_of(kern, kTrackThreads, track_smem_of(R), track_smem_of(R)) : 0;
 }
 
-cudaError_t launch_track(const TrackArgs &a, int R, bool split, int grid, cudaStream_t s) {
-  const int T = kTrackThreads;
-  if (R == 8 && split) band_track_kernel<8, true><<<grid, T, track_smem<8>(), s>>>(a);
-  else if (R == 8) band_track_kernel<8, false><<<grid, T, track_smem<8>(), s>>>(a);
-  else if (R == 16 && split) band_track_kernel<16, true><<<grid, T, track_smem<16>(), s>>>(a);
-  else if (R == 16) band_track_kernel<16, false><<<grid, T, track_smem<16>(), s>>>(a);
-  else if (R == 24 && !split) band_track_kernel<24, false><<<grid, T, track_smem<24>(), s>>>(a);
-  else return cudaErrorInvalidValue;
+cudaError_t launch_track(const TrackArgs &a, int R, int grid, cudaStream_t s) {
+  const TrackKernel kern = track_kernel(R, gap_set(a.sc));
+  if (!kern) return cudaErrorInvalidValue;
+  kern<<<grid, kTrackThreads, track_smem_of(R), s>>>(a);
   return cudaGetLastError();
 }
 
 int band_threads() { return kBandStreamThreads; }
 bool band_supported_R(int R) { return R == 8 || R == 16; }
 size_t band_smem_bytes(int R) { return R == 16 ? smem_of<16>() : smem_of<8>(); }
-int band_max_ctas_per_sm(int R) { return R == 8 ? occupancy_of<8>() : R == 16 ? occupancy_of<16>() : 0; }
+int band_max_ctas_per_sm(int R, int gaps) {
+  const BandKernel kern = band_kernel(R, gaps);
+  // (the limit admits the one-CTA-per-SM reservation as well)
+  return kern ? occupancy_of(kern, kBandStreamThreads, band_smem_bytes(R), std::max(band_smem_bytes(R), one_cta_smem()))
+              : 0;
+}
 
 cudaError_t launch_band(const BandArgs &a, int R, int grid, bool one_per_sm, cudaStream_t s) {
   // one CTA per SM: the launch takes more than half of an SM's shared memory,
   // so that the hardware never places two on an SM, whatever else (the
   // transposed jobs beside it, a kernel finishing before it) holds the SMs
   // when its CTAs are placed
-  const size_t extra = one_per_sm ? one_cta_smem() : 0;
-  if (R == 8) band_stream_kernel<8><<<grid, kBandStreamThreads, std::max(extra, smem_of<8>()), s>>>(a);
-  else if (R == 16) band_stream_kernel<16><<<grid, kBandStreamThreads, std::max(extra, smem_of<16>()), s>>>(a);
-  else return cudaErrorInvalidValue;
+  const BandKernel kern = band_kernel(R, gap_set(a.sc));
+  if (!kern) return cudaErrorInvalidValue;
+  kern<<<grid, kBandStreamThreads, std::max(one_per_sm ? one_cta_smem() : 0, band_smem_bytes(R)), s>>>(a);
   return cudaGetLastError();
 }
 

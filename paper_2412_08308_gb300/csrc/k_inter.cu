@@ -187,7 +187,7 @@ __device__ __forceinline__ void chain_pass(const uint8_t *__restrict__ pch, cons
   if constexpr (SPLIT) S = score_max<FORM>(S, (W)S2);
 }
 
-template <int R, int FORM>
+template <int R, int FORM, int GAPS>
 __global__ void __launch_bounds__(kThreads, 2) inter_kernel(const InterArgs a) {
   using W = Word<FORM>;
   constexpr bool PAIRS = FORM == kFormPacked;
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 2) inter_kernel(const InterArgs a) {
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
-  const Consts cs = make_consts(a.sc);
+  const Consts cs = make_consts<GAPS>(a.sc);
 
   if (threadIdx.x == 0) {
     mbar_init(&mbar[0], 1);
@@ -318,28 +318,14 @@ __global__ void __launch_bounds__(kThreads, 2) inter_kernel(const InterArgs a) {
   }
 }
 
+// The kernel of a form: with the protein penalties compiled in for the 16-bit
+// forms at the heights the planner uses (see GapSet), else the general one.
+using InterKernel = void (*)(const InterArgs);
 template <int R, int FORM>
-cudaError_t launch_one(const InterArgs &a, int grid, int threads, size_t smem, cudaStream_t s) {
-  inter_kernel<R, FORM><<<grid, threads, smem, s>>>(a);
-  return cudaGetLastError();
-}
-
-// Raise the dynamic shared-memory limit of an instantiation (done at plan time,
-// never inside a launch sequence that may be captured into a graph) and return
-// its resident CTAs per SM for the given block size and shared memory.
-template <int R, int FORM>
-int configure_one(int threads, size_t smem) {
-  auto kern = inter_kernel<R, FORM>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return n;
+InterKernel kernel_for(int gaps) {
+  if constexpr (FORM != kFormInt32 && R % 8 == 0)
+    if (gaps == kGapsProtein) return inter_kernel<R, FORM, kGapsProtein>;
+  return inter_kernel<R, FORM, kGapsAny>;
 }
 
 }  // namespace
@@ -371,29 +357,39 @@ int inter_chain_lag(int R, int form, int L) {
   return L - 1;
 }
 
-cudaError_t launch_inter(const InterArgs &a, int R, int form, int grid, int threads, size_t smem,
-                         cudaStream_t s) {
-#define SWGB_CASE(RR)                                                                                 \
-  if (R == RR) {                                                                                      \
-    if (form == kFormInt32) return launch_one<RR, kFormInt32>(a, grid, threads, smem, s);      \
-    if (form == kFormPacked) return launch_one<RR, kFormPacked>(a, grid, threads, smem, s);    \
-    if (form == kFormQPair) return launch_one<RR, kFormQPair>(a, grid, threads, smem, s);      \
+static InterKernel find_kernel(int R, int form, int gaps) {
+#define SWGB_CASE(RR)                                                  \
+  if (R == RR) {                                                       \
+    if (form == kFormInt32) return kernel_for<RR, kFormInt32>(gaps);   \
+    if (form == kFormPacked) return kernel_for<RR, kFormPacked>(gaps); \
+    if (form == kFormQPair) return kernel_for<RR, kFormQPair>(gaps);   \
   }
   SWGB_INTER_R_LIST(SWGB_CASE)
 #undef SWGB_CASE
-  return cudaErrorInvalidValue;
+  return nullptr;
 }
 
-int inter_max_ctas_per_sm(int R, int form, int threads, size_t smem) {
-#define SWGB_CASE(RR)                                                                              \
-  if (R == RR) {                                                                                   \
-    if (form == kFormInt32) return configure_one<RR, kFormInt32>(threads, smem);            \
-    if (form == kFormPacked) return configure_one<RR, kFormPacked>(threads, smem);          \
-    if (form == kFormQPair) return configure_one<RR, kFormQPair>(threads, smem);            \
+cudaError_t launch_inter(const InterArgs &a, int R, int form, int grid, int threads, size_t smem,
+                         cudaStream_t s) {
+  const InterKernel kern = find_kernel(R, form, gap_set(a.sc));
+  if (!kern) return cudaErrorInvalidValue;
+  kern<<<grid, threads, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+// Raise the dynamic shared-memory limit of the kernel (done at plan time,
+// never inside a launch sequence that may be captured into a graph) and return
+// its resident CTAs per SM for the given block size and shared memory.
+int inter_max_ctas_per_sm(int R, int form, int gaps, int threads, size_t smem) {
+  const InterKernel kern = find_kernel(R, form, gaps);
+  if (!kern) return 0;
+  int n = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
   }
-  SWGB_INTER_R_LIST(SWGB_CASE)
-#undef SWGB_CASE
-  return 0;
+  return n;
 }
 
 }  // namespace swgb

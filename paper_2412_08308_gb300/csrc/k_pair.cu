@@ -247,14 +247,14 @@ __device__ __forceinline__ bool band_pass(const uint8_t *__restrict__ pch, const
   return !failed;
 }
 
-template <int R>
+template <int R, int GAPS>
 __global__ void __launch_bounds__(kPairThreads, 1) pair_band_kernel(const PairBandArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
   uint8_t *pbuf = smem + (size_t)warp * (a.pbuf_bytes + kBandRingBytes);
   uint8_t *ring = pbuf + a.pbuf_bytes;
-  const Consts cs = make_consts(a.sc);
+  const Consts cs = make_consts<GAPS>(a.sc);
   const int nblk = (a.npad + kBandLag<R> + kColBlock - 1) / kColBlock;
   int32_t S = 0;
   // global warp g = warp * grid + CTA: bands spread over the SMs first
@@ -281,45 +281,39 @@ __global__ void __launch_bounds__(kPairThreads, 1) pair_band_kernel(const PairBa
   if (lane == 0) atomicMax(a.best, S);
 }
 
-template <int R>
-int configure_pair_one(int threads, size_t smem) {
-  auto kern = pair_band_kernel<R>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return n;
-}
-
-template <int R>
-cudaError_t launch_pair_one(const PairBandArgs &a, int grid, int threads, size_t smem, cudaStream_t s) {
-  void *args[] = {(void *)&a};
-  return cudaLaunchCooperativeKernel((const void *)pair_band_kernel<R>, dim3(grid), dim3(threads), args, smem, s);
+// The kernel of a band height: with the DNA penalties compiled in at the
+// heights the planner picks (see GapSet), else the general one.
+using PairKernel = void (*)(const PairBandArgs);
+PairKernel pair_kernel(int R, int gaps) {
+  const bool d = gaps == kGapsDna;
+  if (R == 4) return pair_band_kernel<4, kGapsAny>;
+  if (R == 8) return d ? pair_band_kernel<8, kGapsDna> : pair_band_kernel<8, kGapsAny>;
+  if (R == 16) return d ? pair_band_kernel<16, kGapsDna> : pair_band_kernel<16, kGapsAny>;
+  if (R == 24) return pair_band_kernel<24, kGapsAny>;
+  return nullptr;
 }
 
 }  // namespace
 
 size_t pair_smem_bytes(int pbuf_bytes, int warps) { return (size_t)warps * (pbuf_bytes + kBandRingBytes); }
 
-int pair_max_ctas_per_sm(int R, int threads, size_t smem) {
-  if (R == 4) return configure_pair_one<4>(threads, smem);
-  if (R == 8) return configure_pair_one<8>(threads, smem);
-  if (R == 16) return configure_pair_one<16>(threads, smem);
-  if (R == 24) return configure_pair_one<24>(threads, smem);
-  return 0;
+int pair_max_ctas_per_sm(int R, int gaps, int threads, size_t smem) {
+  const PairKernel kern = pair_kernel(R, gaps);
+  int n = 0;
+  if (!kern ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
 }
 
 cudaError_t launch_pair(const PairBandArgs &a, int R, int grid, int threads, size_t smem, cudaStream_t s) {
-  if (R == 4) return launch_pair_one<4>(a, grid, threads, smem, s);
-  if (R == 8) return launch_pair_one<8>(a, grid, threads, smem, s);
-  if (R == 16) return launch_pair_one<16>(a, grid, threads, smem, s);
-  if (R == 24) return launch_pair_one<24>(a, grid, threads, smem, s);
-  return cudaErrorInvalidValue;
+  const PairKernel kern = pair_kernel(R, gap_set(a.sc));
+  if (!kern) return cudaErrorInvalidValue;
+  void *args[] = {(void *)&a};
+  return cudaLaunchCooperativeKernel((const void *)kern, dim3(grid), dim3(threads), args, smem, s);
 }
 
 }  // namespace swgb

@@ -134,8 +134,8 @@ extern "C" int sw_search_noalloc(const sw_db *db, const uint8_t *query, int64_t 
       e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
       if (e != cudaSuccess) return cuda_err(e, "cudaGetSymbolAddress");
       const size_t smem = inter_smem_bytes((int)round_up(kProfMax, 128), 2, kNoAllocThreads);
-      st.occ16 = inter_max_ctas_per_sm(16, kFormInt32, kNoAllocThreads, smem);
-      st.occ24 = inter_max_ctas_per_sm(24, kFormInt32, kNoAllocThreads, smem);
+      st.occ16 = inter_max_ctas_per_sm(16, kFormInt32, kGapsAny, kNoAllocThreads, smem);
+      st.occ24 = inter_max_ctas_per_sm(24, kFormInt32, kGapsAny, kNoAllocThreads, smem);
       if (st.occ16 <= 0 || st.occ24 <= 0) return fail_msg(SW_ECUDA, "sw_search_noalloc: kernel configuration failed");
       st.scratch = static_cast<uint8_t *>(p);
     }

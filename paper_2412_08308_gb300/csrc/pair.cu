@@ -136,7 +136,13 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
   const int threads = 32 * warps;
   const size_t smem = pair_smem_bytes(pbuf_bytes, warps);
   if (smem > 200 * 1024) return pair_fail(SW_EINVAL, "sw_align_pair: band profile too large for shared memory");
-  const int occ = pair_max_ctas_per_sm(R, threads, smem);
+  Scoring scr{};
+  scr.go = gap_open + gap_extend;
+  scr.ge = gap_extend;
+  scr.pad = std::min(0, smin);
+  scr.maxp = std::max(0, smax);
+  scr.thresh = 32767 - scr.maxp;
+  const int occ = pair_max_ctas_per_sm(R, gap_set(scr), threads, smem);
   if (occ <= 0) return pair_fail(SW_ECUDA, "sw_align_pair: cannot configure the pair kernel");
   // every SM gets a CTA (the kernel deals bands to the SMs in turn)
   int64_t grid = std::min<int64_t>(std::max<int64_t>((nbands64 + warps - 1) / warps, std::min<int64_t>(sms, nbands64)),
@@ -197,12 +203,6 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
   if (e == cudaSuccess) e = cudaMemsetAsync(d_strip, 0, b_strip + b_prog + b_words, s);
   if (e != cudaSuccess) return pair_cuda(e, "upload");
 
-  Scoring scr{};
-  scr.go = gap_open + gap_extend;
-  scr.ge = gap_extend;
-  scr.pad = std::min(0, smin);
-  scr.maxp = std::max(0, smax);
-  scr.thresh = 32767 - scr.maxp;
   e = launch_build_profiles(d_q, d_qd, 1, d_sub, scr.pad, d_prof, s);
   if (e != cudaSuccess) return pair_cuda(e, "profile kernel");
 
