@@ -93,6 +93,14 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned l
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v));
 }
 
+// Two 64-bit words by one 128-bit store (p 16-byte aligned), each word
+// single-copy atomic like st_relaxed_u64, with no order between them.
+__device__ __forceinline__ void st_relaxed_2xu64(unsigned long long *p, uint32_t lo0, uint32_t hi0, uint32_t lo1,
+                                                 uint32_t hi1) {
+  const unsigned long long v0 = ((unsigned long long)hi0 << 32) | lo0, v1 = ((unsigned long long)hi1 << 32) | lo1;
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(v0), "l"(v1));
+}
+
 // A wait on another warp of a long pipeline, which may legitimately last as
 // long as a whole band takes: ~60 s at GB300 clocks.
 constexpr long long kLongWaitBudgetCycles = 120000000000LL;

@@ -54,7 +54,7 @@ struct QDesc {
   int64_t prof_off;  // byte offset of chunk 0 in the profile buffer
   int64_t qoff;      // offset of the query residues in the query residue buffer
   int32_t track_off; // track plans: index of the plan's first TrackChunk
-  int32_t pad_;
+  int32_t slot;      // byte profiles: bytes of a lane's slot (0 = R; more where R is no multiple of 4)
 };
 
 // Query tracks (query-pair form).  The two 16-bit halves of a chain each run
@@ -150,6 +150,8 @@ struct PairBandArgs {
   Scoring sc;
 };
 size_t pair_smem_bytes(int pbuf_bytes, int warps);
+int pair_max_warps();        // warps of a CTA, at most
+int pair_slot_bytes(int R);  // profile bytes of a lane: R rounded up to whole words
 int pair_max_ctas_per_sm(int R, int gaps, int threads, size_t smem);  // gaps: GapSet, here and below
 cudaError_t launch_pair(const PairBandArgs &a, int R, int grid, int threads, size_t smem, cudaStream_t s);
 

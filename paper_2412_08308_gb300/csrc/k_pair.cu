@@ -36,14 +36,33 @@
 namespace swgb {
 namespace {
 
-constexpr int kPairThreads = 512;  // at most 16 warps per CTA, one band each
-// Split lanes (column_step_split_int): two half-chains per lane, lanes two
-// columns apart, so a band's last lane trails its first by 63 columns.
+// Columns per step.  A lane computes two columns of its R rows in one step:
+// the step's fixed cost (the shuffles' latency, the first lane's selects, the
+// hand-off to the band below) is paid once for both, and the second column's
+// chain down the rows runs one row behind the first one's, so that a warp
+// that has its SM sub-partition to itself has two chains to interleave.  In a
+// loop over one warp per sub-partition a two-column step takes 180 cycles at R
+// = 8 and 316 at R = 16, in a band between two others 244 and 378.
+constexpr int kStepCols = 2;
+constexpr int kBlockSteps = kColBlock / kStepCols;
+// A band's last lane works on columns 62 and 63 behind the first lane's and
+// stores them one step later, at the start of its next step: 64 columns, four
+// blocks, so that the columns it stores in one block are a block of the ring.
+constexpr int kBandLagBlocks = 4;
+constexpr int kResChunk = 512;                              // target residues staged at a time (16 per lane)
+constexpr int kBandRingBytes = 2 * kResChunk + 2 * kColBlock * 8;  // per warp: residues, boundary entries
+// At most this many warps per CTA, one CTA per SM: two per SM sub-partition,
+// with up to 255 registers a thread.  (Sixteen warps of 128 registers: 473
+// against 380 cycles per step at R = 16; a pair long enough for more warps
+// gets taller bands instead, which measured faster: 1M x 1M 273 ms at R = 28
+// and two warps, 283 at R = 20 and three, 284 at R = 14 and four.)
+constexpr int kPairWarps = 8;
+// Steps unrolled: a whole block where its code fits the instruction cache, half
+// of one above (R = 8: 269 -> 244 cycles per step, R = 20: 478 -> 660).
 template <int R>
-constexpr bool kBandSplit = R % 8 == 0;
+constexpr int kUnrolled = R <= 16 ? kBlockSteps : kBlockSteps / 2;
 template <int R>
-constexpr int kBandLag = kBandSplit<R> ? 2 * 32 - 1 : 32 - 1;
-constexpr int kBandRingBytes = 320;  // residues: 2 slots x 32 B; boundary: 2 slots x 16 x 8 B
+constexpr int kSlotBytes = (R + 3) / 4 * 4;  // profile bytes of a lane
 
 struct BandIO {
   const unsigned long long *in;  // ring of the band above
@@ -58,47 +77,59 @@ struct BandIO {
 
 __device__ __forceinline__ uint32_t band_gen(int b, int nslots) { return ((uint32_t)(b / nslots) & 1u) ^ 1u; }
 
-// One band over all target columns.  Lane 0 takes the residues (cp.async ring,
-// two blocks ahead) and the band above's entries; lanes 0..15 load the entries
-// of block blk + 2 at the end of block blk and check their tags at the end of
-// block blk + 1 (loading again until they are fresh), then unpack them into
-// the shared-memory slot lane 0 reads.  Lane 31 stores one entry per column.
-// With split lanes each lane runs two half-chains a column apart (see
-// column_step_split_int).
+// The profile bytes of a lane's R rows, as words.
+template <int R>
+__device__ __forceinline__ void load_rows(const uint8_t *p, uint32_t (&w)[kSlotBytes<R> / 4]) {
+  if constexpr (R % 4 == 0) {
+    load_prof<R>(p, w);
+  } else {
+#pragma unroll
+    for (int i = 0; i < kSlotBytes<R> / 4; ++i) w[i] = reinterpret_cast<const uint32_t *>(p)[i];
+  }
+}
+
+// One band over all target columns.  Each lane passes its bottom row (H and F
+// of both columns) and the residues to the next lane by shuffle; the first
+// lane takes the residues from shared memory (staged 512 at a time, a chunk
+// ahead, by the whole warp) and the band above's entries from its slot there.
+// Residues, profile words and boundary entries of a step are fetched during
+// the step before, off the chain.  Lanes 0..15 load the next block's entries
+// during a block and check their tags at its end (loading again until they
+// are fresh).  Lane 31 stores its two columns with one 128-bit store at the
+// start of the next step, each 64-bit half an entry of its own.
+// (Per block instead, 16 entries through shared memory, residues two blocks
+// ahead by the first lane and a vote on the room in the ring: 326 against 244
+// cycles per step of a band between two others, R = 8.)
 // Returns false when a wait expired.
 template <int R>
 __device__ __forceinline__ bool band_pass(const uint8_t *__restrict__ pch, const int stride, const int lane,
-                                          const int nblk, const int npad, const uint8_t *__restrict__ target,
-                                          uint8_t *ring, const bool prev, const bool next, const Consts &cs,
-                                          int32_t &S, const BandIO &x) {
-  using W = int32_t;
-  LaneState<R, kFormInt32> st;
-  lane_reset(st, cs);
-  W outH = 0, outF = 0;
-  uint32_t outRes = kPadPair;
-  // split lanes: the lower half's residue, diagonal H and incoming F, best
-  uint32_t prevRes = kPadPair;
-  int32_t hdiagB = 0, midF = 0, S2 = 0;
+                                          const int npad, const uint8_t *__restrict__ target, uint8_t *ring,
+                                          const bool prev, const bool next, const Consts &cs, int32_t &Sout,
+                                          const BandIO &x) {
+  constexpr int PW = kSlotBytes<R> / 4;
+  int32_t Hl[R], E[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) Hl[r] = E[r] = 0;
+  int32_t outHA = 0, outFA = 0, outHB = 0, outFB = 0, hdiag = 0, S = 0;
   const int src = lane > 0 ? lane - 1 : lane;
   const bool lead = lane == 0;
-  const bool tail = lane == 31 && next;
-  const int nreal = npad / kColBlock;                // blocks of real columns
-  uint8_t *rres = ring;                              // [slot][16 B] residue codes
-  uint2 *rgb = reinterpret_cast<uint2 *>(ring + 64);  // [slot][16] (H, F) of the band above
-  const uint8_t *prow = pch + lane * R;
+  const int nreal = npad / kColBlock;  // blocks of real columns
+  const int nblk = nreal + kBandLagBlocks;
+  uint8_t *rres = ring;                                           // [2][512] residue codes
+  uint2 *rgb = reinterpret_cast<uint2 *>(ring + 2 * kResChunk);  // [2 slots][16] (H, F) of the band above
+  const uint8_t *prow = pch + lane * kSlotBytes<R>;
   bool failed = false;
 
-  auto prefetch = [&](int blk) {
-    uint8_t *d = rres + (blk & 1) * 32;
-    const int col = blk * kColBlock;
+  constexpr int kChunkBlocks = kResChunk / kColBlock;
+  auto stage = [&](int chunk) {
+    uint8_t *d = rres + (chunk & 1) * kResChunk + lane * 16;
+    const int64_t col = (int64_t)chunk * kResChunk + lane * 16;
     if (col < npad) cp_async16(d, target + col);
     else *reinterpret_cast<uint4 *>(d) = make_uint4(0x14141414u, 0x14141414u, 0x14141414u, 0x14141414u);
     cp_async_commit();
   };
-  if (lead) {
-    prefetch(0);
-    prefetch(1);
-  }
+  __syncwarp();  // (the band before this one on the warp has read its residues)
+  stage(0);
 
   // reading side: ring position and lap parity of the next block to load
   int rpos = 0, consumed = 0, since = 0;
@@ -150,7 +181,7 @@ __device__ __forceinline__ bool band_pass(const uint8_t *__restrict__ pch, const
     }
   };
   // both boundary slots start as the matrix top boundary (the band without
-  // a band above keeps it; the others overwrite block by block, and the two
+  // a band above keeps it; the others overwrite block by block, and the
   // padding blocks at the end get it back below)
   if (lane < kColBlock) {
     rgb[lane] = make_uint2(0u, 0u);
@@ -160,102 +191,138 @@ __device__ __forceinline__ bool band_pass(const uint8_t *__restrict__ pch, const
   if (prev) {
     load();
     land(0);
-    if (!failed && nreal > 1) load();
   }
+  cp_async_wait<0>();
+  __syncwarp();
 
-  // writing side: ring position, lap parity, room as last read
-  int wpos = 0, seen_cons = 0;
-  uint32_t wlap = 0u;
-  const uint32_t gen_bit = x.gen_out << 31;
+  // writing side: this band's ring at the block being stored, its lap bit,
+  // and the columns there is room for, as last read
+  int wpos = 0, room = x.window;
+  uint32_t lap_bit = 0u;
+  const uint32_t f_bias = (uint32_t)cs.go + (x.gen_out << 31);
+
+  // this step's residues (two codes) and profile words
+  uint32_t res = lead ? (uint32_t)*reinterpret_cast<const uint16_t *>(rres)
+                      : (uint32_t)(kPadCode | (kPadCode << 8));
+  uint32_t pwA[PW], pwB[PW];
+  load_rows<R>(prow + (res & 0xffu) * stride, pwA);
+  load_rows<R>(prow + (res >> 8) * stride, pwB);
 
   for (int blk = 0; blk < nblk && !failed; ++blk) {
-    if (tail) {
-      // room in this band's ring for the columns this block writes
-      const int jmax = min(blk * kColBlock + kColBlock - 1 - kBandLag<R>, npad - 1);
-      const int need = jmax + 1 - x.window;
-      if (jmax >= 0 && seen_cons < need) {
-        seen_cons = wait_flag_value(x.cons_out, need, kLongWaitBudgetCycles);
-        if (seen_cons < need) {
-          failed = true;
-          atomicExch(x.status, SW_ETIMEOUT);
-        }
+    // the block of the ring that this block stores (columns 64 behind)
+    const int wblk = blk - kBandLagBlocks;
+    const bool writes = next && wblk >= 0;  // (wblk < nreal: nblk is nreal + 4)
+    if (writes && (wblk + 1) * kColBlock > room) {
+      const int need = (wblk + 1) * kColBlock - x.window;
+      int seen = 0;
+      if (lead) seen = wait_flag_value(x.cons_out, need, kLongWaitBudgetCycles);
+      seen = __shfl_sync(0xffffffffu, seen, 0);
+      if (seen < need) {
+        failed = true;
+        if (lead) atomicExch(x.status, SW_ETIMEOUT);
+        break;
       }
+      // (no farther than the columns themselves: both terms stay in 32 bits)
+      room = seen > npad - x.window ? npad : seen + x.window;
     }
-    if (__any_sync(0xffffffffu, failed)) {
-      failed = true;
-      break;
+    // the next chunk of residues: staged half-way through this one, waited
+    // for before its last block (whose last step takes the next chunk's first)
+    if (blk % kChunkBlocks == kChunkBlocks / 2) stage(blk / kChunkBlocks + 1);
+    if (blk % kChunkBlocks == kChunkBlocks - 1) {
+      cp_async_wait<0>();
+      __syncwarp();
     }
-    const uint2 *gslot = rgb + (blk & 1) * kColBlock;
-    const uint32_t *rw = reinterpret_cast<const uint32_t *>(rres + (blk & 1) * 32);  // this block's residues
-    if (lead) cp_async_wait<1>();
+    const uint4 *gslot = reinterpret_cast<const uint4 *>(rgb + (blk & 1) * kColBlock);
+    const bool more = prev && blk + 1 < nreal;
+    unsigned long long *wp = x.out + wpos;
+    const bool tail = writes && lane == 31;
+    uint4 g = gslot[0];
+    if (more) load();
 #pragma unroll 1
-    for (int g4 = 0; g4 < kColBlock / 4; ++g4) {
-      const uint32_t wa = rw[g4];  // (used by lane 0 only)
+    for (int part = 0; part < kBlockSteps / kUnrolled<R>; ++part) {
 #pragma unroll
-      for (int s4 = 0; s4 < 4; ++s4) {
-        const int s = g4 * 4 + s4;
-        const int t = blk * kColBlock + s;
-        W inH = (W)__shfl_sync(0xffffffffu, outH, src);
-        W inF = (W)__shfl_sync(0xffffffffu, outF, src);
-        uint32_t inRes = __shfl_sync(0xffffffffu, outRes, src);
-        if (lead) {
-          // (the ring holds the pad code past the target's end, the slot the
-          // top boundary where no band lies above)
-          inRes = prmt(wa, 0u, sel_one(s4));
-          const uint2 v = gslot[s];
-          inH = (W)v.x;
-          inF = (W)v.y;
+      for (int s4 = 0; s4 < kUnrolled<R>; ++s4) {
+        const int s = part * kUnrolled<R> + s4;
+        const int t = blk * kBlockSteps + s;
+        if (tail)
+          st_relaxed_2xu64(wp + kStepCols * s, (uint32_t)outHA + lap_bit, (uint32_t)outFA + f_bias,
+                           (uint32_t)outHB + lap_bit, (uint32_t)outFB + f_bias);
+        const int32_t shHA = __shfl_sync(0xffffffffu, outHA, src);
+        const int32_t shFA = __shfl_sync(0xffffffffu, outFA, src);
+        const int32_t shHB = __shfl_sync(0xffffffffu, outHB, src);
+        const int32_t shFB = __shfl_sync(0xffffffffu, outFB, src);
+        uint32_t resN = __shfl_sync(0xffffffffu, res, src);
+        const uint32_t res0 =
+            *reinterpret_cast<const uint16_t *>(rres + ((kStepCols * t + kStepCols) & (2 * kResChunk - 1)));
+        const uint4 gN = gslot[(s + 1) & (kBlockSteps - 1)];
+        if (lead) resN = res0;
+        uint32_t pwAN[PW], pwBN[PW];
+        load_rows<R>(prow + (resN & 0xffu) * stride, pwAN);
+        load_rows<R>(prow + (resN >> 8) * stride, pwBN);
+        int32_t xA[R];  // H_diag + SM of the first column
+#pragma unroll
+        for (int r = R - 1; r >= 0; --r) xA[r] = add_byte(pwA, r, r > 0 ? Hl[r - 1] : hdiag);
+        const int32_t inHA = lead ? (int32_t)g.x : shHA;
+        int32_t fA = lead ? (int32_t)g.y : shFA;
+        const int32_t inHB = lead ? (int32_t)g.z : shHB;
+        int32_t fB = lead ? (int32_t)g.w : shFB;
+        int32_t dB = inHA;  // H of the row above at the first column
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int32_t hA = __vimax3_s32_relu(xA[r], E[r], fA);  // Eq. 1, floor included
+          const int32_t gA = hA - cs.go;
+          const int32_t e = max(E[r] - cs.ge, gA);  // Eq. 2, the second column's E
+          fA = max(fA - cs.ge, gA);                 // Eq. 3, the row below's F
+          const int32_t hB = __vimax3_s32_relu(add_byte(pwB, r, dB), e, fB);
+          const int32_t gB = hB - cs.go;
+          E[r] = max(e - cs.ge, gB);
+          fB = max(fB - cs.ge, gB);
+          S = __vimax3_s32(S, hA, hB);
+          Hl[r] = hB;
+          dB = hA;
         }
-        if constexpr (kBandSplit<R>) {
-          column_step_split_int<R>(st, hdiagB, midF, prow, stride, inRes, prevRes, inH, inF, cs, S, S2, outH,
-                                   outF);
-          outRes = prevRes;
-          prevRes = inRes;
-        } else {
-          column_step<R, kFormInt32>(st, prow, stride, inRes, inH, inF, cs, S, outH, outF);
-          outRes = inRes;
-        }
-        if (tail) {
-          const int j = t - kBandLag<R>;
-          if (j >= 0 && j < npad) {
-            const uint32_t lo = (uint32_t)outH | (wlap << 31);
-            const uint32_t hi = (uint32_t)(outF + cs.go) | gen_bit;
-            st_relaxed_u64(x.out + wpos, ((unsigned long long)hi << 32) | lo);
-            if (++wpos == x.window) {
-              wpos = 0;
-              wlap ^= 1u;
-            }
-          }
+        outHA = dB;
+        outFA = fA;
+        outHB = Hl[R - 1];
+        outFB = fB;
+        hdiag = inHB;
+        res = resN;
+        g = gN;
+#pragma unroll
+        for (int i = 0; i < PW; ++i) {
+          pwA[i] = pwAN[i];
+          pwB[i] = pwBN[i];
         }
       }
     }
-    if (lead) {
-      if (blk + 2 < nblk) prefetch(blk + 2);
-      else cp_async_commit();
+    if (writes) {
+      wpos += kColBlock;
+      if (wpos == x.window) {
+        wpos = 0;
+        lap_bit ^= 0x80000000u;
+      }
     }
-    if (prev && blk + 1 < nreal) {
+    if (more) {
       land((blk + 1) & 1);
-      if (!failed && blk + 2 < nreal) load();
     } else if (prev && blk + 1 < nblk) {
       // the padding blocks after the last real one: top boundary again
       if (lane < kColBlock) rgb[((blk + 1) & 1) * kColBlock + lane] = make_uint2(0u, 0u);
       __syncwarp();
     }
   }
-  if (lead) cp_async_wait<0>();
-  S = max(S, S2);
+  cp_async_wait<0>();
+  Sout = max(Sout, S);
   return !failed;
 }
 
 template <int R, int GAPS>
-__global__ void __launch_bounds__(kPairThreads, 1) pair_band_kernel(const PairBandArgs a) {
+__global__ void __launch_bounds__(32 * kPairWarps, 1) pair_band_kernel(const PairBandArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
   uint8_t *pbuf = smem + (size_t)warp * (a.pbuf_bytes + kBandRingBytes);
   uint8_t *ring = pbuf + a.pbuf_bytes;
   const Consts cs = make_consts<GAPS>(a.sc);
-  const int nblk = (a.npad + kBandLag<R> + kColBlock - 1) / kColBlock;
   int32_t S = 0;
   // global warp g = warp * grid + CTA: bands spread over the SMs first
   for (int b = warp * gridDim.x + blockIdx.x; b < a.nbands; b += gridDim.x * nw) {
@@ -272,7 +339,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) pair_band_kernel(const PairBa
     x.gen_out = band_gen(b, a.nslots);
     x.cons_every = a.cons_every;
     x.status = a.status;
-    const bool ok = band_pass<R>(pbuf, a.stride, lane, nblk, a.npad, a.target, ring, b > 0, b + 1 < a.nbands,
+    const bool ok = band_pass<R>(pbuf, a.stride, lane, a.npad, a.target, ring, b > 0, b + 1 < a.nbands,
                                  cs, S, x);
     __syncwarp();
     if (!ok) break;
@@ -284,16 +351,23 @@ __global__ void __launch_bounds__(kPairThreads, 1) pair_band_kernel(const PairBa
 // The kernel of a band height: with the DNA penalties compiled in at the
 // heights the planner picks (see GapSet), else the general one.
 using PairKernel = void (*)(const PairBandArgs);
+template <int R>
+PairKernel pair_kernel_of(int gaps) {
+  return gaps == kGapsDna ? pair_band_kernel<R, kGapsDna> : pair_band_kernel<R, kGapsAny>;
+}
+#define SWGB_PAIR_R_LIST(X) X(4) X(6) X(8) X(10) X(12) X(14) X(16) X(20) X(24) X(28)
 PairKernel pair_kernel(int R, int gaps) {
-  const bool d = gaps == kGapsDna;
-  if (R == 4) return pair_band_kernel<4, kGapsAny>;
-  if (R == 8) return d ? pair_band_kernel<8, kGapsDna> : pair_band_kernel<8, kGapsAny>;
-  if (R == 16) return d ? pair_band_kernel<16, kGapsDna> : pair_band_kernel<16, kGapsAny>;
-  if (R == 24) return pair_band_kernel<24, kGapsAny>;
+#define SWGB_CASE(RR) \
+  if (R == RR) return pair_kernel_of<RR>(gaps);
+  SWGB_PAIR_R_LIST(SWGB_CASE)
+#undef SWGB_CASE
   return nullptr;
 }
 
 }  // namespace
+
+int pair_max_warps() { return kPairWarps; }
+int pair_slot_bytes(int R) { return (R + 3) / 4 * 4; }
 
 size_t pair_smem_bytes(int pbuf_bytes, int warps) { return (size_t)warps * (pbuf_bytes + kBandRingBytes); }
 

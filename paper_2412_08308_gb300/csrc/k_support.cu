@@ -9,9 +9,10 @@ namespace {
 // and query row i; the pad residue (c = 20) and rows past the query end hold
 // `pad` = min(0, min SM).  Layout per query: nchunks chunks, each
 // [21][chunk_stride] bytes, chunk c covering rows c*L*R .. c*L*R + L*R - 1.
-// A residue row holds profile_slots(L) slots of R bytes; slot s serves lane
-// k = s mod L, i.e. rows k*R .. k*R + R - 1 of the chunk.  Bytes past the
-// last slot hold `pad` too.
+// A residue row holds profile_slots(L) slots of R bytes (QDesc::slot bytes
+// where that is set); slot s serves lane k = s mod L, i.e. rows k*R .. k*R +
+// R - 1 of the chunk.  Bytes past a slot's rows and past the last slot hold
+// `pad` too.
 __global__ void build_profiles_kernel(const uint8_t *__restrict__ qres, const QDesc *__restrict__ qd,
                                       const int8_t *__restrict__ submat, int32_t pad,
                                       uint8_t *__restrict__ prof) {
@@ -22,6 +23,7 @@ __global__ void build_profiles_kernel(const uint8_t *__restrict__ qres, const QD
   const uint8_t *q = qres + d.qoff;
   const int LR = d.L * d.R;
   const int slots = profile_slots(d.L);
+  const int sb = d.slot ? d.slot : d.R;  // bytes of a slot
   const int64_t words = (int64_t)d.nchunks * d.chunk_bytes / 4;
   uint32_t *out = reinterpret_cast<uint32_t *>(prof + d.prof_off);
   for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words; w += (int64_t)gridDim.x * blockDim.x) {
@@ -33,10 +35,10 @@ __global__ void build_profiles_kernel(const uint8_t *__restrict__ qres, const QD
     uint32_t v = 0;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      const int slot = (xb + b) / d.R;
-      const int row = c * LR + (slot % d.L) * d.R + (xb + b - slot * d.R);
+      const int slot = (xb + b) / sb, r = xb + b - slot * sb;
+      const int row = c * LR + (slot % d.L) * d.R + r;
       int32_t val = pad;
-      if (slot < slots && row < d.m && rho < kAlphabet) val = sm[q[row] * kAlphabet + rho];
+      if (slot < slots && r < d.R && row < d.m && rho < kAlphabet) val = sm[q[row] * kAlphabet + rho];
       v |= ((uint32_t)val & 0xffu) << (8 * b);
     }
     out[w] = v;

@@ -56,6 +56,41 @@ struct PairScratch {
   }
 };
 
+// Rows per lane of the bands: the height with the least modelled time.  A
+// warp sweeps its bands over the target in two-column steps, each band about
+// 51 steps behind the one above it (31 lanes, a block of 8 steps of entries
+// that has to be complete and one that is loaded ahead, ~700 cycles for the
+// hand-off); a step takes, from timings of 23 to 1,266 bands at every height,
+// 105 + 17.8 R cycles with one warp per SM sub-partition and 70 + 33.7 R with
+// two (within 8 %).  Bands that do not fit the GPU at once come in rounds.
+// Taller bands cost less per cell and have fewer hand-offs, shorter ones
+// spread a pair over more sub-partitions; one band too many for one per
+// sub-partition (or per two) slows every band, since they move in step.
+//   162K x 172K: R = 10 15.2 ms (507 bands); 8 17.7, 12 16.2, 16 18.5
+//   20K x 25K: R = 4 and 6 1.82 ms, 8 1.92, 16 2.61
+//   300K x 310K: R = 16 33.6 ms, 8 35.2, 12 42.1
+//   1M x 1M: R = 28 273 ms, 24 348, 16 307
+int pick_rows(int64_t m, int64_t n, int sms) {
+  static const int kRows[] = {4, 6, 8, 10, 12, 14, 16, 20, 24, 28};
+  const int64_t parts = 4 * (int64_t)sms;
+  int best = kRows[0];
+  double best_t = 1e300;
+  for (int R : kRows) {
+    const int64_t nb = (m + 32 * R - 1) / (32 * R);
+    const double step1 = 105 + 17.8 * R, step2 = 70 + 33.7 * R;
+    const double fill = 51.0 * (double)std::min<int64_t>(nb, 2 * parts);
+    // full rounds of two per sub-partition, then what is left
+    const int64_t rounds = nb / (2 * parts), left = nb - rounds * 2 * parts;
+    double t = 0.5 * (double)n * ((double)rounds * step2 + (left == 0 ? 0.0 : left <= parts ? step1 : step2));
+    t += fill * (rounds > 0 || left > parts ? step2 : step1);
+    if (t < best_t) {
+      best_t = t;
+      best = R;
+    }
+  }
+  return best;
+}
+
 }  // namespace
 }  // namespace swgb
 
@@ -111,13 +146,9 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
 
   // geometry: bands of 32 * R query rows, one warp each; each warp stages its
   // band's profile (21 residue rows) in shared memory
-  // Bands in flight are the parallelism, one warp each; the warps of a CTA are
-  // the bands per SM, so that every SM gets bands.  Rows per lane 16, or 8
-  // when that leaves fewer than 3 bands per SM (more, shorter bands fill the
-  // SMs better there, while elsewhere the longer ramp of the band pipeline
-  // and the per-column overhead of shorter bands cost more; 4 and 24 rows
-  // measured slower on every pair).
-  const int R = o.rows_per_lane ? o.rows_per_lane : ((m + 511) / 512 < 3 * (int64_t)sms ? 8 : 16);
+  // Bands in flight are the parallelism, one warp each, dealt to the SMs in
+  // turn: up to one per SM sub-partition, then two.
+  const int R = o.rows_per_lane ? o.rows_per_lane : pick_rows(m, n, sms);
   const int64_t B = 32 * (int64_t)R;
   const int64_t nbands64 = (m + B - 1) / B;
   if (nbands64 >= ((int64_t)1 << 31)) return pair_fail(SW_EINVAL, "sw_align_pair: too many bands");
@@ -127,10 +158,11 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
   qd.L = 32;
   qd.R = R;
   qd.nchunks = (int32_t)nbands64;
-  qd.chunk_stride = (int32_t)round_up((int64_t)profile_slots(32) * R, 128);
+  qd.slot = pair_slot_bytes(R);
+  qd.chunk_stride = (int32_t)round_up((int64_t)profile_slots(32) * qd.slot, 128);
   qd.chunk_bytes = kProfRows * qd.chunk_stride;
   const int pbuf_bytes = (int)round_up(qd.chunk_bytes, 128);
-  int warps = (int)std::min<int64_t>(16, std::max<int64_t>(1, (nbands64 + sms - 1) / sms));
+  int warps = (int)std::min<int64_t>(pair_max_warps(), std::max<int64_t>(1, (nbands64 + sms - 1) / sms));
   while (warps > 1 && pair_smem_bytes(pbuf_bytes, warps) > 200 * 1024) --warps;
   if (o.band_warps) warps = std::min(warps, o.band_warps);
   const int threads = 32 * warps;
@@ -166,7 +198,7 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
   int64_t window = o.ring_columns ? o.ring_columns : 32768;
   window = std::max<int64_t>(window, round_up(((npad + gw - 1) / gw + 64) * 8 / 7 + 1, kColBlock));
   window = std::min<int64_t>(window, npad);
-  const int cons_every = (int)std::max<int64_t>(1, std::min<int64_t>(16, window / kColBlock / 8));
+  const int cons_every = (int)std::max<int64_t>(1, std::min<int64_t>(128, window / kColBlock / 8));
 
   // device scratch: query, target, matrix, plan, profile, strips, progress, result words
   const size_t b_q = round_up(m, 256), b_t = round_up(npad, 256), b_sub = 512, b_qd = 256;
