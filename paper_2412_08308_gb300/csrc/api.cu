@@ -56,8 +56,25 @@ int cuda_fail(cudaError_t e, const char *what) {
 
 inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
-// transposed jobs: rows per lane
-constexpr int kTrackRows = 16;
+// Rows per lane of the transposed jobs (heights whose kernels exist), and the
+// cycles of one step (two columns) of a band that has its SM sub-partition to
+// itself, or per band where two or more share it: from timings of 500 to
+// 20,000 proteins at every height.  (More than 16 rows share a launch with the
+// 16-row lanes of longer sequences, whose code they evict.)
+struct TrackHeight {
+  int rows;
+  double packed1, packed2, int1, int2;
+};
+constexpr TrackHeight kTrackHeights[] = {{8, 302, 211, 229, 161},
+                                         {12, 382, 318, 291, 221},
+                                         {16, 461, 397, 353, 287},
+                                         {20, 540, 486, 415, 373},
+                                         {24, 620, 620, 477, 498}};
+double track_step_cycles(bool packed, int rows, int w) {
+  for (const TrackHeight &h : kTrackHeights)
+    if (h.rows == rows) return w <= 1 ? (packed ? h.packed1 : h.int1) : w * (packed ? h.packed2 : h.int2);
+  return 1e9;
+}
 
 int sm_count(int dev) {
   int n = 0;
@@ -149,106 +166,113 @@ bool is_device_ptr(const void *p) {
 }
 
 // --- the database in row tracks (transposed jobs, k_band.cu) ----------------
-// Sequences (sorted order, longest first), padded to whole lanes of tR rows,
-// go to the 16-bit tracks (f = 0; two tracks share each word) when their
-// length is at most `cut`, else to int32 tracks (f = 1).  A sequence longer
-// than a band (32 tR rows) gets a track of its own, whose bands run as a
-// pipeline; the others are packed into one-band tracks without crossing a
-// band boundary (each into the first of the last 64 open tracks with room),
-// so those bands depend on no other band.  Empty sequences score 0 without a
-// lane.
+// Sequences (sorted order, longest first) go to the 16-bit tracks (f = 0; two
+// tracks share each word) when their length is at most `cut`, else to int32
+// tracks (f = 1).  A sequence that fits a band (32 lanes of tR rows) takes
+// whole lanes of the fullest band that has room, so these bands depend on no
+// other band.  A longer one gets a track of its own, in lanes of
+// track_long_rows(tR) rows, whose bands run as a pipeline: its last band
+// starts about 50 steps per band above it late, and the shorter lanes' steps
+// make up for that (one 144-residue query x 2,000 proteins: the few proteins
+// past 768 rows cost 15 of 58 us in 24-row lanes).  Lanes that it leaves free
+// in its last band take short sequences too.  Empty sequences score 0 without
+// a lane.
 struct TrackSeg {
-  int32_t pos, row0, rows, bin;  // sequence, first row in its track, rows (whole lanes), track
+  int32_t pos, bin, lane0, lanes;  // sequence, track, first lane in the track, lanes
 };
 struct TrackBins {
   std::vector<TrackSeg> seg[2];
-  std::vector<int32_t> used[2];  // rows of each track
+  std::vector<int32_t> used[2];  // lanes of each track
+  std::vector<char> tall[2];     // 1: tR rows per lane (one band), 0: track_long_rows(tR)
 };
 // a pipeline of bands: one int32 track, or two 16-bit tracks sharing words
 struct TrackPipe {
-  int32_t packed, nb, lane0;
+  int32_t packed, nb, lane0, rows;  // rows per lane
 };
 
 void bin_tracks(const std::vector<int32_t> &len, int tR, int32_t cut, TrackBins &b) {
-  const int32_t kRows = 32 * tR;  // rows per band
+  const int tL = track_long_rows(tR);
+  // tracks by the lanes free in their last band, per height
+  std::vector<int32_t> room[2][2][33];
   for (int f = 0; f < 2; ++f) {
     b.seg[f].clear();
     b.used[f].clear();
+    b.tall[f].clear();
   }
   for (size_t k = 0; k < len.size(); ++k) {
     if (len[k] == 0) continue;
     const int f = len[k] <= cut ? 0 : 1;
-    const int32_t rows = (int32_t)round_up(len[k], tR);
-    std::vector<int32_t> &U = b.used[f];
-    if (rows > kRows) {
-      b.seg[f].push_back({(int32_t)k, 0, rows, (int32_t)U.size()});
-      U.push_back(rows);
-      continue;
+    const int32_t lanes_t = (len[k] + tR - 1) / tR, lanes_l = (len[k] + tL - 1) / tL;
+    int32_t bin = -1, tall = lanes_t <= 32 ? 1 : 0, lanes = tall ? lanes_t : lanes_l;
+    if (tall) {  // the track with room whose free rows it leaves fewest of
+      int32_t best = 32 * tR + 1;
+      for (int h = 0; h < 2; ++h)
+        for (int32_t r = h ? lanes_t : lanes_l; r <= 32; ++r)
+          if (!room[f][h][r].empty()) {
+            const int32_t left = (r - (h ? lanes_t : lanes_l)) * (h ? tR : tL);
+            if (left < best) {
+              best = left;
+              tall = h;
+              lanes = h ? lanes_t : lanes_l;
+              bin = room[f][h][r].back();
+            }
+            break;
+          }
     }
-    size_t i = U.size();
-    for (size_t j = U.size() > 64 ? U.size() - 64 : 0; j < U.size(); ++j)
-      if (U[j] <= kRows - rows) {
-        i = j;
-        break;
-      }
-    if (i == U.size()) U.push_back(0);
-    b.seg[f].push_back({(int32_t)k, U[i], rows, (int32_t)i});
-    U[i] += rows;
+    if (bin < 0) {
+      bin = (int32_t)b.used[f].size();
+      b.used[f].push_back(0);
+      b.tall[f].push_back((char)tall);
+    } else {
+      room[f][tall][32 - (b.used[f][bin] + 31) % 32 - 1].pop_back();
+    }
+    b.seg[f].push_back({(int32_t)k, bin, b.used[f][bin], lanes});
+    b.used[f][bin] += lanes;
+    room[f][tall][32 - (b.used[f][bin] + 31) % 32 - 1].push_back(bin);
   }
 }
 
-// Bands of one query over all pipelines: the tracks ordered by band count
-// (longest first), 16-bit ones paired.
-int64_t track_bands(const TrackBins &b, int tR) {
-  const int32_t kRows = 32 * tR;
-  int64_t total = 0;
-  for (int f = 0; f < 2; ++f) {
-    std::vector<int32_t> nb(b.used[f].size());
-    for (size_t t = 0; t < nb.size(); ++t) nb[t] = (b.used[f][t] + kRows - 1) / kRows;
-    std::sort(nb.begin(), nb.end(), std::greater<int32_t>());
-    for (size_t i = 0; i < nb.size(); i += (f == 0 ? 2 : 1)) total += nb[i];
-  }
-  return total;
-}
-
-// The pipelines (deeper first; 16-bit ones pair consecutive tracks in that
-// order) and their lane table: band b, lane l of a pipeline covers rows
-// (32 b + l) tR .. + tR - 1 of its track(s); each segment writes its own
-// lanes (whole lanes from a lane boundary), the others stay idle.
+// The pipelines (deeper first; 16-bit ones pair consecutive tracks of the same
+// height in that order) and their lane table: band b, lane l of a pipeline
+// covers the rows of lane 32 b + l of its track(s); each segment writes its
+// own lanes, the others stay idle.
 void lay_tracks(const TrackBins &b, int tR, std::vector<TrackPipe> &pipes, std::vector<TrackLane> &lanes) {
-  const int32_t kRows = 32 * tR;
   pipes.clear();
   lanes.clear();
+  const int rows_of[2] = {track_long_rows(tR), tR};
   for (int f = 0; f < 2; ++f) {
     const std::vector<int32_t> &U = b.used[f];
     const int32_t B = (int32_t)U.size();
-    auto bands = [&](int32_t t) { return (int32_t)((U[t] + kRows - 1) / kRows); };
+    auto bands = [&](int32_t t) { return (U[t] + 31) / 32; };
     std::vector<int32_t> order(B), base(B), high(B);
     std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return bands(x) > bands(y); });
-    const int32_t step = f == 0 ? 2 : 1;
-    for (int32_t i = 0; i < B; i += step) {
-      const int32_t ta = order[i], tb = (f == 0 && i + 1 < B) ? order[i + 1] : -1;
-      const int32_t nb = std::max(bands(ta), tb >= 0 ? bands(tb) : 1);
-      TrackPipe pp{f == 0 ? 1 : 0, nb, (int32_t)lanes.size()};
+    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+      return b.tall[f][x] != b.tall[f][y] ? b.tall[f][x] < b.tall[f][y] : bands(x) > bands(y);
+    });
+    for (int32_t i = 0; i < B; ++i) {
+      const int32_t ta = order[i];
+      const bool pair = f == 0 && i + 1 < B && b.tall[f][order[i + 1]] == b.tall[f][ta];
+      TrackPipe pp{f == 0 ? 1 : 0, bands(ta), (int32_t)lanes.size(), rows_of[(int)b.tall[f][ta]]};
       base[ta] = pp.lane0;
       high[ta] = 0;
-      if (tb >= 0) {
-        base[tb] = pp.lane0;
-        high[tb] = 1;
+      if (pair) {  // (bands(order[i + 1]) <= bands(ta): sorted)
+        ++i;
+        base[order[i]] = pp.lane0;
+        high[order[i]] = 1;
       }
-      lanes.resize(lanes.size() + 32 * (size_t)nb, TrackLane{-1, 0, -1, 0});
+      lanes.resize(lanes.size() + 32 * (size_t)pp.nb, TrackLane{-1, 0, -1, 0});
       pipes.push_back(pp);
     }
     for (const TrackSeg &g : b.seg[f]) {
-      TrackLane *L = lanes.data() + base[g.bin] + g.row0 / tR;
-      for (int32_t k = 0; k < g.rows / tR; ++k) {
+      const int32_t rows = rows_of[(int)b.tall[f][g.bin]];
+      TrackLane *L = lanes.data() + base[g.bin] + g.lane0;
+      for (int32_t k = 0; k < g.lanes; ++k) {
         if (high[g.bin]) {
           L[k].pb = g.pos;
-          L[k].rb = k * tR;
+          L[k].rb = k * rows;
         } else {
           L[k].pa = g.pos;
-          L[k].ra = k * tR;
+          L[k].ra = k * rows;
         }
       }
     }
@@ -310,6 +334,7 @@ struct sw_db {
   struct TrackLayout {
     int32_t tR = 0, cut = 0;
     int64_t bands = 0;    // bands of one query over all pipelines
+    int32_t deepest = 1;  // most bands of a pipeline
     int64_t n_lanes = 0;
     std::vector<TrackPipe> pipes;
     TrackLane *d_lanes = nullptr;
@@ -328,8 +353,8 @@ struct sw_db {
       cudaGetLastError();
       return nullptr;
     }
-    // at most one lane per tR residues and one more per sequence
-    if ((total / tR + n) * (int64_t)sizeof(TrackLane) > kTrackLayoutBytes) return nullptr;
+    // at most one lane per track_long_rows(tR) residues and one more per sequence
+    if ((total / track_long_rows(tR) + n) * (int64_t)sizeof(TrackLane) > kTrackLayoutBytes) return nullptr;
     TrackBins b;
     bin_tracks(h_len, tR, cut, b);
     std::unique_ptr<TrackLayout> t(new TrackLayout());
@@ -337,7 +362,11 @@ struct sw_db {
     t->cut = cut;
     std::vector<TrackLane> lanes;
     lay_tracks(b, tR, t->pipes, lanes);
-    for (const TrackPipe &p : t->pipes) t->bands += p.nb;
+    if ((int64_t)(lanes.size() * sizeof(TrackLane)) > kTrackLayoutBytes) return nullptr;
+    for (const TrackPipe &p : t->pipes) {
+      t->bands += p.nb;
+      t->deepest = std::max(t->deepest, p.nb);
+    }
     t->n_lanes = (int64_t)lanes.size();
     if (!lanes.empty()) {
       void *d = nullptr;
@@ -794,17 +823,16 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   //    units, all its bands sweeping the stream together.  A unit whose pair
   //    with the query could pass the 16-bit range is split into its
   //    sequences in int32; the others keep two sequences per word.  Streams
-  //    are cut so that every warp of one launch gets about two jobs' worth
-  //    of columns (one unit at least);
+  //    are cut so that every warp of one launch gets about one and a half
+  //    jobs' worth of columns (one unit at least);
   //  - every shorter query runs transposed: the database sequences are the
-  //    rows, stacked in row tracks of whole lanes (16 rows; 8 beside
-  //    band-stream jobs; 24 when that gives one band per SM sub-partition),
-  //    and the query the columns; each band of a track is one warp, several
-  //    short sequences share a band, and the bands of a longer one run as a
-  //    pipeline.  In packed mode two tracks share each word (their
-  //    substitution bytes paired per row), except sequences whose pair with
-  //    the longest of these queries could pass the 16-bit range (int32
-  //    tracks).
+  //    rows, stacked in row tracks of whole lanes (8 to 24 rows, the height
+  //    with the least modelled time), and the query the columns; each band of
+  //    a track is one warp, several short sequences share a band, and the
+  //    bands of a longer one run as a pipeline.  In packed mode two tracks
+  //    share each word (their substitution bytes paired per row), except
+  //    sequences whose pair with the longest of these queries could pass the
+  //    16-bit range (int32 tracks).
   // The inter- and intra-task kernels are then not used.  If the rings (one
   // entry per column between consecutive bands) do not fit a memory budget,
   // the batch takes the regular plan.
@@ -822,6 +850,47 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   std::vector<int64_t> qt_off(std::max<int64_t>(n_queries, 1), 0);
   std::vector<int32_t> qt_npad(std::max<int64_t>(n_queries, 1), 16);
   bool band_mode = false;
+  // Bands of one query in lanes of tR rows, and the most bands of one
+  // sequence, estimated from the length histogram.
+  auto track_estimate = [&](int tR, const sw_db::UnitStats &single, double *bands, int64_t *deepest) {
+    const int tL = track_long_rows(tR);
+    double lanes = 0;
+    *bands = 0;
+    *deepest = 1;
+    for (size_t h = 1; h < single.hist.size(); ++h) {
+      if (!single.hist[h]) continue;
+      const int64_t len = (int64_t)h * kColBlock - 7;  // (the middle of the bin)
+      if (len <= 32 * tR) {
+        lanes += (double)single.hist[h] * (double)((len + tR - 1) / tR);
+      } else {
+        const int64_t nb = (len + 32 * tL - 1) / (32 * tL);
+        *bands += (double)(single.hist[h] * nb);
+        *deepest = std::max(*deepest, nb);
+        // (short sequences fill most of what the last band leaves)
+        lanes -= 0.8 * (double)single.hist[h] * (double)(32 * tL * nb - len) / tR;
+      }
+    }
+    *bands = std::ceil((*bands + std::max(0.0, lanes) / 32 / 0.98) * (packed ? 0.5 : 1.0));
+  };
+  // Modelled time (cycles) of the transposed jobs: their bands over the SM
+  // sub-partitions, up to the launch's residency at a time; at least the
+  // longest pipeline, whose bands start about 50 steps after one another.
+  auto track_time = [&](int tR, int occ, double bands, int64_t deepest) {
+    double work = 0, steps_max = 0, nb = 0;
+    for (int64_t q = 0; q < n_queries; ++q) {
+      if (!track_q[q]) continue;
+      const double steps = (double)(round_up(std::max(1, qlen(q)), kColBlock) + 64) / 2;
+      work += bands * steps;
+      steps_max = std::max(steps_max, steps);
+      nb += bands;
+    }
+    const double parts = 4.0 * sms;
+    const int w = (int)std::max(1.0, std::min((double)occ, std::ceil(nb / parts)));
+    const double step = track_step_cycles(packed, tR, w);
+    const double all = nb > parts * w ? work * step / (parts * w) + 0.5 * steps_max * step : steps_max * step;
+    const double chain = (steps_max + 50.0 * (double)(deepest - 1)) * track_step_cycles(packed, track_long_rows(tR), w);
+    return deepest > 1 ? std::max(all, chain) : all;
+  };
   if (o.band_stream != 1 && (o.band_stream == 2 || latency_bound) && n > 0 && n_queries > 0) {
     const int brows = 32 * bR;
     bool any_band = false, any_track = false;
@@ -833,12 +902,27 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
     }
     const int bmax = any_band ? cached_occupancy(1, bR, 0, gaps, 0, 0) : 1;
     int bocc = bmax;
-    // transposed jobs beside band-stream jobs take 8-row lanes: twice the
-    // bands, each half the work per step, which fill in around the
-    // band-stream pipelines (homolog workload 2.29 -> 2.14 ms, A/B medians);
-    // alone (one short query) 16-row lanes are faster (0.081 against 0.084 ms)
-    const int tRows = any_band ? 8 : kTrackRows;
-    int tocc = any_track ? cached_occupancy(2, tRows, 0, gaps, 0, 0) : 1;
+    // rows per lane of the transposed jobs, in order of the modelled time
+    struct TrackChoice {
+      double time;
+      int tR, occ;
+    };
+    std::vector<TrackChoice> heights;
+    if (any_track) {
+      const sw_db::UnitStats &single = db->units(false);
+      for (const TrackHeight &h : kTrackHeights) {
+        const int tR = h.rows;
+        const int occ = cached_occupancy(2, tR, 0, gaps, 0, 0);
+        if (occ <= 0) continue;
+        double bands = 0;
+        int64_t deepest = 1;
+        track_estimate(tR, single, &bands, &deepest);
+        heights.push_back({track_time(tR, occ, bands, deepest), tR, occ});
+      }
+      std::sort(heights.begin(), heights.end(),
+                [](const TrackChoice &x, const TrackChoice &y) { return x.time < y.time; });
+    }
+    int tocc = !any_track ? 1 : heights.empty() ? 0 : heights[0].occ;
     int64_t ring = 0, band = 0, tring = 0, tband = 0, n_tlanes = 0;
     if (bocc > 0 && tocc > 0) {
       // band jobs: each band query against every unit
@@ -878,9 +962,11 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
             lists.push_back(std::move(*L));
           }
       }
-      // Streams are cut into jobs of about per_warp columns, two jobs per warp
-      // of the launch (a warp that finishes early takes a band of the second
-      // wave, whose pipeline fill overlaps the first wave's drain).  Units
+      // Streams are cut into jobs of about per_warp columns, three jobs per two
+      // warps of the launch (a warp that finishes early takes a band of the
+      // second wave, whose pipeline fill overlaps the first wave's drain; one,
+      // two and three jobs per warp: 663, 564, 559 against 528 us for a
+      // 1,301-residue query x 5,000 proteins).  Units
       // are not cut, so an int32 unit wider than per_warp makes a job that
       // sets the pace of the launch: it runs in bands of half the height
       // (half the work per step; its steps run one after the other), and if
@@ -888,7 +974,7 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
       // (those of every CTA on the SM, all computing), would outlast the
       // launch's average load, the launch keeps one CTA per SM (a choice
       // only for band heights whose CTAs fit twice on an SM).
-      constexpr double kWaves = 2.0;
+      constexpr double kWaves = 1.5;
       const int wpc = band_threads() / 32;  // warps per CTA
       auto per_warp_at = [&](int occ) {
         return std::max<int64_t>(1, (int64_t)std::ceil(total / ((double)sms * occ * wpc * kWaves)));
@@ -974,6 +1060,7 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
             j.q = (int32_t)q;
             j.packed = pp.packed;
             j.nb = pp.nb;
+            j.rows = pp.rows;
             j.band0 = (int32_t)tband;
             j.lane0 = pp.lane0;
             j.ring0 = tring;
@@ -984,39 +1071,26 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
           }
       };
       if (any_track) {
-        // one wave of 16-row bands that leaves some SM sub-partitions two
-        // bands: 24-row lanes (768-row bands, one CTA of 4 warps per SM) when
-        // their bands then fit one per sub-partition -- each band's steps no
-        // longer share the issue slots.  One 144-residue query x 2,000
-        // proteins, packed: 0.081-0.085 -> 0.066 ms (32-row lanes the same);
-        // int32 (twice the bands) and larger databases stay at 16 rows
-        // (8,000 proteins: 0.189 ms at 16 rows, 0.228 at 24).  The layouts
-        // come from the database's kept ones where it keeps them, so that
-        // repeated searches skip the binning and the lane upload.
+        // the height with the least modelled time; one that its packed bands
+        // make slower than the next one's estimate gives way to that.  The
+        // layouts come from the database's kept ones where it keeps them, so
+        // that repeated searches skip the binning and the lane upload.
         TrackBins &bins = scratch.bins;
-        TrackBins bins24;
-        int tR = tRows;
-        const sw_db::TrackLayout *lay = db->track_layout(tR, cut, s);
-        if (!lay) bin_tracks(db->h_len, tR, cut, bins);
-        const int64_t subparts = 4 * (int64_t)sms;
-        const int64_t bands16 =
-            (!any_band && tRows == 16) ? (lay ? lay->bands : track_bands(bins, 16)) * n_track_q : 0;
-        if (bands16 > subparts && bands16 <= subparts * tocc) {
-          const int occ24 = cached_occupancy(2, 24, 0, gaps, 0, 0);
-          const sw_db::TrackLayout *lay24 = nullptr;
-          int64_t bands24 = 0;
-          if (occ24 > 0) {
-            lay24 = db->track_layout(24, cut, s);
-            if (!lay24) bin_tracks(db->h_len, 24, cut, bins24);
-            bands24 = (lay24 ? lay24->bands : track_bands(bins24, 24)) * n_track_q;
-          }
-          if (occ24 > 0 && bands24 <= subparts && bands24 <= (int64_t)sms * occ24 * (track_threads() / 32)) {
-            tR = 24;
-            tocc = occ24;
-            lay = lay24;
-            if (!lay) std::swap(bins, bins24);
+        TrackChoice c = heights[0];
+        const sw_db::TrackLayout *lay = db->track_layout(c.tR, cut, s);
+        if (lay) c.time = track_time(c.tR, c.occ, (double)lay->bands, lay->deepest);
+        for (size_t k = 1; lay && k < heights.size() && heights[k].time < c.time; ++k) {
+          const sw_db::TrackLayout *other = db->track_layout(heights[k].tR, cut, s);
+          if (!other) break;
+          const double t = track_time(heights[k].tR, heights[k].occ, (double)other->bands, other->deepest);
+          if (t < c.time) {
+            c = {t, heights[k].tR, heights[k].occ};
+            lay = other;
           }
         }
+        if (!lay) bin_tracks(db->h_len, c.tR, cut, bins);
+        const int tR = c.tR;
+        tocc = c.occ;
         if (lay) {
           make_jobs(lay->pipes);
           Q->d_tlanes = lay->d_lanes;  // the database's (not the batch's block)
@@ -1649,7 +1723,6 @@ int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev
       ba.n_tpos = Q->n_btargets;
       ba.sc = Q->sc;
       ba.status = w + 2;
-      ba.short_int = packed ? 1 : 0;
       SW_CUDA(launch_band(ba, Q->bR, Q->bgrid, Q->bone, Q->side), "band-stream kernel");
     }
     InterArgs b = a;

@@ -1,4 +1,4 @@
-// Cell arithmetic shared by the inter-task, intra-task and pair-band kernels:
+// Cell arithmetic shared by the inter-task and intra-task kernels:
 // one column step of R query rows owned by one lane (Sec. 2.2 Eqs. 1-3), or,
 // with split lanes, the lane's two halves of R/2 rows a column apart.
 //
@@ -198,32 +198,6 @@ __device__ __forceinline__ void word_rows(uint32_t hd0, const uint32_t (&p)[N], 
   S = __vimax3_s16x2(S, a, b);
 }
 
-// word_rows with a one-operation chain down the rows, for kernels bound by
-// one chain's latency rather than by throughput (the band-stream and
-// transposed jobs of small batches).  U = max(H_diag + SM, E, 0) does not
-// depend on the row above; since Ge <= Go, the F passed down is
-// max(F - Ge, H - Go) = max(F - Ge, U - Go, F - Go) = max(F - Ge, U - Go), so
-// the only operation on the chain is that max-add, and H = max(U, F), the
-// running best and E' = max(E - Ge, H - Go) hang off it.  One more maximum
-// and one more addition per word than word_rows.
-template <int R0, int N, int R>
-__device__ __forceinline__ void word_rows_short(uint32_t hd0, const uint32_t (&p)[N], uint32_t (&E)[R],
-                                                uint32_t (&Hl)[R], uint32_t &f, uint32_t &S, const Consts &cs) {
-  static_assert(R0 + N <= R && N % 2 == 0, "rows in range, whole pairs of rows");
-  uint32_t u[N];
-#pragma unroll
-  for (int r = N - 1; r >= 0; --r)
-    u[r] = __vimax_s16x2_relu(__vadd2(r > 0 ? Hl[R0 + r - 1] : hd0, p[r]), E[R0 + r]);  // max(H_diag + SM, E, 0)
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    const uint32_t h = __vmaxs2(u[r], f);  // H = max(U, F)
-    f = __vmaxs2(__vsub2(f, cs.geW), __vsub2(u[r], cs.goW));
-    E[R0 + r] = __vmaxs2(__vsub2(E[R0 + r], cs.geW), __vsub2(h, cs.goW));
-    Hl[R0 + r] = h;
-    if (r & 1) S = __vimax3_s16x2(S, Hl[R0 + r - 1], h);
-  }
-}
-
 template <int FORM>
 using Word = typename std::conditional<FORM != kFormInt32, uint32_t, int32_t>::type;
 
@@ -248,26 +222,6 @@ __device__ __forceinline__ void int_rows_of(int32_t hd0, Add add, int32_t (&E)[R
     const int32_t hgo = h - cs.go;
     E[R0 + r] = max(E[R0 + r] - cs.ge, hgo);
     f = max(f - cs.ge, hgo);
-    Hl[R0 + r] = h;
-    if (r & 1) S = __vimax3_s32(S, Hl[R0 + r - 1], h);
-  }
-}
-
-// int_rows_of with the one-operation F chain of word_rows_short, for the
-// int32 units of the 16-bit path's small-batch jobs (pairs that could pass
-// the 16-bit range).
-template <int R0, int N, int R, class Add>
-__device__ __forceinline__ void int_rows_short_of(int32_t hd0, Add add, int32_t (&E)[R], int32_t (&Hl)[R], int32_t &f,
-                                                  int32_t &S, const Consts &cs) {
-  static_assert(R0 + N <= R && N % 2 == 0, "rows in range, whole pairs of rows");
-  int32_t u[N];
-#pragma unroll
-  for (int r = N - 1; r >= 0; --r) u[r] = __vimax_s32_relu(add(r, r > 0 ? Hl[R0 + r - 1] : hd0), E[R0 + r]);
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    const int32_t h = max(u[r], f);
-    f = max(f - cs.ge, u[r] - cs.go);
-    E[R0 + r] = max(E[R0 + r] - cs.ge, h - cs.go);
     Hl[R0 + r] = h;
     if (r & 1) S = __vimax3_s32(S, Hl[R0 + r - 1], h);
   }
@@ -310,8 +264,7 @@ __device__ __forceinline__ void lane_reset(LaneState<R, FORM> &st, const Consts 
 // 32 lanes of a warp read 32 consecutive 16-byte groups: no bank conflict).
 // Outputs the (H, F) pair for the row below: H of the last row, F of the row
 // below it.
-// SHORTF: rows by word_rows_short / int_rows_short_of, the one-operation chain.
-template <int R, int FORM, bool SHORTF = false>
+template <int R, int FORM>
 __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_t *prow, int stride,
                                             uint32_t res, Word<FORM> inH, Word<FORM> inF, const Consts &cs,
                                             Word<FORM> &S, Word<FORM> &outH, Word<FORM> &outF, int gstride = 0) {
@@ -325,8 +278,7 @@ __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_
       pw[4 * i + 0] = v.x; pw[4 * i + 1] = v.y; pw[4 * i + 2] = v.z; pw[4 * i + 3] = v.w;
     }
     uint32_t f = (uint32_t)inF, s = (uint32_t)S;
-    if constexpr (SHORTF) word_rows_short<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
-    else word_rows<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
+    word_rows<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
     S = (W)s;
     outH = st.Hl[R - 1];
     outF = (W)f;
@@ -338,8 +290,7 @@ __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_
 #pragma unroll
     for (int r = 0; r < R; ++r) pw[r] = prmt(pa[r >> 2], pb[r >> 2], sel_pair(r & 3));  // (SM_a, SM_b), signed halves
     uint32_t f = (uint32_t)inF, s = (uint32_t)S;
-    if constexpr (SHORTF) word_rows_short<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
-    else word_rows<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
+    word_rows<0, R>((uint32_t)st.hdiag, pw, st.E, st.Hl, f, s, cs);
     S = (W)s;
     outH = st.Hl[R - 1];
     outF = (W)f;
@@ -347,9 +298,7 @@ __device__ __forceinline__ void column_step(LaneState<R, FORM> &st, const uint8_
     int32_t f = inF, s = S;
     uint32_t pa[R / 4];
     load_prof<R>(prow + (res & 0xffu) * stride, pa);
-    const auto add = [&](int r, int32_t h) { return add_byte(pa, r, h); };
-    if constexpr (SHORTF) int_rows_short_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
-    else int_rows_of<0, R, R>(st.hdiag, add, st.E, st.Hl, f, s, cs);
+    int_rows_of<0, R, R>(st.hdiag, [&](int r, int32_t h) { return add_byte(pa, r, h); }, st.E, st.Hl, f, s, cs);
     S = (W)s;
     outH = st.Hl[R - 1];
     outF = (W)f;
@@ -414,7 +363,7 @@ __device__ __forceinline__ void column_step_split(LaneState<R, FORM> &st, uint32
   st.hdiag = inH;
 }
 
-// int32 form with split lanes (the pair-band and intra-task kernels): as
+// int32 form with split lanes (the intra-task kernel): as
 // column_step_split, with byte profiles.
 template <int R>
 __device__ __forceinline__ void column_step_split_int(LaneState<R, kFormInt32> &st, int32_t &hdiagB, int32_t &midF,

@@ -189,8 +189,6 @@ struct BandArgs {
   int64_t out_stride;
   Scoring sc;
   int32_t *status;            // SW_ETIMEOUT on an expired wait
-  int32_t short_int;          // 1 (16-bit batches): int32 units with the one-operation F chain;
-                              // 0 (int32 batches): Algorithm 1's statement order
   // buffer sizes, tested by the checked build (-DSW_CHECK) before every access
   int64_t ring_entries;       // entries of `rings`
   int64_t out_size;           // entries of `out`
@@ -213,7 +211,7 @@ struct TrackJob {
   int32_t nb;      // bands
   int32_t band0;   // global index of the job's band 0
   int32_t lane0;   // band b's lanes at TrackArgs::lanes[lane0 + 32 b ...]
-  int32_t pad_;
+  int32_t rows;    // rows per lane: the launch's, or track_long_rows() of it
   int64_t ring0;   // entry offset of ring 0 (between bands 0 and 1); rings are qt_npad[q] long
 };
 struct TrackArgs {
@@ -235,8 +233,9 @@ struct TrackArgs {
   // buffer sizes, tested by the checked build (-DSW_CHECK) before every access
   int64_t n_lanes, ring_entries, out_size, qt_bytes;
 };
-// R: rows per lane of the transposed jobs (8, 16 or 24: bands of 256, 512 or 768 database rows)
-bool track_supported_R(int R);
+// R: rows per lane of the transposed jobs (8, 12, 16, 20 or 24: bands of 256 to 768 database
+// rows).  Sequences longer than a band run in lanes of track_long_rows(R) rows.
+__host__ __device__ constexpr int track_long_rows(int R) { return R > 16 ? 16 : R; }
 int track_max_ctas_per_sm(int R, int gaps);  // plan time: raises the shared-memory limit; 0 on failure
 int track_threads();
 cudaError_t launch_track(const TrackArgs &a, int R, int grid, cudaStream_t s);

@@ -14,14 +14,12 @@
 // short enough (a few thousand columns) that many jobs run at once, and every
 // unit's cells are spread over all the job's warps instead of one.
 //
-// Forms: int32 cells, one database sequence per unit (Algorithm 1's
-// statements in int32 batches; in 16-bit batches, for the pairs that could
-// pass the 16-bit range, the one-operation F chain), or two sequences per
-// unit in the 16-bit halves of a word (only for pairs that cannot pass the
-// 16-bit range, so no rescue is needed).  A
-// lane's R rows form one chain down the column (no split lanes: the pipeline
-// lag between consecutive bands is then 31 columns instead of 63, which
-// measured faster here, where several bands share each SM sub-partition).
+// Forms: int32 cells, one database sequence per unit (in 16-bit batches for
+// the pairs that could pass the 16-bit range), or two sequences per unit in
+// the 16-bit halves of a word (only for pairs that cannot pass the 16-bit
+// range, so no rescue is needed).  One column per step (band_core.cuh): every
+// unit is a matrix of its own, and a band's last lane finishes it 32 columns
+// after its first; two columns per step would make that 64.
 //
 // Rings and progress.  Each ring holds one 64-bit entry per column of the
 // job's whole stream, zeroed before the launch, and is written once: the
@@ -38,30 +36,26 @@
 // caller-order output with atomicMax (the host zeroes the jobs' output rows
 // first); the maximum over the bands is the unit's score.
 #include <algorithm>
-#include "devutil.cuh"
-#include "dp_common.cuh"
-#include "internal.h"
-#include "../../include/swgb.h"
+#include "band_core.cuh"
 
 namespace swgb {
 namespace {
 
 // 12 warps, one band at a time each, one CTA per SM with up to 168
-// registers a thread (the 512-row bands' profiles take 134 KB of shared
-// memory).  Homolog workload, ms per search (packed / int32): 8 warps at 128
-// registers (one or two CTAs per SM) 2.14 / 3.43; 10 warps 2.15 / 3.71; 12
-// warps 1.95 / 3.31 (2.10 / 3.28 capped at 128 registers); 14 warps 2.33 /
-// 3.50; 16 warps 2.37 / 3.25.
+// registers a thread (the 512-row bands' profiles and residues take 157 KB of
+// shared memory).  Homolog search, ms (packed / int32): 8 warps 1.82 / 3.19;
+// 10 warps 1.91 / 2.88; 12 warps 1.68 / 2.52; 14 warps 1.82 / 2.52; 16 warps
+// 1.83 / 2.41.  (Before the steps of band_core.cuh: 1.89 / 2.71 at 12.)
 constexpr int kBandStreamThreads = 384;
-constexpr int kLag = 32 - 1;  // a band's last lane trails its first by 31 columns
 constexpr int kSubmatBytes = 512;
 // R rows per lane: bands of 32 R query rows; a band's profile is [21][32 lanes
-// x R] bytes, followed by its residue slots (2 x 32 B) and boundary slots (2 x
-// 16 x 8 B)
+// x R] bytes, followed by its residues (two sequences, two chunks) and
+// boundary slots (2 x 16 x 8 B)
 template <int R>
 constexpr int kProfBytes = kProfRows * 32 * R;
+constexpr int kBandIoBytes = 4 * kResChunk + 2 * kColBlock * 8;
 template <int R>
-constexpr int kWarpBytes = ((kProfBytes<R> + 320) + 127) / 128 * 128;
+constexpr int kWarpBytes = (kProfBytes<R> + kBandIoBytes + 127) / 128 * 128;
 
 // A band's profile in the warp's shared-memory block: byte [c][lane * R + r]
 // = SM(Q[row], c) for row = band * 32 R + lane * R + r, the pad value for the
@@ -90,154 +84,34 @@ __device__ __forceinline__ void build_band_profile(uint8_t *prof, const int8_t *
   }
 }
 
-// One band over one database unit (columns sbase .. sbase + npad - 1 of the
-// job's stream).  Returns false when a wait expired.
-template <int R, int FORM, bool SHORTF>
-__device__ __forceinline__ bool band_unit(const BandArgs &a, const uint8_t *__restrict__ prof, uint8_t *ring,
+// One band over one database unit (columns sbase .. of the job's stream, its
+// padded length); io: the warp's residues and boundary slots.  Returns false
+// when a wait expired.
+template <int R, int FORM>
+__device__ __forceinline__ bool band_unit(const BandArgs &a, const uint8_t *__restrict__ prof, uint8_t *io,
                                           const int lane, const int posA, const int posB, const int64_t sbase,
                                           const unsigned long long *ring_in, unsigned long long *ring_out,
                                           const Consts &cs, Word<FORM> &Sout) {
-  using W = Word<FORM>;
   constexpr bool PACKED = FORM == kFormPacked;
-  const W H0 = (W)0;
-  const W F0 = PACKED ? (W)cs.F0W : (W)0;
+  using Prof = std::conditional_t<PACKED, SeqPairProfile<R, 1>, IntProfile<R, 1>>;
   const int npa = a.db.npad[posA];
   const int npb = PACKED ? a.db.npad[posB] : 0;
   const int npad = max(npa, npb);
-  const uint8_t *resA = a.db.res + a.db.off[posA];
-  const uint8_t *resB = a.db.res + a.db.off[posB];
-  constexpr int LAG = kLag;
-  const int nblk = (npad + LAG + kColBlock - 1) / kColBlock;
-  const int nreal = npad / kColBlock;
-  const bool prev = ring_in != nullptr, next = ring_out != nullptr;
-  const bool lead = lane == 0;
-  const bool tail = lane == 31 && next;
-  const int src = lane > 0 ? lane - 1 : lane;
-
-  LaneState<R, FORM> st;
-  lane_reset(st, cs);
-  W outH = H0, outF = F0, S = (W)0;
-  uint32_t outRes = kPadPair;
-  uint8_t *rres = ring;                              // [slot][2 seqs][16 B] residue codes
-  uint2 *rgb = reinterpret_cast<uint2 *>(ring + 64);  // [slot][16] (H, F) of the band above
-  const uint8_t *prow = prof + lane * R;
-  bool failed = false;
-
-  auto prefetch = [&](int blk) {
-    uint8_t *d = rres + (blk & 1) * 32;
-    const int col = blk * kColBlock;
-    if (col < npa && in_range(resA + col + 15 - a.db.res, a.db.res_bytes, a.status)) cp_async16(d, resA + col);
-    else *reinterpret_cast<uint4 *>(d) = make_uint4(0x14141414u, 0x14141414u, 0x14141414u, 0x14141414u);
-    if (PACKED) {
-      if (col < npb && in_range(resB + col + 15 - a.db.res, a.db.res_bytes, a.status)) cp_async16(d + 16, resB + col);
-      else *reinterpret_cast<uint4 *>(d + 16) = make_uint4(0x14141414u, 0x14141414u, 0x14141414u, 0x14141414u);
-    }
-    cp_async_commit();
-  };
-  if (lead) {
-    prefetch(0);
-    prefetch(1);
-  }
-
-  // reading side: the next block to load (lanes 0..15 hold one entry each)
-  int64_t rpos = sbase;
-  unsigned long long pend = 0ull;
-  auto load = [&]() {
-    if (lane < kColBlock && in_range(ring_in - a.rings + rpos + lane, a.ring_entries, a.status))
-      pend = ld_relaxed_u64(ring_in + rpos + lane);
-  };
-  // wait until the loaded entries are written, unpack them into `slot`, advance
-  auto land = [&](int slot) {
-    bool ok = lane >= kColBlock || (pend >> 31 & 1ull);
-    long long t0 = 0;
-    bool waited = false;
-    while (!__all_sync(0xffffffffu, ok)) {
-      if (!waited) {
-        t0 = clock64();
-        waited = true;
-      }
-      if (__any_sync(0xffffffffu, clock64() - t0 > kWaitBudgetCycles)) {
-        failed = true;
-        if (lead) atomicExch(a.status, SW_ETIMEOUT);
-        return;
-      }
-      if (!ok) {
-        __nanosleep(32);  // (a waiting band leaves the issue slots to the bands that compute)
-        if (in_range(ring_in - a.rings + rpos + lane, a.ring_entries, a.status))
-          pend = ld_relaxed_u64(ring_in + rpos + lane);
-        ok = (pend >> 31 & 1ull) != 0ull;
-      }
-    }
-    if (lane < kColBlock)
-      rgb[slot * kColBlock + lane] = make_uint2((uint32_t)pend & 0x7fffffffu, (uint32_t)(pend >> 32));
-    rpos += kColBlock;
-    __syncwarp();
-  };
-  // both boundary slots start as the matrix top boundary (a band without a
-  // band above keeps it; the others overwrite them block by block)
-  if (lane < kColBlock) {
-    rgb[lane] = make_uint2((uint32_t)H0, (uint32_t)F0);
-    rgb[kColBlock + lane] = make_uint2((uint32_t)H0, (uint32_t)F0);
-  }
-  __syncwarp();
-  if (prev && nreal > 0) {
-    load();
-    land(0);
-    if (!failed && nreal > 1) load();
-  }
-
-  int64_t wpos = sbase;
-  for (int blk = 0; blk < nblk && !failed; ++blk) {
-    const uint2 *gslot = rgb + (blk & 1) * kColBlock;
-    const uint32_t *rw = reinterpret_cast<const uint32_t *>(rres + (blk & 1) * 32);
-    if (lead) cp_async_wait<1>();
-#pragma unroll 1
-    for (int g4 = 0; g4 < kColBlock / 4; ++g4) {
-      const uint32_t wa = rw[g4], wb = PACKED ? rw[4 + g4] : 0u;  // (used by lane 0 only)
-#pragma unroll
-      for (int s4 = 0; s4 < 4; ++s4) {
-        const int s = g4 * 4 + s4;
-        const int t = blk * kColBlock + s;
-        W inH = (W)__shfl_sync(0xffffffffu, outH, src);
-        W inF = (W)__shfl_sync(0xffffffffu, outF, src);
-        uint32_t inRes = __shfl_sync(0xffffffffu, outRes, src);
-        if (lead) {
-          // (the residue ring holds the pad code past the unit's end, the
-          // boundary slot the top boundary where no band lies above)
-          inRes = PACKED ? prmt(wa, wb, sel_pair(s4)) : prmt(wa, 0u, sel_one(s4));
-          const uint2 v = gslot[s];
-          inH = (W)v.x;
-          inF = (W)v.y;
-        }
-        if constexpr (kChecked) inRes = checked_codes<FORM>(inRes, a.status);
-        column_step<R, FORM, SHORTF>(st, prow, 32 * R, inRes, inH, inF, cs, S, outH, outF, 0);
-        outRes = inRes;
-        if (tail) {
-          const int j = t - LAG;
-          if (j >= 0 && j < npad && in_range(ring_out - a.rings + wpos, a.ring_entries, a.status)) {
-            const uint32_t lo = (uint32_t)outH | 0x80000000u;
-            st_relaxed_u64(ring_out + wpos, ((unsigned long long)(uint32_t)outF << 32) | lo);
-            ++wpos;
-          }
-        }
-      }
-    }
-    if (lead) {
-      if (blk + 2 < nblk) prefetch(blk + 2);
-      else cp_async_commit();
-    }
-    if (prev && blk + 1 < nreal) {
-      land((blk + 1) & 1);
-      if (!failed && blk + 2 < nreal) load();
-    } else if (prev && blk + 1 < nblk) {
-      // the padding blocks after the last real one: top boundary again
-      if (lane < kColBlock) rgb[((blk + 1) & 1) * kColBlock + lane] = make_uint2((uint32_t)H0, (uint32_t)F0);
-      __syncwarp();
-    }
-  }
-  if (lead) cp_async_wait<0>();
-  Sout = S;
-  return !failed;
+  ResidueStage<PACKED ? 2 : 1> rs{io,   a.db.res + a.db.off[posA], a.db.res + a.db.off[posB], npa, npb, lane,
+                                  a.db.res, a.db.res_bytes, a.status};
+  uint2 *rgb = reinterpret_cast<uint2 *>(io + 4 * kResChunk);
+  __syncwarp();  // (the unit before this one has read its residues and slots)
+  rs.stage(0);
+  clear_slots(rgb, lane, PACKED ? cs.F0W : 0u);
+  OnceRing x{ring_in ? ring_in + sbase : nullptr, ring_out ? ring_out + sbase : nullptr, rgb, lane, a.rings,
+             a.ring_entries, a.status, ring_in != nullptr, ring_out != nullptr};
+  BandLane<R, FORM, 1> ln;
+  ln.reset(cs);
+  const bool ok = band_sweep<R, FORM, 1, false, Prof>(ln, rs, x, rgb, prof + lane * R, 32 * R, lane,
+                                                      npad / kColBlock, (Word<FORM>)-1, (Word<FORM>)0, cs, a.status);
+  cp_async_wait<0>();
+  Sout = ln.S;
+  return ok;
 }
 
 template <int R, int GAPS>
@@ -247,7 +121,7 @@ __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(cons
   int8_t *sm = reinterpret_cast<int8_t *>(smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint8_t *prof = smem + kSubmatBytes + (size_t)warp * kWarpBytes<R>;
-  uint8_t *ring = prof + kProfBytes<R>;
+  uint8_t *io = prof + kProfBytes<R>;
   for (int i = threadIdx.x; i < kAlphabet * kAlphabet; i += blockDim.x) sm[i] = a.submat[i];
   __syncthreads();
   const Consts cs = make_consts<GAPS>(a.sc);
@@ -276,9 +150,7 @@ __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(cons
       if (!in_range(p.x, a.db.n, a.status) || !in_range(p.y, a.db.n, a.status)) p = make_int2(0, 0);
       if (job.form == kBandPacked) {
         uint32_t S = 0u;
-        // the one-operation F chain in 16-row lanes (3 % faster on the homolog
-        // workload; with 8 rows 2 % slower)
-        ok = band_unit<R, kFormPacked, (R >= 16)>(a, prof, ring, lane, p.x, p.y, sbase, ring_in, ring_out, cs, S);
+        ok = band_unit<R, kFormPacked>(a, prof, io, lane, p.x, p.y, sbase, ring_in, ring_out, cs, S);
         for (int d = 16; d > 0; d >>= 1) S = __vmaxs2(S, __shfl_xor_sync(0xffffffffu, S, d));
         if (ok && lane == 0) {
           if (in_range(job.q * a.out_stride + a.db.perm[p.x], a.out_size, a.status))
@@ -289,13 +161,8 @@ __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(cons
         sbase += max(a.db.npad[p.x], a.db.npad[p.y]);
       } else {
         int32_t S = 0;
-        // (the int32 units of a 16-bit batch: the one-operation F chain too)
-        if (half && a.short_int)
-          ok = band_unit<RH, kFormInt32, true>(a, prof, ring, lane, p.x, p.x, sbase, ring_in, ring_out, cs, S);
-        else if (half) ok = band_unit<RH, kFormInt32, false>(a, prof, ring, lane, p.x, p.x, sbase, ring_in, ring_out, cs, S);
-        else if (a.short_int)
-          ok = band_unit<R, kFormInt32, true>(a, prof, ring, lane, p.x, p.x, sbase, ring_in, ring_out, cs, S);
-        else ok = band_unit<R, kFormInt32, false>(a, prof, ring, lane, p.x, p.x, sbase, ring_in, ring_out, cs, S);
+        if (half) ok = band_unit<RH, kFormInt32>(a, prof, io, lane, p.x, p.x, sbase, ring_in, ring_out, cs, S);
+        else ok = band_unit<R, kFormInt32>(a, prof, io, lane, p.x, p.x, sbase, ring_in, ring_out, cs, S);
         for (int d = 16; d > 0; d >>= 1) S = max(S, __shfl_xor_sync(0xffffffffu, S, d));
         if (ok && lane == 0 && in_range(job.q * a.out_stride + a.db.perm[p.x], a.out_size, a.status))
           atomicMax(&orow[a.db.perm[p.x]], S);
@@ -324,193 +191,106 @@ __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(cons
 // of 8 warps put two on each sub-partition of half the SMs while the others
 // idle
 constexpr int kTrackThreads = 128;
+constexpr int kTrackCols = 2;  // columns per step (band_core.cuh)
+// Score table of the database residues: row k holds SM(c, k) for the query
+// residues c = 0..20 (pad), one byte each, rows 28 bytes apart (seven words:
+// the 21 codes of a word's lookups fall in different banks)
+constexpr int kScoreRow = 28;
+constexpr int kScoreBytes = 640;
 template <int R>
 constexpr int kTrackStride = 32 * R;                                // bytes per residue row of one table
 template <int R>
 constexpr int kTrackProfBytes = 2 * kProfRows * kTrackStride<R>;    // two tables of [21][32 lanes x R] bytes
+constexpr int kTrackIoBytes = 2 * kResChunk + 2 * kColBlock * 8;    // residues, boundary slots
 template <int R>
-constexpr int kTrackWarpBytes = ((kTrackProfBytes<R> + 320) + 127) / 128 * 128;
+constexpr int kTrackWarpBytes = (kTrackProfBytes<R> + kTrackIoBytes + 127) / 128 * 128;
+
+// N words to byte p (as aligned as load_prof reads them).
+template <int N>
+__device__ __forceinline__ void store_words(uint8_t *p, const uint32_t (&w)[N]) {
+  if constexpr (N % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i)
+      reinterpret_cast<uint4 *>(p)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+  } else if constexpr (N % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) reinterpret_cast<uint2 *>(p)[i] = make_uint2(w[2 * i], w[2 * i + 1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) reinterpret_cast<uint32_t *>(p)[i] = w[i];
+  }
+}
 
 // Profile of a band's rows: the substitution score of query residue c
 // (column) against each database row, SM(c, D[row]) (the query residue is
 // the matrix's row index): table t, byte (c, lane, r) at (21 t + c) * stride
 // + lane * R + r, for the low (t = 0) and high (t = 1) track.  Rows past a
 // sequence's end, idle lanes and the pad residue (c = 20) hold the pad value.
+// Four rows' scores against four query residues are four words of the score
+// table, transposed by byte shuffles: the whole profile takes a byte lookup's
+// instructions per four bytes (R = 24: 10.4 -> 2 us of a small search).
 template <int R, bool TWO>
-__device__ __forceinline__ void build_track_profile(uint8_t *prof, const int8_t *sm, const DbView &db,
-                                                    const TrackLane &L, int lane, int32_t pad, int32_t *status) {
-#pragma unroll
+__device__ __forceinline__ void build_track_profile(uint8_t *prof, const uint8_t *score, const DbView &db,
+                                                    const TrackLane &L, int lane, int32_t *status) {
+#pragma unroll 1
   for (int t = 0; t < (TWO ? 2 : 1); ++t) {
     const int32_t pos = t ? L.pb : L.pa, r0 = t ? L.rb : L.ra;
     const bool ok = pos >= 0 && in_range(pos, db.n, status);
-    const int32_t len = ok ? db.len[pos] : 0;
+    const int32_t npad = ok ? db.npad[pos] : 0;
     const uint8_t *res = db.res + (ok ? db.off[pos] : 0);
-    uint8_t code[R];
+    uint32_t code[R / 4];  // (a sequence's padding up to npad, a multiple of 16, holds the pad code)
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int32_t row = r0 + r;
-      code[r] = (ok && row < len && in_range(res + row - db.res, db.res_bytes, status)) ? res[row] : (uint8_t)kPadCode;
+    for (int i = 0; i < R / 4; ++i) {
+      const int32_t row = r0 + 4 * i;
+      code[i] = (row < npad && in_range(res + row + 3 - db.res, db.res_bytes, status))
+                    ? *reinterpret_cast<const uint32_t *>(res + row) : 0x14141414u;
     }
-    for (int c = 0; c < kProfRows; ++c) {
+    uint8_t *p = prof + t * kProfRows * kTrackStride<R> + lane * R;
+#pragma unroll 1
+    for (int w = 0; w < (kProfRows + 3) / 4; ++w) {
+      uint32_t out[4][R / 4];
 #pragma unroll
       for (int i = 0; i < R / 4; ++i) {
-        uint32_t v = 0;
+        uint32_t v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int r = 4 * i + j;
-          const int32_t x = (c < kAlphabet && code[r] < kAlphabet) ? (int32_t)sm[c * kAlphabet + code[r]] : pad;
-          v |= ((uint32_t)x & 0xffu) << (8 * j);
-        }
-        *reinterpret_cast<uint32_t *>(prof + (t * kProfRows + c) * kTrackStride<R> + lane * R + 4 * i) = v;
+        for (int j = 0; j < 4; ++j)
+          v[j] = *reinterpret_cast<const uint32_t *>(score + prmt(code[i], 0u, sel_one(j)) * kScoreRow + 4 * w);
+        const uint32_t a = prmt(v[0], v[1], 0x5140u), b = prmt(v[2], v[3], 0x5140u);
+        const uint32_t c = prmt(v[0], v[1], 0x7362u), d = prmt(v[2], v[3], 0x7362u);
+        out[0][i] = prmt(a, b, 0x5410u);
+        out[1][i] = prmt(a, b, 0x7632u);
+        out[2][i] = prmt(c, d, 0x5410u);
+        out[3][i] = prmt(c, d, 0x7632u);
       }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (4 * w + j < kProfRows) store_words(p + (4 * w + j) * kTrackStride<R>, out[j]);
     }
   }
 }
 
 // One band of a row track over all columns of its query.  keepH / addF: the
 // lane's restart masks (a half whose rows start a sequence takes the matrix
-// top boundary (0, F0) instead of the row above).  Returns false when a wait
-// expired.
+// top boundary (0, F0) instead of the row above).  io: the warp's residues
+// and boundary slots, the first chunk of residues staged.  Returns false when
+// a wait expired.
 template <int R, int FORM>
-__device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__restrict__ prof, uint8_t *ring,
-                                           const int lane, const uint8_t *resQ, const int npad,
+__device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__restrict__ prof, ResidueStage<1> &rs,
+                                           uint2 *rgb, const int lane, const int npad,
                                            const unsigned long long *ring_in, unsigned long long *ring_out,
                                            const Word<FORM> keepH, const Word<FORM> addF, const Consts &cs,
                                            Word<FORM> &Sout) {
-  using W = Word<FORM>;
   constexpr bool PACKED = FORM != kFormInt32;
-  const W H0 = (W)0;
-  const W F0 = PACKED ? (W)cs.F0W : (W)0;
-  const int nblk = (npad + kLag + kColBlock - 1) / kColBlock;
-  const int nreal = npad / kColBlock;
-  const bool prev = ring_in != nullptr, next = ring_out != nullptr;
-  const bool lead = lane == 0;
-  const bool tail = lane == 31 && next;
-  const int src = lane > 0 ? lane - 1 : lane;
-  const uint8_t *prow = prof + lane * R;
-  // the column's residue code(s): one table, or the pair (c, c + 21) of the two tables
-  constexpr uint32_t kPadRes = PACKED ? (kPadCode | ((kPadCode + kProfRows) << 16)) : kPadCode;
-
-  LaneState<R, FORM> st;
-  lane_reset(st, cs);
-  W outH = H0, outF = F0, S = (W)0;
-  uint32_t outRes = kPadRes;
-  uint8_t *rres = ring;                              // [slot][16 B] query residue codes
-  uint2 *rgb = reinterpret_cast<uint2 *>(ring + 64);  // [slot][16] (H, F) of the band above
-  bool failed = false;
-
-  auto prefetch = [&](int blk) {
-    uint8_t *d = rres + (blk & 1) * 32;
-    const int col = blk * kColBlock;
-    if (col < npad && in_range(resQ + col + 15 - a.qt, a.qt_bytes, a.status)) cp_async16(d, resQ + col);
-    else *reinterpret_cast<uint4 *>(d) = make_uint4(0x14141414u, 0x14141414u, 0x14141414u, 0x14141414u);
-    cp_async_commit();
-  };
-  if (lead) {
-    prefetch(0);
-    prefetch(1);
-  }
-
-  int64_t rpos = 0;
-  unsigned long long pend = 0ull;
-  auto load = [&]() {
-    if (lane < kColBlock && in_range(ring_in - a.rings + rpos + lane, a.ring_entries, a.status))
-      pend = ld_relaxed_u64(ring_in + rpos + lane);
-  };
-  auto land = [&](int slot) {
-    bool ok = lane >= kColBlock || (pend >> 31 & 1ull);
-    long long t0 = 0;
-    bool waited = false;
-    while (!__all_sync(0xffffffffu, ok)) {
-      if (!waited) {
-        t0 = clock64();
-        waited = true;
-      }
-      if (__any_sync(0xffffffffu, clock64() - t0 > kWaitBudgetCycles)) {
-        failed = true;
-        if (lead) atomicExch(a.status, SW_ETIMEOUT);
-        return;
-      }
-      if (!ok) {
-        __nanosleep(32);
-        if (in_range(ring_in - a.rings + rpos + lane, a.ring_entries, a.status))
-          pend = ld_relaxed_u64(ring_in + rpos + lane);
-        ok = (pend >> 31 & 1ull) != 0ull;
-      }
-    }
-    if (lane < kColBlock)
-      rgb[slot * kColBlock + lane] = make_uint2((uint32_t)pend & 0x7fffffffu, (uint32_t)(pend >> 32));
-    rpos += kColBlock;
-    __syncwarp();
-  };
-  if (lane < kColBlock) {
-    rgb[lane] = make_uint2((uint32_t)H0, (uint32_t)F0);
-    rgb[kColBlock + lane] = make_uint2((uint32_t)H0, (uint32_t)F0);
-  }
-  __syncwarp();
-  if (prev && nreal > 0) {
-    load();
-    land(0);
-    if (!failed && nreal > 1) load();
-  }
-
-  for (int blk = 0; blk < nblk && !failed; ++blk) {
-    const uint2 *gslot = rgb + (blk & 1) * kColBlock;
-    const uint32_t *rw = reinterpret_cast<const uint32_t *>(rres + (blk & 1) * 32);
-    if (lead) cp_async_wait<1>();
-#pragma unroll 1
-    for (int g4 = 0; g4 < kColBlock / 4; ++g4) {
-      const uint32_t wa = rw[g4];  // (used by lane 0 only)
-#pragma unroll
-      for (int s4 = 0; s4 < 4; ++s4) {
-        const int s = g4 * 4 + s4;
-        const int t = blk * kColBlock + s;
-        W inH = (W)__shfl_sync(0xffffffffu, outH, src);
-        W inF = (W)__shfl_sync(0xffffffffu, outF, src);
-        uint32_t inRes = __shfl_sync(0xffffffffu, outRes, src);
-        if (lead) {
-          const uint32_t c = prmt(wa, 0u, sel_one(s4));
-          inRes = PACKED ? (c | ((c + kProfRows) << 16)) : c;
-          const uint2 v = gslot[s];
-          inH = (W)v.x;
-          inF = (W)v.y;
-        }
-        // a half whose rows start a sequence: the top boundary
-        inH = (W)((uint32_t)inH & (uint32_t)keepH);
-        inF = (W)(((uint32_t)inF & (uint32_t)keepH) | (uint32_t)addF);
-        if constexpr (kChecked) {
-          if ((inRes & 0xffffu) > (uint32_t)kPadCode ||
-              (PACKED && (inRes >> 16) - (uint32_t)kProfRows > (uint32_t)kPadCode) || (!PACKED && (inRes >> 16))) {
-            atomicExch(a.status, kStatusBounds);
-            inRes = kPadRes;
-          }
-        }
-        column_step<R, FORM, PACKED>(st, prow, kTrackStride<R>, inRes, inH, inF, cs, S, outH, outF, 0);
-        outRes = inRes;
-        if (tail) {
-          const int j = t - kLag;
-          if (j >= 0 && j < npad && in_range(ring_out - a.rings + j, a.ring_entries, a.status)) {
-            const uint32_t lo = (uint32_t)outH | 0x80000000u;
-            st_relaxed_u64(ring_out + j, ((unsigned long long)(uint32_t)outF << 32) | lo);
-          }
-        }
-      }
-    }
-    if (lead) {
-      if (blk + 2 < nblk) prefetch(blk + 2);
-      else cp_async_commit();
-    }
-    if (prev && blk + 1 < nreal) {
-      land((blk + 1) & 1);
-      if (!failed && blk + 2 < nreal) load();
-    } else if (prev && blk + 1 < nblk) {
-      if (lane < kColBlock) rgb[((blk + 1) & 1) * kColBlock + lane] = make_uint2((uint32_t)H0, (uint32_t)F0);
-      __syncwarp();
-    }
-  }
-  if (lead) cp_async_wait<0>();
-  Sout = S;
-  return !failed;
+  using Prof = std::conditional_t<PACKED, TablePairProfile<R, kTrackCols>, IntProfile<R, kTrackCols>>;
+  clear_slots(rgb, lane, PACKED ? cs.F0W : 0u);
+  OnceRing x{ring_in, ring_out, rgb, lane, a.rings, a.ring_entries, a.status, ring_in != nullptr, ring_out != nullptr};
+  BandLane<R, FORM, kTrackCols> ln;
+  ln.reset(cs);
+  const bool ok = band_sweep<R, FORM, kTrackCols, true, Prof>(ln, rs, x, rgb, prof + lane * R, kTrackStride<R>, lane,
+                                                              npad / kColBlock, keepH, addF, cs, a.status);
+  cp_async_wait<0>();
+  Sout = ln.S;
+  return ok;
 }
 
 // The best score of each sequence among a band's lanes (its rows are
@@ -531,14 +311,45 @@ __device__ __forceinline__ void track_scores(const TrackArgs &a, int32_t q, int3
   }
 }
 
+// One band: its rows' profile, the sweep, and the scores of its sequences.
+template <int R>
+__device__ __forceinline__ bool track_band(const TrackArgs &a, uint8_t *prof, const uint8_t *score,
+                                           ResidueStage<1> &rs, uint2 *rgb, const int32_t q, const bool packed,
+                                           const TrackLane &L, const int lane, const int npad,
+                                           const unsigned long long *ring_in, unsigned long long *ring_out,
+                                           const Consts &cs) {
+  const bool ra0 = L.pa < 0 || L.ra == 0, rb0 = L.pb < 0 || L.rb == 0;  // halves that restart
+  bool ok;
+  if (packed) {
+    build_track_profile<R, true>(prof, score, a.db, L, lane, a.status);
+    __syncwarp();
+    const uint32_t mask = (ra0 ? 0x0000ffffu : 0u) | (rb0 ? 0xffff0000u : 0u);
+    uint32_t S = 0u;
+    ok = track_pass<R, kFormPacked>(a, prof, rs, rgb, lane, npad, ring_in, ring_out, ~mask, cs.F0W & mask, cs, S);
+    track_scores(a, q, L.pa, (int32_t)(S & 0xffffu), lane);
+    track_scores(a, q, L.pb, (int32_t)(S >> 16), lane);
+  } else {
+    build_track_profile<R, false>(prof, score, a.db, L, lane, a.status);
+    __syncwarp();
+    int32_t S = 0;
+    ok = track_pass<R, kFormInt32>(a, prof, rs, rgb, lane, npad, ring_in, ring_out, ra0 ? 0 : -1, 0, cs, S);
+    track_scores(a, q, L.pa, S, lane);
+  }
+  return ok;
+}
+
 template <int R, int GAPS>
-__global__ void __launch_bounds__(kTrackThreads, R == 8 ? 4 : R == 16 ? 2 : 1) band_track_kernel(const TrackArgs a) {
+__global__ void __launch_bounds__(kTrackThreads, R <= 8 ? 4 : R <= 20 ? 2 : 1) band_track_kernel(const TrackArgs a) {
+  constexpr int RL = track_long_rows(R);  // sequences longer than a band
   extern __shared__ __align__(128) uint8_t smem[];
-  int8_t *sm = reinterpret_cast<int8_t *>(smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint8_t *prof = smem + kSubmatBytes + (size_t)warp * kTrackWarpBytes<R>;
-  uint8_t *ring = prof + kTrackProfBytes<R>;
-  for (int i = threadIdx.x; i < kAlphabet * kAlphabet; i += blockDim.x) sm[i] = a.submat[i];
+  uint8_t *prof = smem + kScoreBytes + (size_t)warp * kTrackWarpBytes<R>;
+  uint8_t *io = prof + kTrackProfBytes<R>;
+  uint2 *rgb = reinterpret_cast<uint2 *>(io + 2 * kResChunk);
+  for (int i = threadIdx.x; i < kProfRows * kScoreRow; i += blockDim.x) {
+    const int k = i / kScoreRow, c = i - k * kScoreRow;
+    smem[i] = (uint8_t)(k < kAlphabet && c < kAlphabet ? a.submat[c * kAlphabet + k] : a.sc.pad);
+  }
   __syncthreads();
   const Consts cs = make_consts<GAPS>(a.sc);
   const TrackLane idle{-1, 0, -1, 0};
@@ -568,27 +379,16 @@ __global__ void __launch_bounds__(kTrackThreads, R == 8 ? 4 : R == 16 ? 2 : 1) b
     const bool next = __shfl_sync(0xffffffffu, nxt, 0) != 0;
     const int32_t npad = a.qt_npad[job.q];
     const uint8_t *resQ = a.qt + a.qt_off[job.q];
+    __syncwarp();  // (the band before this one has read its profile, residues and slots)
+    ResidueStage<1> rs{io, resQ, nullptr, npad, 0, lane, a.qt, a.qt_bytes, a.status};
+    rs.stage(0);
     const unsigned long long *ring_in = prev ? a.rings + job.ring0 + (int64_t)(b - 1) * npad : nullptr;
     unsigned long long *ring_out = next ? a.rings + job.ring0 + (int64_t)b * npad : nullptr;
-    const bool ra0 = L.pa < 0 || L.ra == 0, rb0 = L.pb < 0 || L.rb == 0;  // halves that restart
-    __syncwarp();
     bool ok;
-    if (packed) {
-      build_track_profile<R, true>(prof, sm, a.db, L, lane, a.sc.pad, a.status);
-      __syncwarp();
-      const uint32_t mask = (ra0 ? 0x0000ffffu : 0u) | (rb0 ? 0xffff0000u : 0u);
-      uint32_t S = 0u;
-      ok = track_pass<R, kFormPacked>(a, prof, ring, lane, resQ, npad, ring_in, ring_out, ~mask, cs.F0W & mask,
-                                          cs, S);
-      track_scores(a, job.q, L.pa, (int32_t)(S & 0xffffu), lane);
-      track_scores(a, job.q, L.pb, (int32_t)(S >> 16), lane);
-    } else {
-      build_track_profile<R, false>(prof, sm, a.db, L, lane, a.sc.pad, a.status);
-      __syncwarp();
-      int32_t S = 0;
-      ok = track_pass<R, kFormInt32>(a, prof, ring, lane, resQ, npad, ring_in, ring_out, ra0 ? 0 : -1, 0, cs, S);
-      track_scores(a, job.q, L.pa, S, lane);
-    }
+    if (R == RL || job.rows == R)
+      ok = track_band<R>(a, prof, smem, rs, rgb, job.q, packed, L, lane, npad, ring_in, ring_out, cs);
+    else
+      ok = track_band<RL>(a, prof, smem, rs, rgb, job.q, packed, L, lane, npad, ring_in, ring_out, cs);
     __syncwarp();
     if (!ok) break;
   }
@@ -622,11 +422,16 @@ BandKernel band_kernel(int R, int gaps) {
   return nullptr;
 }
 using TrackKernel = void (*)(const TrackArgs);
+template <int R>
+TrackKernel track_kernel_of(int gaps) {
+  return gaps == kGapsProtein ? band_track_kernel<R, kGapsProtein> : band_track_kernel<R, kGapsAny>;
+}
+#define SWGB_TRACK_R_LIST(X) X(8) X(12) X(16) X(20) X(24)
 TrackKernel track_kernel(int R, int gaps) {
-  const bool p = gaps == kGapsProtein;
-  if (R == 8) return p ? band_track_kernel<8, kGapsProtein> : band_track_kernel<8, kGapsAny>;
-  if (R == 16) return p ? band_track_kernel<16, kGapsProtein> : band_track_kernel<16, kGapsAny>;
-  if (R == 24) return p ? band_track_kernel<24, kGapsProtein> : band_track_kernel<24, kGapsAny>;
+#define SWGB_CASE(RR) \
+  if (R == RR) return track_kernel_of<RR>(gaps);
+  SWGB_TRACK_R_LIST(SWGB_CASE)
+#undef SWGB_CASE
   return nullptr;
 }
 
@@ -641,15 +446,18 @@ int occupancy_of(Kernel kern, int threads, size_t smem, size_t limit) {
   return n;
 }
 
-template <int R>
-size_t track_smem() { return kSubmatBytes + (size_t)(kTrackThreads / 32) * kTrackWarpBytes<R>; }
-size_t track_smem_of(int R) { return R == 8 ? track_smem<8>() : R == 16 ? track_smem<16>() : track_smem<24>(); }
+size_t track_smem_of(int R) {
+  size_t warp_bytes = 0;
+#define SWGB_CASE(RR) \
+  if (R == RR) warp_bytes = kTrackWarpBytes<RR>;
+  SWGB_TRACK_R_LIST(SWGB_CASE)
+#undef SWGB_CASE
+  return kScoreBytes + (kTrackThreads / 32) * warp_bytes;
+}
 
 }  // namespace
 
 int track_threads() { return kTrackThreads; }
-
-bool track_supported_R(int R) { return R == 8 || R == 16 || R == 24; }
 
 int track_max_ctas_per_sm(int R, int gaps) {
   const TrackKernel kern = track_kernel(R, gaps);
