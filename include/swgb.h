@@ -108,21 +108,22 @@ typedef struct sw_options {
                               residues use the intra-task (multi-warp) kernel; 0 = 2048;
                               a value above every length sends everything inter-task */
   int32_t rows_per_lane;   /* query rows per lane of the inter-task kernel: 4, 8, 12, 16 or 24;
-                              0 = 24, or 8 for batches too small to fill the GPU */
+                              0 = 8, 16 or 24, the one with the least modelled time */
   int32_t lanes_per_chain; /* lanes per chain of the inter-task kernel, 4..32; 0 = chosen per query */
   int32_t intra_rows;      /* query rows per lane of the intra-task kernel: 8 or 16; 0 = 16 */
   int32_t query_pairs;     /* packed mode, inter-task kernel: 0 = pair queries of similar length
                               into the two 16-bit halves where no lane can overflow (one
                               database sequence per chain), 1 = never pair (two database
                               sequences per chain for every query) */
-  int32_t band_stream;     /* batches too small to fill the GPU (0 = auto) run in the band-stream
-                              kernel instead of the inter- and intra-task kernels: a query of at
-                              least two bands (see band_rows) against every database unit, its
-                              rows cut into bands, one warp each, the bands of a query running
-                              as a pipeline over a stream of units; every shorter query
-                              transposed, the database sequences stacked as rows in bands of
-                              256 to 768 rows and the query's residues as the columns; 1 = never;
-                              2 = for every batch, however large */
+  int32_t band_stream;     /* 0 = auto: batches against up to 16,384 sequences run in the small-batch
+                              kernels instead of the inter- and intra-task kernels where their
+                              modelled time is less: a query of at least two bands (see
+                              band_rows) against every database unit, its rows cut into bands,
+                              one warp each, the bands of a query running as a pipeline over a
+                              stream of units; every shorter query (or all of them, where that
+                              takes less) transposed, the database sequences stacked as rows in
+                              bands of 256 to 768 rows and the query's residues as the columns;
+                              1 = never; 2 = for every batch, however large */
   int32_t band_rows;       /* query rows per lane of the band-stream kernel: 8 or 16 (bands of
                               256 or 512 rows); 0 = 16 */
   int32_t reserved[1];     /* must be 0 */

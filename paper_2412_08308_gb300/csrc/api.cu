@@ -59,21 +59,33 @@ inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 // Rows per lane of the transposed jobs (heights whose kernels exist), and the
 // cycles of one step (two columns) of a band that has its SM sub-partition to
 // itself, or per band where two or more share it: from timings of 500 to
-// 20,000 proteins at every height.  (More than 16 rows share a launch with the
-// 16-row lanes of longer sequences, whose code they evict.)
+// 20,000 proteins at every height.
 struct TrackHeight {
   int rows;
   double packed1, packed2, int1, int2;
 };
-constexpr TrackHeight kTrackHeights[] = {{8, 302, 211, 229, 161},
-                                         {12, 382, 318, 291, 221},
-                                         {16, 461, 397, 353, 287},
-                                         {20, 540, 486, 415, 373},
-                                         {24, 620, 620, 477, 498}};
+constexpr TrackHeight kTrackHeights[] = {{8, 290, 245, 229, 183},
+                                         {12, 351, 356, 290, 264},
+                                         {16, 460, 445, 353, 324},
+                                         {20, 585, 538, 511, 395},
+                                         {24, 685, 680, 560, 509}};
 double track_step_cycles(bool packed, int rows, int w) {
   for (const TrackHeight &h : kTrackHeights)
     if (h.rows == rows) return w <= 1 ? (packed ? h.packed1 : h.int1) : w * (packed ? h.packed2 : h.int2);
   return 1e9;
+}
+
+// Cycles of one step of an inter-task warp with w warps on its SM
+// sub-partition: its share of the sub-partition's rate (row, step), or, with
+// few warps, its own latency (row1, step1).  From 1,850 timings of one query
+// of 60 to 6,000 residues x 500 to 160,000 proteins at 8, 16 and 24 rows and 4
+// to 32 lanes: the lanes and rows that the model picks measure within 5 % of
+// the best ones in 9 of 10 cases.
+double chain_step_cycles(int form, int R, int w) {
+  const bool i32 = form == kFormInt32;
+  const double row = i32 ? 8.0 : form == kFormPacked ? 10.2 : 8.5, step = i32 ? 26 : 22;
+  const double row1 = i32 ? 14.0 : 12.5, step1 = i32 ? 171 : 110;
+  return std::max(step1 + row1 * R, w * (row * R + step));
 }
 
 int sm_count(int dev) {
@@ -465,11 +477,11 @@ namespace {
 // steps per column (fill[L], below) x idle lanes, with a small charge per
 // chunk for the boundary strip and the CTA barrier.  (Against the measured
 // time of the 20-query benchmark with L forced to 4..32, this model is
-// proportional to within 1.5 %.)
-int choose_lanes(int m, int R, const double *fill, int Lmax = 32) {
-  int bestL = 4;
+// proportional to within 1.5 %.)  At least Lmin lanes.
+int choose_lanes(int m, int R, const double *fill, int Lmin = 4) {
+  int bestL = Lmin;
   double best = 1e300;
-  for (int L = 4; L <= Lmax; ++L) {
+  for (int L = Lmin; L <= 32; ++L) {
     const int LR = L * R;
     const int C = std::max(1, (m + LR - 1) / LR);
     const double rows = (double)C * LR;
@@ -753,66 +765,305 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   // fill[L]: steps a chain of L lanes spends per real column of a short unit.
   // A pass over a unit of n padded columns takes n + lag steps (lag = L - 1,
   // or 2 L - 1 for the split lanes of the 16-bit forms) rounded up to whole
-  // 16-column blocks.  fill for the solo plans of this mode; fillq (below)
-  // for the query-pair plans.
+  // 16-column blocks.
   // (padded lengths are multiples of 16 and every long unit is longer than
   // every short one, so the short units' counts are the first bins)
   std::vector<int64_t> len_hist(max_short / kColBlock + 1, 0);
   if (n_long < Q->n_units)
     std::copy(ust.hist.begin(), ust.hist.begin() + std::min(len_hist.size(), ust.hist.size()), len_hist.begin());
-  auto make_fill = [&](int form, double *out) {
-    for (int L = 0; L <= 32; ++L) {
-      const int lag = L > 0 ? inter_chain_lag(R, form, L) : 0;
-      double steps = 0;
-      for (size_t b = 1; b < len_hist.size(); ++b)
-        steps += (double)len_hist[b] * (double)((b * kColBlock + lag + kColBlock - 1) / kColBlock * kColBlock);
-      out[L] = sum_short > 0 ? steps / sum_short : 1.0;
-    }
+  // (the lag does not depend on the rows beyond whether they split)
+  double fills[2][33];
+  bool have_fill[2] = {false, false};
+  auto fill_of = [&](int form, int rows) -> const double * {
+    const int k = inter_chain_lag(rows, form, 4) > 3;
+    double *out = fills[k];
+    if (!have_fill[k])
+      for (int L = 0; L <= 32; ++L) {
+        const int lag = L > 0 ? inter_chain_lag(rows, form, L) : 0;
+        double steps = 0;
+        for (size_t b = 1; b < len_hist.size(); ++b)
+          steps += (double)len_hist[b] * (double)((b * kColBlock + lag + kColBlock - 1) / kColBlock * kColBlock);
+        out[L] = sum_short > 0 ? steps / sum_short : 1.0;
+      }
+    have_fill[k] = true;
+    return out;
   };
-  double fill[33];
-  make_fill(packed ? kFormPacked : kFormInt32, fill);
-
-  // --- rows per lane and CTA size of the inter-task kernel.  A small batch
-  // (few units x queries) cannot fill the GPU with 16-row lanes: halve the
-  // rows per lane (twice the lanes, half the per-step dependency chain), and
-  // shrink CTAs until the tasks cover every SM twice.
   const int64_t n_short = Q->n_units - n_long;
-  auto lanes_needed = [&](int rr) {
-    double lanes = 0;
-    for (int64_t q = 0; q < n_queries; ++q) {
-      const int m = std::max<int>(1, (int)(q_offsets[q + 1] - q_offsets[q]));
-      lanes += (double)n_short * (forceL ? forceL : choose_lanes(m, rr, fill));
-    }
-    return lanes;
-  };
-  // A small batch is latency-bound: each chain's sweep over its longest
-  // sequence is the critical path, multiplied by the number of chunks.  Use
-  // the fewest chunks the lanes allow (one chunk of up to 32 lanes) rather
-  // than the fewest idle lanes.
-  const bool latency_bound = lanes_needed(16) < (double)sms * 2048;
-  if (!o.rows_per_lane && latency_bound) R = 8;
-  Q->R = R;
-  auto pick_lanes = [&](int m, int Lmax) {
-    if (forceL) return std::min(forceL, Lmax);
-    if (latency_bound) return std::min(Lmax, std::max(4, (m + R - 1) / R));
-    return choose_lanes(m, R, fill, Lmax);
-  };
-  int warps = inter_threads() / 32;
-  for (; warps > 2; warps /= 2) {
-    int64_t tasks = 0;
-    for (int64_t q = 0; q < n_queries; ++q) {
-      const int m = std::max<int>(1, (int)(q_offsets[q + 1] - q_offsets[q]));
-      const int chains = warps * (32 / pick_lanes(m, 32));
-      tasks += (n_short + chains - 1) / chains;
-    }
-    if (tasks >= 2 * sms) break;
-  }
-  const int threads = warps * 32;
-  Q->threads = threads;
   auto qlen = [&](int64_t q) { return (int32_t)(q_offsets[q + 1] - q_offsets[q]); };
   auto may_flag = [&](int64_t q, int32_t n_upper) {
     return packed && (int64_t)sc.maxp * std::min<int64_t>(qlen(q), n_upper) > sc.thresh;
   };
+
+  // --- the inter-task kernel's plan: rows per lane, lanes per chain, CTA size,
+  // and (packed mode) query tracks.
+  // Query tracks: two queries share one chain, one per
+  // 16-bit half: the database residue of a column is common to both, so one
+  // 32-bit profile word per row feeds both halves and the residue-pair byte
+  // shuffle of the two-sequence form disappears.  Each half runs a track of
+  // queries laid end to end chunk by chunk, so queries of different lengths
+  // share chains without idle rows (greedy longest-first packing into
+  // balanced tracks).  Only queries that cannot pass the 16-bit threshold
+  // against the short database units join tracks (the form has no rescue
+  // pass); the others keep the two-sequence form.
+  const int64_t s0 = packed ? std::min<int64_t>(n, 2 * n_long) : n_long;  // first short sequence
+  Q->n_single = n - s0;
+  std::vector<int32_t> elig;
+  if (packed && o.query_pairs == 0 && n_queries >= 2 && Q->n_single > 0) {
+    for (int64_t q = 0; q < n_queries; ++q)
+      if (!may_flag(q, max_short)) elig.push_back((int32_t)q);
+    if (elig.size() < 2) elig.clear();
+    std::stable_sort(elig.begin(), elig.end(), [&](int32_t x, int32_t y) { return qlen(x) > qlen(y); });
+  }
+  struct InterPlan {
+    int R = 24, warps = 8;
+    std::vector<int> L;                        // lanes per chain of each query's own plan
+    std::vector<char> in_track;                // query runs in a track plan
+    std::vector<std::vector<int32_t>> tracks;  // two per track plan
+    std::vector<int> plan_L;
+    double time = 0;       // modelled cycles
+    bool even = false;     // many tasks per CTA: no task sets the time
+  };
+  struct Part {
+    int C, L;  // chunks and lanes per chain of a query's (a track plan's) chains
+  };
+  // Modelled cycles of one launch of `parts` over nu units, longest first:
+  // the average work of a CTA, and what list scheduling cannot split -- the
+  // longest task, and j + 1 tasks on some CTA as long as there are more than j
+  // per CTA.  *even: the average is many times the longest task.
+  auto launch_time = [&](int form, int rows, int W, const std::vector<Part> &parts, int64_t nu, double sum_len,
+                         int32_t max_len, const std::vector<int64_t> &at_least, const double *fl, bool *even) {
+    const double slots = (double)sms * 16 / W;
+    double tasks = 0, work = 0, longest = 0;
+    for (const Part &p : parts) {
+      const int chains = W * (32 / p.L);
+      tasks += (double)((nu + chains - 1) / chains);
+      work += (double)p.C * std::max(fl[p.L] * sum_len / chains, (double)max_len);
+      longest = std::max(longest, (double)p.C * (double)round_up(max_len + inter_chain_lag(rows, form, p.L), kColBlock));
+    }
+    if (tasks <= 0) return 0.0;
+    const int w = (int)std::max(1.0, std::min(4.0, std::ceil(tasks * W / (4.0 * sms))));
+    const double cyc = chain_step_cycles(form, rows, w);
+    if (tasks <= slots) {
+      *even = false;
+      return longest * cyc;
+    }
+    double bound = std::max(work / slots, longest);
+    if (work / slots < 8 * longest) {
+      *even = false;
+      // x: the largest length with more than j * slots tasks at least that long
+      for (int j = 1; j <= 3 && tasks > j * slots; ++j) {
+        double lo = 0, hi = longest;
+        for (int it = 0; it < 10; ++it) {
+          const double x = 0.5 * (lo + hi);
+          double cnt = 0;
+          for (const Part &p : parts) {
+            const double len = x / p.C - inter_chain_lag(rows, form, p.L);
+            const size_t bin = len <= 0 ? 0 : (size_t)std::ceil(len / kColBlock);
+            cnt += bin < at_least.size() ? std::ceil((double)at_least[bin] / (W * (32 / p.L))) : 0.0;
+          }
+          (cnt > j * slots ? lo : hi) = x;
+        }
+        bound = std::max(bound, (j + 1) * lo);
+      }
+    }
+    return bound * cyc;
+  };
+  // counts of short units (of this mode; single sequences) at least 16 b long
+  auto suffix_counts = [&](const std::vector<int64_t> &hist, size_t bins) {
+    std::vector<int64_t> c(std::min(hist.size(), bins), 0);
+    int64_t acc = 0;
+    for (size_t b = c.size(); b-- > 0;) c[b] = acc += hist[b];
+    return c;
+  };
+  const std::vector<int64_t> units_ge = suffix_counts(ust.hist, len_hist.size());
+  std::vector<int64_t> singles_ge;
+  double sum_single = 0;
+  if (!elig.empty()) {
+    const sw_db::UnitStats &single = db->units(false);
+    singles_ge = suffix_counts(single.hist, len_hist.size());
+    sum_single = (double)(single.prefix[(size_t)n] - single.prefix[(size_t)s0]);
+  }
+  // The plan at `rows` rows per lane with at least Lfloor lanes per chain
+  // (where the query has that many): more lanes mean fewer chunks, so shorter
+  // tasks, at the price of idle lanes and longer pipeline fill.
+  auto make_plan = [&](int rows, int Lfloor) {
+    InterPlan P;
+    P.R = rows;
+    const double *fl = fill_of(packed ? kFormPacked : kFormInt32, rows), *flq = fill_of(kFormQPair, rows);
+    auto floor_of = [&](int m) { return std::min({32, Lfloor, std::max(4, (m + rows - 1) / rows)}); };
+    auto chunks_of = [&](int32_t q, int L) { return std::max(1, (qlen(q) + L * rows - 1) / (L * rows)); };
+    P.L.resize((size_t)n_queries);
+    for (int64_t q = 0; q < n_queries; ++q) {
+      const int m = std::max(1, qlen(q));
+      P.L[q] = forceL ? forceL
+               : q > 0 && qlen(q) == qlen(q - 1) ? P.L[q - 1]  // (batches of one length: chosen once)
+                                                 : choose_lanes(m, rows, fl, floor_of(m));
+    }
+    P.in_track.assign((size_t)n_queries, 0);
+    if (!elig.empty()) {
+      // Two ways to lay the eligible queries out, priced with the same model as
+      // choose_lanes (padded rows x steps per column / lane use, the two halves of
+      // a plan running max(track) chunks), the cheaper one kept:
+      //  - grouped tracks: the queries sorted by length and cut into K consecutive
+      //    groups, each packed longest first into two balanced tracks.  K grows
+      //    with the query count (at least 8 queries per plan keep the tracks
+      //    balanced) and so that every resident CTA sees several tiles;
+      //  - pairs: neighbours in length order whose shorter one has at least 3/4
+      //    of the longer one's rows share a plan (one query per track); the
+      //    others keep the two-sequence form (two database sequences per chain;
+      //    pairing their scores costs a byte shuffle per word, priced as 6/5 of
+      //    the query-pair form's time per cell).
+      // Each plan has its own lanes per chain.  (Many queries of similar length
+      // favour pairs: each pair's L fits its length; few queries of spread-out
+      // lengths favour tracks: no idle half.)
+      // best L for a group packed into two tracks, and its modelled cost
+      int last_a = -1, last_b = -1, last_L = 4;
+      double last_cost = 0;
+      auto plan_group = [&](const int32_t *g0, const int32_t *g1, std::vector<int32_t> *tr, int *Lout) {
+        auto pack = [&](int L, std::vector<int32_t> *out) {
+          int64_t load[2] = {0, 0};
+          for (const int32_t *q = g0; q < g1; ++q) {
+            const int t = load[1] < load[0] ? 1 : 0;
+            if (out) out[t].push_back(*q);
+            load[t] += chunks_of(*q, L);
+          }
+          return std::max(load[0], load[1]);
+        };
+        auto cost_of = [&](int L) {
+          const double eff = (double)((32 / L) * L) / 32.0, chunks = (double)pack(L, nullptr);
+          return chunks * L * rows * flq[L] / eff * (1.0 + 0.002 * chunks / std::max<double>(1.0, (double)(g1 - g0)));
+        };
+        int Lp = forceL ? forceL : 4;
+        // (neighbouring pairs of the same two lengths: chosen once)
+        const bool again = g1 - g0 == 2 && last_a == qlen(g0[0]) && last_b == qlen(g0[1]);
+        if (again) {
+          pack(last_L, tr);
+          *Lout = last_L;
+          return last_cost;
+        }
+        if (!forceL) {
+          double best = 1e300;
+          for (int L = floor_of(qlen(*g0)); L <= 32; ++L) {
+            const double c = cost_of(L);
+            if (c < best - 1e-9) {
+              best = c;
+              Lp = L;
+            }
+          }
+        }
+        pack(Lp, tr);
+        *Lout = Lp;
+        const double cost = cost_of(Lp);
+        if (g1 - g0 == 2) {
+          last_a = qlen(g0[0]);
+          last_b = qlen(g0[1]);
+          last_L = Lp;
+          last_cost = cost;
+        }
+        return cost;
+      };
+      auto solo_cost = [&](int32_t q) {  // two-sequence form: half the columns, 6/5 the time per word
+        const int L = P.L[q];
+        const double C = chunks_of(q, L), eff = (double)((32 / L) * L) / 32.0;
+        return C * L * rows * fl[L] / eff * (1.0 + 0.001 * C) * 0.6;
+      };
+      const int64_t ne = (int64_t)elig.size();
+      // grouped tracks
+      std::vector<std::vector<int32_t>> tA, tB;
+      std::vector<int> LA, LB;
+      double costA = 0, costB = 0;
+      const int64_t tiles8 = std::max<int64_t>(1, (Q->n_single + 31) / 32);
+      int64_t K = std::max<int64_t>((8 * 2 * (int64_t)sms + tiles8 - 1) / tiles8, std::min<int64_t>(8, ne / 8));
+      K = std::max<int64_t>(1, std::min<int64_t>(K, ne / 2));
+      auto add = [&](int64_t i0, int64_t i1, std::vector<std::vector<int32_t>> &t, std::vector<int> &Ls) {
+        std::vector<int32_t> tr[2];
+        int Lp = 4;
+        const double c = plan_group(elig.data() + i0, elig.data() + i1, tr, &Lp);
+        t.push_back(std::move(tr[0]));
+        t.push_back(std::move(tr[1]));
+        Ls.push_back(Lp);
+        return c;
+      };
+      for (int64_t k = 0; k < K; ++k) costA += add(ne * k / K, ne * (k + 1) / K, tA, LA);
+      // pairs
+      std::vector<int32_t> soloB;
+      for (int64_t i = 0; i < ne; ++i) {
+        if (i + 1 < ne && 4 * (int64_t)qlen(elig[i + 1]) >= 3 * (int64_t)qlen(elig[i])) {
+          costB += add(i, i + 2, tB, LB);
+          ++i;
+        } else {
+          soloB.push_back(elig[i]);
+          costB += solo_cost(elig[i]);
+        }
+      }
+      for (int32_t q : elig) P.in_track[q] = 1;
+      if (costB < costA) {
+        P.tracks = std::move(tB);
+        P.plan_L = std::move(LB);
+        for (int32_t q : soloB) P.in_track[q] = 0;
+      } else {
+        P.tracks = std::move(tA);
+        P.plan_L = std::move(LA);
+      }
+    }
+    std::vector<Part> solo, pairs;
+    for (int64_t q = 0; q < n_queries; ++q)
+      if (!P.in_track[q]) solo.push_back({chunks_of((int32_t)q, P.L[q]), P.L[q]});
+    for (size_t k = 0; k < P.plan_L.size(); ++k) {
+      int64_t load[2] = {0, 0};
+      for (int h = 0; h < 2; ++h)
+        for (int32_t q : P.tracks[2 * k + h]) load[h] += chunks_of(q, P.plan_L[k]);
+      pairs.push_back({(int)std::max<int64_t>({1, load[0], load[1]}), P.plan_L[k]});
+    }
+    // CTAs shrink until the tasks cover every SM twice
+    for (P.warps = inter_threads() / 32; P.warps > 2; P.warps /= 2) {
+      int64_t tasks = 0;
+      for (const Part &p : solo) tasks += (n_short + P.warps * (32 / p.L) - 1) / (P.warps * (32 / p.L));
+      for (const Part &p : pairs) tasks += (Q->n_single + P.warps * (32 / p.L) - 1) / (P.warps * (32 / p.L));
+      if (tasks >= 2 * sms) break;
+    }
+    P.even = true;
+    P.time = launch_time(packed ? kFormPacked : kFormInt32, rows, P.warps, solo, n_short, sum_short, max_short,
+                         units_ge, fl, &P.even);
+    if (!pairs.empty())
+      P.time += launch_time(kFormQPair, rows, P.warps, pairs, Q->n_single, sum_single, max_short, singles_ge, flq,
+                            &P.even);
+    return P;
+  };
+  // The plan with the least modelled time over the rows per lane and the
+  // fewest lanes.  (Measured, GCUPS: one 1,301-residue query x 80,000 proteins
+  // 24 rows x 8 lanes 5,783, x 4 5,050; 20 queries x 40,000 proteins 8 lanes
+  // 6,745, 4 lanes 5,908; one 60-residue query x 80,000 16 rows x 4 lanes
+  // 4,759, 24 rows x 4 2,982.)
+  auto best_plan = [&]() {
+    static const int kRows[] = {24, 16, 8};
+    static const int kFloors[] = {5, 6, 8, 10, 12, 16, 20, 24, 32};
+    InterPlan best;
+    bool first = true;
+    auto consider = [&](int rows, int Lfloor) {
+      InterPlan P = make_plan(rows, Lfloor);
+      const bool even = P.even;
+      if (first || P.time < best.time * (1 - 1e-9)) best = std::move(P);
+      first = false;
+      return even;
+    };
+    bool even = true;
+    for (int rows : kRows)
+      if (o.rows_per_lane ? rows == o.rows_per_lane : rows > 8 || n_queries <= 32) even &= consider(rows, 4);
+    if (first) even = consider(R, 4);  // (4 or 12 rows, by option)
+    if (even || forceL) return best;
+    if (n_queries > 32) {  // (many queries: each plan costs more, and the choice matters less)
+      const int rows = best.R;
+      for (int Lfloor : {8, 16, 32}) consider(rows, Lfloor);
+      return best;
+    }
+    for (int Lfloor : kFloors)
+      if (o.rows_per_lane) consider(o.rows_per_lane, Lfloor);
+      else
+        for (int rows : kRows) consider(rows, Lfloor);
+    return best;
+  };
+  InterPlan plan;
 
   // --- small batches: band-stream jobs and transposed jobs (k_band.cu).  In
   // a batch too small to fill the GPU, the longest chains of the inter-task
@@ -852,7 +1103,7 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   bool band_mode = false;
   // Bands of one query in lanes of tR rows, and the most bands of one
   // sequence, estimated from the length histogram.
-  auto track_estimate = [&](int tR, const sw_db::UnitStats &single, double *bands, int64_t *deepest) {
+  auto track_estimate = [&](int tR, const sw_db::UnitStats &single, int32_t cut, double *bands, int64_t *deepest) {
     const int tL = track_long_rows(tR);
     double lanes = 0;
     *bands = 0;
@@ -864,7 +1115,8 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
         lanes += (double)single.hist[h] * (double)((len + tR - 1) / tR);
       } else {
         const int64_t nb = (len + 32 * tL - 1) / (32 * tL);
-        *bands += (double)(single.hist[h] * nb);
+        // (two 16-bit tracks share a band; int32 ones, past the cut, do not)
+        *bands += (double)(single.hist[h] * nb) * (packed && len > cut ? 2 : 1);
         *deepest = std::max(*deepest, nb);
         // (short sequences fill most of what the last band leaves)
         lanes -= 0.8 * (double)single.hist[h] * (double)(32 * tL * nb - len) / tR;
@@ -891,37 +1143,116 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
     const double chain = (steps_max + 50.0 * (double)(deepest - 1)) * track_step_cycles(packed, track_long_rows(tR), w);
     return deepest > 1 ? std::max(all, chain) : all;
   };
-  if (o.band_stream != 1 && (o.band_stream == 2 || latency_bound) && n > 0 && n_queries > 0) {
+  // a sequence takes the 16-bit tracks (packed mode) unless its pair with the
+  // longest of these queries could pass the 16-bit range: a length cut that
+  // depends on the queries only through that longest one
+  auto track_cut = [&]() {
+    int32_t mtq = 0;
+    for (int64_t q = 0; q < n_queries; ++q)
+      if (track_q[q]) mtq = std::max(mtq, qlen(q));
+    return !packed ? -1
+           : (int64_t)sc.maxp * mtq <= sc.thresh ? std::numeric_limits<int32_t>::max()
+                                                 : sc.thresh / sc.maxp;
+  };
+  // rows per lane of the transposed jobs, in order of the modelled time
+  struct TrackChoice {
+    double time;
+    int tR, occ;
+  };
+  std::vector<TrackChoice> heights;
+  auto rank_heights = [&]() {
+    heights.clear();
+    const sw_db::UnitStats &single = db->units(false);
+    const int32_t cut = track_cut();
+    for (const TrackHeight &h : kTrackHeights) {
+      const int occ = cached_occupancy(2, h.rows, 0, gaps, 0, 0);
+      if (occ <= 0) continue;
+      double bands = 0;
+      int64_t deepest = 1;
+      track_estimate(h.rows, single, cut, &bands, &deepest);
+      heights.push_back({track_time(h.rows, occ, bands, deepest), h.rows, occ});
+    }
+    std::sort(heights.begin(), heights.end(),
+              [](const TrackChoice &x, const TrackChoice &y) { return x.time < y.time; });
+    return heights.empty() ? 1e300 : heights[0].time;
+  };
+  auto rank_heights_of = [&]() {
+    for (int64_t q = 0; q < n_queries; ++q)
+      if (track_q[q]) return rank_heights();
+    return 0.0;
+  };
+  // Modelled time (cycles) of the band-stream jobs of the queries in band_q:
+  // padded cells at the kernel's rate, or one stream's columns and the bands'
+  // hand-offs one after another (from timings of one query of 1,301 to 6,000
+  // residues x 500 to 40,000 proteins, within 20 %).
+  auto band_time = [&]() {
+    double thr = 0, lat = 0;
+    const int brows = 32 * bR;
+    const double widest = Q->n_units > 0 ? (double)unit_len(0) : 0.0;
+    for (int64_t q = 0; q < n_queries; ++q) {
+      if (!band_q[q]) continue;
+      const double nb = (double)((qlen(q) + brows - 1) / brows), rows = nb * brows;
+      const bool i32 = !packed || may_flag(q, (int32_t)widest);  // (some units in int32: their columns set the pace)
+      thr += rows * (double)db->total / (packed ? 2246 : 1329);
+      lat = std::max(lat, packed && !i32 ? 528 * widest + 24800 * nb : (packed ? 180 : 310) * widest + 27000 * nb);
+    }
+    return 0.95 * std::max(thr, lat) + 0.15 * std::min(thr, lat);
+  };
+  // Which kernels: the small-batch ones (band-stream jobs for the long queries
+  // and transposed ones for the others, or all transposed), or the inter- and
+  // intra-task ones, by modelled time.  Above 16,384 sequences the inter-task
+  // kernel measures equal or faster (20,000 proteins, packed: 60 residues 177
+  // against 205 us, 144 336 / 302, 400 655 / 604, 1,000 1,318 / 1,318, 1,301
+  // 1,938 / 2,207), and a new database need not lay its row tracks first.
+  bool small = o.band_stream == 2;
+  if (n > 0 && n_queries > 0 && o.band_stream != 1) {
+    bool any_band = false;
+    for (int64_t q = 0; q < n_queries; ++q) {
+      band_q[q] = qlen(q) >= 2 * 32 * bR;
+      track_q[q] = !band_q[q];
+      any_band |= band_q[q] != 0;
+    }
+    if (o.band_stream == 0 && n <= 16384) {
+      plan = best_plan();
+      double inter = plan.time;
+      if (n_long) {  // the intra-task kernel beside it: about 4.4 int32 cells per cycle and SM
+        double m_sum = 0, m_max = 0;
+        for (int64_t q = 0; q < n_queries; ++q) {
+          m_sum += qlen(q);
+          m_max = std::max<double>(m_max, qlen(q));
+        }
+        const double rate = packed && (int64_t)sc.maxp * max_long <= sc.thresh ? 9.6 : 4.4;
+        const double cols = (double)ust.prefix[(size_t)n_long] * (packed ? 2 : 1);
+        const double intra = std::max(m_max * max_long, m_sum * cols / sms) / rate;
+        inter = std::max(inter, intra) + 0.3 * std::min(inter, intra);
+      }
+      const double tracks_a = rank_heights_of(), bands_a = any_band ? band_time() : 0.0;
+      double best_small = std::max(tracks_a, bands_a) + 0.5 * std::min(tracks_a, bands_a);
+      if (any_band) {  // all transposed?
+        std::vector<char> bq = band_q, tq = track_q;
+        std::fill(band_q.begin(), band_q.end(), 0);
+        std::fill(track_q.begin(), track_q.end(), 1);
+        const double all = rank_heights_of();
+        if (all < best_small) {
+          best_small = all;
+        } else {
+          band_q.swap(bq);
+          track_q.swap(tq);
+        }
+      }
+      small = best_small < inter;
+    }
+  }
+  if (small) {
     const int brows = 32 * bR;
     bool any_band = false, any_track = false;
     for (int64_t q = 0; q < n_queries; ++q) {
-      band_q[q] = qlen(q) >= 2 * brows;
-      track_q[q] = !band_q[q];
       any_band |= band_q[q] != 0;
       any_track |= track_q[q] != 0;
     }
     const int bmax = any_band ? cached_occupancy(1, bR, 0, gaps, 0, 0) : 1;
     int bocc = bmax;
-    // rows per lane of the transposed jobs, in order of the modelled time
-    struct TrackChoice {
-      double time;
-      int tR, occ;
-    };
-    std::vector<TrackChoice> heights;
-    if (any_track) {
-      const sw_db::UnitStats &single = db->units(false);
-      for (const TrackHeight &h : kTrackHeights) {
-        const int tR = h.rows;
-        const int occ = cached_occupancy(2, tR, 0, gaps, 0, 0);
-        if (occ <= 0) continue;
-        double bands = 0;
-        int64_t deepest = 1;
-        track_estimate(tR, single, &bands, &deepest);
-        heights.push_back({track_time(tR, occ, bands, deepest), tR, occ});
-      }
-      std::sort(heights.begin(), heights.end(),
-                [](const TrackChoice &x, const TrackChoice &y) { return x.time < y.time; });
-    }
+    if (any_track) rank_heights();
     int tocc = !any_track ? 1 : heights.empty() ? 0 : heights[0].occ;
     int64_t ring = 0, band = 0, tring = 0, tband = 0, n_tlanes = 0;
     if (bocc > 0 && tocc > 0) {
@@ -1029,24 +1360,17 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
       }
 
       // transposed jobs: the database in row tracks, each short query as columns
-      int32_t mtq = 0;
       int64_t qt = 0;
       int64_t n_track_q = 0;
       for (int64_t q = 0; q < n_queries; ++q) {
         if (!track_q[q]) continue;
         ++n_track_q;
-        mtq = std::max(mtq, qlen(q));
         qt_npad[q] = (int32_t)std::max<int64_t>(kColBlock, round_up(qlen(q), kColBlock));
         qt_off[q] = qt;
         qt += qt_npad[q];
       }
       Q->qt_bytes = std::max<int64_t>(qt, 16);
-      // a sequence takes the 16-bit tracks (packed mode) unless its pair with
-      // the longest of these queries could pass the 16-bit range: a length
-      // cut that depends on the queries only through that longest one
-      const int32_t cut = !packed ? -1
-                          : (int64_t)sc.maxp * mtq <= sc.thresh ? std::numeric_limits<int32_t>::max()
-                                                                : sc.thresh / sc.maxp;
+      const int32_t cut = track_cut();
       // the jobs: each pipeline once per query (deeper pipelines first)
       auto make_jobs = [&](const std::vector<TrackPipe> &pipes) {
         tjobs.clear();
@@ -1125,8 +1449,6 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
       }
     }
     if (!band_mode) {
-      std::fill(band_q.begin(), band_q.end(), 0);
-      std::fill(track_q.begin(), track_q.end(), 0);
       bjobs.clear();
       bjob_of.clear();
       btpos.clear();
@@ -1136,142 +1458,23 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
       Q->d_tlanes = nullptr;
     }
   }
+  if (!band_mode) {
+    std::fill(band_q.begin(), band_q.end(), 0);
+    std::fill(track_q.begin(), track_q.end(), 0);
+  }
 
-  // --- query tracks (packed mode).  Two queries share one chain, one per
-  // 16-bit half: the database residue of a column is common to both, so one
-  // 32-bit profile word per row feeds both halves and the residue-pair byte
-  // shuffle of the two-sequence form disappears.  Each half runs a track of
-  // queries laid end to end chunk by chunk, so queries of different lengths
-  // share chains without idle rows (greedy longest-first packing into
-  // balanced tracks).  Only queries that cannot pass the 16-bit threshold
-  // against the short database units join tracks (the form has no rescue
-  // pass); the others keep the two-sequence form.
-  const int64_t s0 = packed ? std::min<int64_t>(n, 2 * n_long) : n_long;  // first short sequence
-  Q->n_single = n - s0;
-  std::vector<int32_t> in_track(n_queries, 0), elig;
-  if (packed && o.query_pairs == 0 && n_queries >= 2 && Q->n_single > 0) {
-    for (int64_t q = 0; q < n_queries; ++q)
-      if (!may_flag(q, max_short) && !small_q[q]) elig.push_back((int32_t)q);
-    if (elig.size() < 2) elig.clear();
-  }
-  for (int32_t q : elig) in_track[q] = 1;
-  // Two ways to lay the eligible queries out, priced with the same model as
-  // choose_lanes (padded rows x steps per column / lane use, the two halves of
-  // a plan running max(track) chunks), the cheaper one kept:
-  //  - grouped tracks: the queries sorted by length and cut into K consecutive
-  //    groups, each packed longest first into two balanced tracks.  K grows
-  //    with the query count (at least 8 queries per plan keep the tracks
-  //    balanced) and so that every resident CTA sees several tiles;
-  //  - pairs: neighbours in length order whose shorter one has at least 3/4
-  //    of the longer one's rows share a plan (one query per track); the
-  //    others keep the two-sequence form (two database sequences per chain;
-  //    pairing their scores costs a seventh instruction per word, priced as
-  //    7/6 of the query-pair form's time per cell).
-  // Each plan has its own lanes per chain.  (Many queries of similar length
-  // favour pairs: each pair's L fits its length; few queries of spread-out
-  // lengths favour tracks: no idle half.)
-  auto chunks_of = [&](int32_t q, int L) { return std::max(1, (qlen(q) + L * R - 1) / (L * R)); };
-  double fillq[33];
-  make_fill(kFormQPair, fillq);
-  // best L for a group packed into two tracks, and its modelled cost
-  auto plan_group = [&](const std::vector<int32_t> &grp, std::vector<int32_t> *tr, int *Lout) {
-    auto pack = [&](int L, std::vector<int32_t> *out) {
-      int64_t load[2] = {0, 0};
-      for (int32_t q : grp) {
-        const int t = load[1] < load[0] ? 1 : 0;
-        if (out) out[t].push_back(q);
-        load[t] += chunks_of(q, L);
-      }
-      return std::max(load[0], load[1]);
-    };
-    auto cost_of = [&](int L) {
-      const double eff = (double)((32 / L) * L) / 32.0;
-      return (double)pack(L, nullptr) * L * R * fillq[L] / eff * (1.0 + 0.001 * (double)pack(L, nullptr) /
-                                                                          std::max<size_t>(1, grp.size()) * 2);
-    };
-    int Lp = 4;
-    if (forceL) {
-      Lp = forceL;
-    } else if (latency_bound) {
-      int mmax = 1;
-      for (int32_t q : grp) mmax = std::max(mmax, qlen(q));
-      Lp = std::min(32, std::max(4, (mmax + R - 1) / R));
-    } else {
-      double best = 1e300;
-      for (int L = 4; L <= 32; ++L) {
-        const double c = cost_of(L);
-        if (c < best - 1e-9) {
-          best = c;
-          Lp = L;
-        }
-      }
-    }
-    if (tr) pack(Lp, tr);
-    if (Lout) *Lout = Lp;
-    return cost_of(Lp);
-  };
-  auto solo_cost = [&](int32_t q) {  // two-sequence form: half the columns, 7/6 the instructions per word
-    double best = 1e300;
-    for (int L = 4; L <= 32; ++L) {
-      const int C = chunks_of(q, L);
-      const double eff = (double)((32 / L) * L) / 32.0;
-      best = std::min(best, (double)C * L * R * fill[L] / eff * (1.0 + 0.001 * C));
-    }
-    return best * 7.0 / 12.0;
-  };
-  std::vector<std::vector<int32_t>> tracks;  // 2 per plan
-  std::vector<int> plan_L;
-  if (!elig.empty()) {
-    std::vector<int32_t> ord = elig;
-    std::stable_sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) { return qlen(x) > qlen(y); });
-    const int64_t ne = (int64_t)ord.size();
-    // grouped tracks
-    std::vector<std::vector<int32_t>> tA;
-    std::vector<int> LA;
-    double costA = 0;
-    {
-      const int64_t tiles8 = std::max<int64_t>(1, (Q->n_single + warps * 4 - 1) / (warps * 4));
-      int64_t K = std::max<int64_t>((8 * 2 * (int64_t)sms + tiles8 - 1) / tiles8, std::min<int64_t>(8, ne / 8));
-      K = std::max<int64_t>(1, std::min<int64_t>(K, ne / 2));
-      for (int64_t p = 0; p < K; ++p) {
-        std::vector<int32_t> grp(ord.begin() + ne * p / K, ord.begin() + ne * (p + 1) / K);
-        std::vector<int32_t> tr[2];
-        int Lp = 4;
-        costA += plan_group(grp, tr, &Lp);
-        tA.push_back(tr[0]);
-        tA.push_back(tr[1]);
-        LA.push_back(Lp);
-      }
-    }
-    // pairs
-    std::vector<std::vector<int32_t>> tB;
-    std::vector<int> LB;
-    std::vector<int32_t> soloB;
-    double costB = 0;
-    for (int64_t i = 0; i < ne; ++i) {
-      const int32_t x = ord[i];
-      if (i + 1 < ne && 4 * (int64_t)qlen(ord[i + 1]) >= 3 * (int64_t)qlen(x)) {
-        std::vector<int32_t> grp{x, ord[i + 1]}, tr[2];
-        int Lp = 4;
-        costB += plan_group(grp, tr, &Lp);
-        tB.push_back(tr[0]);
-        tB.push_back(tr[1]);
-        LB.push_back(Lp);
-        ++i;
-      } else {
-        soloB.push_back(x);
-        costB += solo_cost(x);
-      }
-    }
-    if (costB < costA) {
-      tracks = tB;
-      plan_L = LB;
-      for (int32_t q : soloB) in_track[q] = 0;
-    } else {
-      tracks = tA;
-      plan_L = LA;
-    }
-  }
+  // --- the inter-task plan, unless the batch takes the small-batch kernels
+  if (band_mode) plan = InterPlan();
+  else if (plan.L.empty()) plan = best_plan();
+  R = plan.R;
+  Q->R = R;
+  const int warps = plan.warps, threads = warps * 32;
+  Q->threads = threads;
+  std::vector<char> &in_track = plan.in_track;
+  std::vector<std::vector<int32_t>> &tracks = plan.tracks;
+  std::vector<int> &plan_L = plan.plan_L;
+  in_track.resize((size_t)n_queries, 0);
+  plan.L.resize((size_t)n_queries, 32);
   Q->n_solo = 0;  // queries with a profile of their own (not in query-pair tracks, not band-stream jobs)
   for (int64_t q = 0; q < n_queries; ++q) Q->n_solo += (in_track[q] || small_q[q]) ? 0 : 1;
   Q->npairs = (int64_t)plan_L.size();  // track plans
@@ -1286,7 +1489,7 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
     QDesc &d = Q->qd[q];
     d.m = qlen(q);
     d.R = R;
-    d.L = pick_lanes(std::max(1, d.m), 32);
+    d.L = plan.L[q];
     const int LR = d.L * R;
     d.nchunks = std::max(1, (d.m + LR - 1) / LR);
     d.chunk_stride = (int32_t)round_up((int64_t)profile_slots(d.L) * R, 128);
@@ -1438,9 +1641,11 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   std::stable_sort(twi.begin(), twi.end(), [](const TW &a, const TW &b) { return a.w > b.w; });
   std::stable_sort(twi32.begin(), twi32.end(), [](const TW &a, const TW &b) { return a.w > b.w; });
   // track tiles plan by plan (each plan's profile stays hot in L2 while the
-  // CTAs stream it), longest tiles first within a plan
-  std::stable_sort(twp.begin(), twp.end(),
-                   [](const TW &a, const TW &b) { return a.t.q != b.t.q ? a.t.q < b.t.q : a.w > b.w; });
+  // CTAs stream it), longest tiles first within a plan; where single tasks set
+  // the time, longest first over all plans
+  std::stable_sort(twp.begin(), twp.end(), [&](const TW &a, const TW &b) {
+    return plan.even && a.t.q != b.t.q ? a.t.q < b.t.q : a.w > b.w;
+  });
   Q->n_ptasks = (int64_t)twp.size();
   Q->n_tasks = (int64_t)tw.size();
   Q->n_itasks = (int64_t)twi.size();

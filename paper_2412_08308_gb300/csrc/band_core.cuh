@@ -223,14 +223,6 @@ struct ResidueStage {
 template <int COLS>
 constexpr int kStoreLagBlocks = 32 * COLS / kColBlock;
 
-// Steps unrolled: what fits the instruction cache, beside the code of the
-// launch's other band heights.  (Pairs, two columns, 4 -> 8 steps: R = 8 269
-// -> 244 cycles per step, R = 20 478 -> 660; one 144-residue query x 2,000
-// proteins, 24-row words: 75 -> 96 us.  One column: homolog search 1,747 ->
-// 1,719 us packed, 2,570 -> 2,528 int32.)
-template <int R, int FORM, int COLS>
-constexpr int kUnrolled = COLS == 1 || R <= (FORM == kFormInt32 ? 16 : 12) ? 8 : 4;
-
 // Sweep a band over nreal blocks of columns.  rgb: the two slots of 16 (H, F)
 // entries of the band above, both holding the matrix top boundary (0, F0) on
 // entry.  Io passes the rows between bands:
@@ -241,15 +233,16 @@ constexpr int kUnrolled = COLS == 1 || R <= (FORM == kFormInt32 ? 16 : 12) ? 8 :
 //   out(wblk), lo_bias, hi_bias   where block wblk goes; what an entry's words
 //                   are on top of H and F
 //   done(wblk)      block wblk has been written
-// MASK: a lane whose rows start a sequence takes (in & keepH) and (in & keepH)
+// U: steps unrolled.  MASK: a lane whose rows start a sequence takes (in & keepH) and (in & keepH)
 // | addF in place of the row above.  Returns false when a wait expired.
-template <int R, int FORM, int COLS, bool MASK, class Prof, class Res, class Io>
+template <int R, int FORM, int COLS, int U, bool MASK, class Prof, class Res, class Io>
 __device__ __forceinline__ bool band_sweep(BandLane<R, FORM, COLS> &ln, Res &rs, Io &io, uint2 *rgb,
                                            const uint8_t *prow, const int stride, const int lane, const int nreal,
                                            const Word<FORM> keepH, const Word<FORM> addF, const Consts &cs,
                                            int32_t *status) {
   using W = Word<FORM>;
-  constexpr int kSteps = kColBlock / COLS, U = kUnrolled<R, FORM, COLS>;
+  constexpr int kSteps = kColBlock / COLS;
+  static_assert(kSteps % U == 0, "whole blocks");
   constexpr int kChunkBlocks = kResChunk / kColBlock;
   const uint32_t F0 = FORM != kFormInt32 ? cs.F0W : 0u;
   const int src = lane > 0 ? lane - 1 : lane;

@@ -47,6 +47,9 @@ namespace {
 // 10 warps 1.91 / 2.88; 12 warps 1.68 / 2.52; 14 warps 1.82 / 2.52; 16 warps
 // 1.83 / 2.41.  (Before the steps of band_core.cuh: 1.89 / 2.71 at 12.)
 constexpr int kBandStreamThreads = 384;
+// Steps unrolled (4 -> 8: homolog search 1,747 -> 1,719 us packed, 2,570 ->
+// 2,528 int32).
+constexpr int kBandUnroll = 8;
 constexpr int kSubmatBytes = 512;
 // R rows per lane: bands of 32 R query rows; a band's profile is [21][32 lanes
 // x R] bytes, followed by its residues (two sequences, two chunks) and
@@ -107,7 +110,7 @@ __device__ __forceinline__ bool band_unit(const BandArgs &a, const uint8_t *__re
              a.ring_entries, a.status, ring_in != nullptr, ring_out != nullptr};
   BandLane<R, FORM, 1> ln;
   ln.reset(cs);
-  const bool ok = band_sweep<R, FORM, 1, false, Prof>(ln, rs, x, rgb, prof + lane * R, 32 * R, lane,
+  const bool ok = band_sweep<R, FORM, 1, kBandUnroll, false, Prof>(ln, rs, x, rgb, prof + lane * R, 32 * R, lane,
                                                       npad / kColBlock, (Word<FORM>)-1, (Word<FORM>)0, cs, a.status);
   cp_async_wait<0>();
   Sout = ln.S;
@@ -274,7 +277,7 @@ __device__ __forceinline__ void build_track_profile(uint8_t *prof, const uint8_t
 // top boundary (0, F0) instead of the row above).  io: the warp's residues
 // and boundary slots, the first chunk of residues staged.  Returns false when
 // a wait expired.
-template <int R, int FORM>
+template <int R, int FORM, int U>
 __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__restrict__ prof, ResidueStage<1> &rs,
                                            uint2 *rgb, const int lane, const int npad,
                                            const unsigned long long *ring_in, unsigned long long *ring_out,
@@ -286,7 +289,7 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
   OnceRing x{ring_in, ring_out, rgb, lane, a.rings, a.ring_entries, a.status, ring_in != nullptr, ring_out != nullptr};
   BandLane<R, FORM, kTrackCols> ln;
   ln.reset(cs);
-  const bool ok = band_sweep<R, FORM, kTrackCols, true, Prof>(ln, rs, x, rgb, prof + lane * R, kTrackStride<R>, lane,
+  const bool ok = band_sweep<R, FORM, kTrackCols, U, true, Prof>(ln, rs, x, rgb, prof + lane * R, kTrackStride<R>, lane,
                                                               npad / kColBlock, keepH, addF, cs, a.status);
   cp_async_wait<0>();
   Sout = ln.S;
@@ -312,7 +315,7 @@ __device__ __forceinline__ void track_scores(const TrackArgs &a, int32_t q, int3
 }
 
 // One band: its rows' profile, the sweep, and the scores of its sequences.
-template <int R>
+template <int R, int UP, int UI>
 __device__ __forceinline__ bool track_band(const TrackArgs &a, uint8_t *prof, const uint8_t *score,
                                            ResidueStage<1> &rs, uint2 *rgb, const int32_t q, const bool packed,
                                            const TrackLane &L, const int lane, const int npad,
@@ -325,14 +328,14 @@ __device__ __forceinline__ bool track_band(const TrackArgs &a, uint8_t *prof, co
     __syncwarp();
     const uint32_t mask = (ra0 ? 0x0000ffffu : 0u) | (rb0 ? 0xffff0000u : 0u);
     uint32_t S = 0u;
-    ok = track_pass<R, kFormPacked>(a, prof, rs, rgb, lane, npad, ring_in, ring_out, ~mask, cs.F0W & mask, cs, S);
+    ok = track_pass<R, kFormPacked, UP>(a, prof, rs, rgb, lane, npad, ring_in, ring_out, ~mask, cs.F0W & mask, cs, S);
     track_scores(a, q, L.pa, (int32_t)(S & 0xffffu), lane);
     track_scores(a, q, L.pb, (int32_t)(S >> 16), lane);
   } else {
     build_track_profile<R, false>(prof, score, a.db, L, lane, a.status);
     __syncwarp();
     int32_t S = 0;
-    ok = track_pass<R, kFormInt32>(a, prof, rs, rgb, lane, npad, ring_in, ring_out, ra0 ? 0 : -1, 0, cs, S);
+    ok = track_pass<R, kFormInt32, UI>(a, prof, rs, rgb, lane, npad, ring_in, ring_out, ra0 ? 0 : -1, 0, cs, S);
     track_scores(a, q, L.pa, S, lane);
   }
   return ok;
@@ -341,6 +344,11 @@ __device__ __forceinline__ bool track_band(const TrackArgs &a, uint8_t *prof, co
 template <int R, int GAPS>
 __global__ void __launch_bounds__(kTrackThreads, R <= 8 ? 4 : R <= 20 ? 2 : 1) band_track_kernel(const TrackArgs a) {
   constexpr int RL = track_long_rows(R);  // sequences longer than a band
+  // steps unrolled (16-bit words, int32): what fits the instruction cache,
+  // together with the longer sequences' height where that is another one (one
+  // query x 2,000 proteins, 20-row words beside 16-row ones: 4 -> 2 steps 54.5
+  // -> 47.7 us at 144 residues, 210 -> 171 us at 1,000)
+  constexpr int UP = R == RL ? (R <= 12 ? 8 : 4) : 2, UI = R == RL ? 8 : 4;
   extern __shared__ __align__(128) uint8_t smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint8_t *prof = smem + kScoreBytes + (size_t)warp * kTrackWarpBytes<R>;
@@ -386,9 +394,9 @@ __global__ void __launch_bounds__(kTrackThreads, R <= 8 ? 4 : R <= 20 ? 2 : 1) b
     unsigned long long *ring_out = next ? a.rings + job.ring0 + (int64_t)b * npad : nullptr;
     bool ok;
     if (R == RL || job.rows == R)
-      ok = track_band<R>(a, prof, smem, rs, rgb, job.q, packed, L, lane, npad, ring_in, ring_out, cs);
+      ok = track_band<R, UP, UI>(a, prof, smem, rs, rgb, job.q, packed, L, lane, npad, ring_in, ring_out, cs);
     else
-      ok = track_band<RL>(a, prof, smem, rs, rgb, job.q, packed, L, lane, npad, ring_in, ring_out, cs);
+      ok = track_band<RL, UP, UI>(a, prof, smem, rs, rgb, job.q, packed, L, lane, npad, ring_in, ring_out, cs);
     __syncwarp();
     if (!ok) break;
   }
