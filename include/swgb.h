@@ -347,11 +347,13 @@ int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *target, int64_
  * the path that produced it is the alignment).  The paper's search reports
  * scores only; this recovers the alignments of the hits a caller keeps.
  *
- * One CTA per hit recomputes the pair's matrix in int32, its warps taking
- * the query's 512-row chunks as a pipeline, and records 4 bits per cell (where
- * H came from; whether E and F extend a gap); one thread per hit walks them
- * back from the first cell, in row-major order, that holds the score.  Device
- * memory: about m * n / 2 bytes per hit (held during the call).
+ * The hits' matrices are recomputed in int32, in bands of 256 query rows that
+ * one warp each sweeps as a pipeline, recording 4 bits per cell (whether H is
+ * the diagonal's or E's value; whether E and F extend a gap); one warp per hit
+ * walks them back from the first cell, in row-major order, that holds the
+ * score.  Device memory: m rounded up to 256, times n + 32 (to 48), / 2 bytes
+ * per hit, held during the call; hits that don't fit together are taken in
+ * halves.
  *
  *   db                    a prepared database
  *   queries, q_offsets, n_queries   host pointers, as sw_queries_prepare

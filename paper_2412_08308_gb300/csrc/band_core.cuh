@@ -1,5 +1,5 @@
 // The sweep shared by the pipelines of one-warp bands (long pairs, band-stream
-// jobs, transposed jobs): 32 lanes of R rows, an anti-diagonal wavefront down
+// jobs, transposed jobs, tracebacks): 32 lanes of R rows, an anti-diagonal wavefront down
 // the lanes, the bottom row handed to the band below through a ring of 64-bit
 // entries in global memory.
 //
@@ -30,6 +30,66 @@ __device__ __forceinline__ void load_rows(const uint8_t *p, uint32_t (&w)[kSlotB
   } else {
 #pragma unroll
     for (int i = 0; i < kSlotBytes<R> / 4; ++i) w[i] = reinterpret_cast<const uint32_t *>(p)[i];
+  }
+}
+
+// N words to byte p (as aligned as load_prof reads them).
+template <int N>
+__device__ __forceinline__ void store_words(uint8_t *p, const uint32_t (&w)[N]) {
+  if constexpr (N % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i)
+      reinterpret_cast<uint4 *>(p)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+  } else if constexpr (N % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) reinterpret_cast<uint2 *>(p)[i] = make_uint2(w[2 * i], w[2 * i + 1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) reinterpret_cast<uint32_t *>(p)[i] = w[i];
+  }
+}
+
+// Score table in shared memory: row k holds the scores of residue k (of the
+// bands' rows) against the columns' residues c = 0..20 (pad), one byte each;
+// rows are 28 bytes apart (seven words: the 21 rows' words of a lookup fall in
+// different banks).  TARGET_ROWS: the bands' rows are database residues and
+// the columns the query's (SM's row index), else the other way round.
+constexpr int kScoreRow = 28;
+constexpr int kScoreBytes = 640;
+template <bool TARGET_ROWS>
+__device__ __forceinline__ void build_scores(uint8_t *score, const int8_t *submat, int32_t pad) {
+  for (int i = threadIdx.x; i < kProfRows * kScoreRow; i += blockDim.x) {
+    const int k = i / kScoreRow, c = i - k * kScoreRow;
+    score[i] = (uint8_t)(k < kAlphabet && c < kAlphabet ? submat[TARGET_ROWS ? c * kAlphabet + k : k * kAlphabet + c]
+                                                        : pad);
+  }
+}
+
+// A lane's profile bytes from its rows' residue codes (four per word): row r
+// at residue c to p[c * stride + r].  Four rows against four residues are four
+// words of the score table, transposed by byte shuffles.
+template <int R>
+__device__ __forceinline__ void profile_from_scores(uint8_t *p, int stride, const uint8_t *score,
+                                                    const uint32_t (&code)[R / 4]) {
+#pragma unroll 1
+  for (int w = 0; w < (kProfRows + 3) / 4; ++w) {
+    uint32_t out[4][R / 4];
+#pragma unroll
+    for (int i = 0; i < R / 4; ++i) {
+      uint32_t v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[j] = *reinterpret_cast<const uint32_t *>(score + prmt(code[i], 0u, sel_one(j)) * kScoreRow + 4 * w);
+      const uint32_t a = prmt(v[0], v[1], 0x5140u), b = prmt(v[2], v[3], 0x5140u);
+      const uint32_t c = prmt(v[0], v[1], 0x7362u), d = prmt(v[2], v[3], 0x7362u);
+      out[0][i] = prmt(a, b, 0x5410u);
+      out[1][i] = prmt(a, b, 0x7632u);
+      out[2][i] = prmt(c, d, 0x5410u);
+      out[3][i] = prmt(c, d, 0x7632u);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (4 * w + j < kProfRows) store_words(p + (4 * w + j) * stride, out[j]);
   }
 }
 
@@ -223,7 +283,8 @@ struct ResidueStage {
 template <int COLS>
 constexpr int kStoreLagBlocks = 32 * COLS / kColBlock;
 
-// Sweep a band over nreal blocks of columns.  rgb: the two slots of 16 (H, F)
+// Sweep a band over nreal blocks of columns.  ln: the lane's rows (BandLane, or
+// a class with its step(), outH and outF).  rgb: the two slots of 16 (H, F)
 // entries of the band above, both holding the matrix top boundary (0, F0) on
 // entry.  Io passes the rows between bands:
 //   prev, next      a band above / below
@@ -235,8 +296,8 @@ constexpr int kStoreLagBlocks = 32 * COLS / kColBlock;
 //   done(wblk)      block wblk has been written
 // U: steps unrolled.  MASK: a lane whose rows start a sequence takes (in & keepH) and (in & keepH)
 // | addF in place of the row above.  Returns false when a wait expired.
-template <int R, int FORM, int COLS, int U, bool MASK, class Prof, class Res, class Io>
-__device__ __forceinline__ bool band_sweep(BandLane<R, FORM, COLS> &ln, Res &rs, Io &io, uint2 *rgb,
+template <int FORM, int COLS, int U, bool MASK, class Prof, class Lane, class Res, class Io>
+__device__ __forceinline__ bool band_sweep(Lane &ln, Res &rs, Io &io, uint2 *rgb,
                                            const uint8_t *prow, const int stride, const int lane, const int nreal,
                                            const Word<FORM> keepH, const Word<FORM> addF, const Consts &cs,
                                            int32_t *status) {
@@ -353,6 +414,8 @@ __device__ __forceinline__ void clear_slots(uint2 *rgb, int lane, uint32_t F0) {
 // zeroed before the launch, (H | 1 << 31, F).  H is below 2^31 (int32: bounded
 // by the host; 16-bit halves: both non-negative), so bit 31 tells a written
 // entry, and entries need no other flag or fence.
+// STRIDE: entries from one block of 16 columns to the next.
+template <int STRIDE = kColBlock>
 struct OnceRing {
   const unsigned long long *in;  // at the first column, or nullptr
   unsigned long long *own;       // at the first column, or nullptr
@@ -387,16 +450,16 @@ struct OnceRing {
     }
     if (lane < kColBlock)
       rgb[slot * kColBlock + lane] = make_uint2((uint32_t)pend & 0x7fffffffu, (uint32_t)(pend >> 32));
-    in += kColBlock;
+    in += STRIDE;
     pend = 0ull;
     __syncwarp();
     return true;
   }
   __device__ __forceinline__ bool room(int wblk) {
     // (every column has a place of its own; the checked build tests that)
-    return in_range(own - base + (int64_t)wblk * kColBlock + kColBlock - 1, entries, status);
+    return in_range(own - base + (int64_t)wblk * STRIDE + kColBlock - 1, entries, status);
   }
-  __device__ __forceinline__ unsigned long long *out(int wblk) const { return own + (int64_t)wblk * kColBlock; }
+  __device__ __forceinline__ unsigned long long *out(int wblk) const { return own + (int64_t)wblk * STRIDE; }
   __device__ __forceinline__ void done(int) {}
 };
 

@@ -220,7 +220,7 @@ struct TrackArgs {
   const TrackJob *jobs;
   const int32_t *band_job;    // [nbands] job of each global band
   int32_t nbands;
-  int32_t *band_counter;      // zeroed before the launch
+  int32_t *band_counter;      // (cleared by launch_trace, as is the status)
   const uint8_t *qt;          // queries padded to multiples of 16 with the pad code
   const int64_t *qt_off;      // [nq] offset of each padded query in qt
   const int32_t *qt_npad;     // [nq] padded length
@@ -247,36 +247,41 @@ int band_max_ctas_per_sm(int R, int gaps);  // plan time: raises the shared-memo
 // one_per_sm: reserve shared memory so that the launch places at most one CTA per SM
 cudaError_t launch_band(const BandArgs &a, int R, int grid, bool one_per_sm, cudaStream_t s);
 
-// Traceback of selected hits (k_trace.cu): one warp per hit fills 4-bit
-// provenance codes per cell, one thread per hit walks them back.
+// Traceback of selected hits (k_trace.cu): bands of query rows, one warp each,
+// fill 4-bit provenance codes per cell; one warp per hit walks them back.
 struct TraceHit {
   int64_t qoff;       // query residues in qres
   int64_t toff;       // target residues in tres (the database's sorted, padded residues)
-  int64_t dir_off;    // bytes into dirs: mrow * npad / 2, column-major nibbles (row i of column j at j * mrow + i)
-  int64_t strip_off;  // uint2 entries into strips: npad (bottom rows passed from the last warp to the first)
+  int64_t dir0;       // words into dirs: band b, step t, lane l at dir0 + (b * (npad + 32) + t) * 32 + l
+                      // (8 rows of column t - l, 4 bits each)
   int64_t ops_off;    // bytes into ops: m + n
-  int32_t m, n, npad, mrow;  // query and target lengths, padded target length, rows padded to whole chunks
+  int32_t m, n, npad; // query and target lengths, padded target length
+  int32_t nb, band0;  // bands, and the first one's index among all hits'
+  int32_t pad_;
 };
 struct TraceResult {
   int32_t score, end_i, end_j;  // best score and its cell (1-based row, column; first in row-major order)
   int32_t begin_i, begin_j;     // the alignment covers rows begin_i+1 .. end_i, columns begin_j+1 .. end_j
-  int32_t n_ops;                // -1: the fill gave up on a bounded wait
+  int32_t n_ops;
 };
 struct TraceArgs {
   const uint8_t *qres, *tres;
   const int8_t *submat;  // 20x20
   const TraceHit *hits;
-  int32_t nhits;
-  uint8_t *dirs;
-  uint2 *strips;
+  const int32_t *band_hit;    // [nbands] hit of each band (a hit's bands consecutive, in order)
+  int32_t nhits, nbands;
+  int32_t *band_counter;      // (cleared by launch_trace, as is the status)
+  int32_t *status;            // SW_ETIMEOUT on an expired wait
+  uint32_t *dirs;
+  int4 *best;                 // [nbands] best score of each band and its cell
   uint8_t *ops;
   TraceResult *results;
   Scoring sc;
+  // buffer sizes, tested by the checked build (-DSW_CHECK) before every access
+  int64_t tres_bytes, dir_words;
 };
-int trace_rows_per_chunk();
-int trace_warps(int max_chunks);  // warps per CTA of the fill: chunks of one hit in flight
-size_t trace_smem_bytes(int warps);
-cudaError_t launch_trace(const TraceArgs &a, int warps, cudaStream_t s);
+int trace_rows_per_band();
+cudaError_t launch_trace(const TraceArgs &a, int sms, cudaStream_t s);
 
 // launchers (k_inter.cu)
 int inter_threads();

@@ -106,11 +106,11 @@ __device__ __forceinline__ bool band_unit(const BandArgs &a, const uint8_t *__re
   __syncwarp();  // (the unit before this one has read its residues and slots)
   rs.stage(0);
   clear_slots(rgb, lane, PACKED ? cs.F0W : 0u);
-  OnceRing x{ring_in ? ring_in + sbase : nullptr, ring_out ? ring_out + sbase : nullptr, rgb, lane, a.rings,
+  OnceRing<> x{ring_in ? ring_in + sbase : nullptr, ring_out ? ring_out + sbase : nullptr, rgb, lane, a.rings,
              a.ring_entries, a.status, ring_in != nullptr, ring_out != nullptr};
   BandLane<R, FORM, 1> ln;
   ln.reset(cs);
-  const bool ok = band_sweep<R, FORM, 1, kBandUnroll, false, Prof>(ln, rs, x, rgb, prof + lane * R, 32 * R, lane,
+  const bool ok = band_sweep<FORM, 1, kBandUnroll, false, Prof>(ln, rs, x, rgb, prof + lane * R, 32 * R, lane,
                                                       npad / kColBlock, (Word<FORM>)-1, (Word<FORM>)0, cs, a.status);
   cp_async_wait<0>();
   Sout = ln.S;
@@ -195,11 +195,6 @@ __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(cons
 // idle
 constexpr int kTrackThreads = 128;
 constexpr int kTrackCols = 2;  // columns per step (band_core.cuh)
-// Score table of the database residues: row k holds SM(c, k) for the query
-// residues c = 0..20 (pad), one byte each, rows 28 bytes apart (seven words:
-// the 21 codes of a word's lookups fall in different banks)
-constexpr int kScoreRow = 28;
-constexpr int kScoreBytes = 640;
 template <int R>
 constexpr int kTrackStride = 32 * R;                                // bytes per residue row of one table
 template <int R>
@@ -208,30 +203,12 @@ constexpr int kTrackIoBytes = 2 * kResChunk + 2 * kColBlock * 8;    // residues,
 template <int R>
 constexpr int kTrackWarpBytes = (kTrackProfBytes<R> + kTrackIoBytes + 127) / 128 * 128;
 
-// N words to byte p (as aligned as load_prof reads them).
-template <int N>
-__device__ __forceinline__ void store_words(uint8_t *p, const uint32_t (&w)[N]) {
-  if constexpr (N % 4 == 0) {
-#pragma unroll
-    for (int i = 0; i < N / 4; ++i)
-      reinterpret_cast<uint4 *>(p)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
-  } else if constexpr (N % 2 == 0) {
-#pragma unroll
-    for (int i = 0; i < N / 2; ++i) reinterpret_cast<uint2 *>(p)[i] = make_uint2(w[2 * i], w[2 * i + 1]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < N; ++i) reinterpret_cast<uint32_t *>(p)[i] = w[i];
-  }
-}
-
 // Profile of a band's rows: the substitution score of query residue c
 // (column) against each database row, SM(c, D[row]) (the query residue is
 // the matrix's row index): table t, byte (c, lane, r) at (21 t + c) * stride
 // + lane * R + r, for the low (t = 0) and high (t = 1) track.  Rows past a
 // sequence's end, idle lanes and the pad residue (c = 20) hold the pad value.
-// Four rows' scores against four query residues are four words of the score
-// table, transposed by byte shuffles: the whole profile takes a byte lookup's
-// instructions per four bytes (R = 24: 10.4 -> 2 us of a small search).
+// (R = 24: 10.4 -> 3.4 us of a small search against a byte lookup per score.)
 template <int R, bool TWO>
 __device__ __forceinline__ void build_track_profile(uint8_t *prof, const uint8_t *score, const DbView &db,
                                                     const TrackLane &L, int lane, int32_t *status) {
@@ -248,27 +225,7 @@ __device__ __forceinline__ void build_track_profile(uint8_t *prof, const uint8_t
       code[i] = (row < npad && in_range(res + row + 3 - db.res, db.res_bytes, status))
                     ? *reinterpret_cast<const uint32_t *>(res + row) : 0x14141414u;
     }
-    uint8_t *p = prof + t * kProfRows * kTrackStride<R> + lane * R;
-#pragma unroll 1
-    for (int w = 0; w < (kProfRows + 3) / 4; ++w) {
-      uint32_t out[4][R / 4];
-#pragma unroll
-      for (int i = 0; i < R / 4; ++i) {
-        uint32_t v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          v[j] = *reinterpret_cast<const uint32_t *>(score + prmt(code[i], 0u, sel_one(j)) * kScoreRow + 4 * w);
-        const uint32_t a = prmt(v[0], v[1], 0x5140u), b = prmt(v[2], v[3], 0x5140u);
-        const uint32_t c = prmt(v[0], v[1], 0x7362u), d = prmt(v[2], v[3], 0x7362u);
-        out[0][i] = prmt(a, b, 0x5410u);
-        out[1][i] = prmt(a, b, 0x7632u);
-        out[2][i] = prmt(c, d, 0x5410u);
-        out[3][i] = prmt(c, d, 0x7632u);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (4 * w + j < kProfRows) store_words(p + (4 * w + j) * kTrackStride<R>, out[j]);
-    }
+    profile_from_scores<R>(prof + t * kProfRows * kTrackStride<R> + lane * R, kTrackStride<R>, score, code);
   }
 }
 
@@ -286,10 +243,10 @@ __device__ __forceinline__ bool track_pass(const TrackArgs &a, const uint8_t *__
   constexpr bool PACKED = FORM != kFormInt32;
   using Prof = std::conditional_t<PACKED, TablePairProfile<R, kTrackCols>, IntProfile<R, kTrackCols>>;
   clear_slots(rgb, lane, PACKED ? cs.F0W : 0u);
-  OnceRing x{ring_in, ring_out, rgb, lane, a.rings, a.ring_entries, a.status, ring_in != nullptr, ring_out != nullptr};
+  OnceRing<> x{ring_in, ring_out, rgb, lane, a.rings, a.ring_entries, a.status, ring_in != nullptr, ring_out != nullptr};
   BandLane<R, FORM, kTrackCols> ln;
   ln.reset(cs);
-  const bool ok = band_sweep<R, FORM, kTrackCols, U, true, Prof>(ln, rs, x, rgb, prof + lane * R, kTrackStride<R>, lane,
+  const bool ok = band_sweep<FORM, kTrackCols, U, true, Prof>(ln, rs, x, rgb, prof + lane * R, kTrackStride<R>, lane,
                                                               npad / kColBlock, keepH, addF, cs, a.status);
   cp_async_wait<0>();
   Sout = ln.S;
@@ -354,10 +311,7 @@ __global__ void __launch_bounds__(kTrackThreads, R <= 8 ? 4 : R <= 20 ? 2 : 1) b
   uint8_t *prof = smem + kScoreBytes + (size_t)warp * kTrackWarpBytes<R>;
   uint8_t *io = prof + kTrackProfBytes<R>;
   uint2 *rgb = reinterpret_cast<uint2 *>(io + 2 * kResChunk);
-  for (int i = threadIdx.x; i < kProfRows * kScoreRow; i += blockDim.x) {
-    const int k = i / kScoreRow, c = i - k * kScoreRow;
-    smem[i] = (uint8_t)(k < kAlphabet && c < kAlphabet ? a.submat[c * kAlphabet + k] : a.sc.pad);
-  }
+  build_scores<true>(smem, a.submat, a.sc.pad);
   __syncthreads();
   const Consts cs = make_consts<GAPS>(a.sc);
   const TrackLane idle{-1, 0, -1, 0};

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(32 * kPairWarps, 1) pair_band_kernel(const Pai
     x.hi_bias = (uint32_t)cs.go + (band_gen(b, a.nslots) << 31);
     BandLane<R, kFormInt32, kPairCols> ln;
     ln.reset(cs);
-    const bool ok = band_sweep<R, kFormInt32, kPairCols, kPairUnroll<R>, false, IntProfile<R, kPairCols>>(
+    const bool ok = band_sweep<kFormInt32, kPairCols, kPairUnroll<R>, false, IntProfile<R, kPairCols>>(
         ln, rs, x, rgb, pbuf + lane * kSlotBytes<R>, a.stride, lane, a.npad / kColBlock, -1, 0, cs, a.status);
     cp_async_wait<0>();
     S = max(S, ln.S);

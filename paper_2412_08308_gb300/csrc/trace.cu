@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <numeric>
 #include <vector>
 
 #include "host_pool.h"
@@ -67,11 +68,10 @@ extern "C" int sw_traceback(const sw_db *db, const uint8_t *queries, const int64
     return tr_fail(SW_EINVAL, "sw_traceback: gap penalties out of range (%lld, %lld)", gap_open, gap_extend);
   const int64_t ndb = db_view(db).n;
 
-  // per-hit layout: direction nibbles, operations
-  const int chunk = trace_rows_per_chunk();
+  // per-hit layout: bands, direction words, operations
+  const int band_rows = trace_rows_per_band();
   std::vector<TraceHit> th((size_t)n_hits);
-  int64_t dir_bytes = 0, strip_entries = 0, ops_bytes = 0;
-  int max_chunks = 1;
+  int64_t dir_words = 0, ops_bytes = 0, nbands = 0;
   for (int64_t h = 0; h < n_hits; ++h) {
     const int32_t qi = hits[h].query, ti = hits[h].target;
     if (qi < 0 || qi >= n_queries) return tr_fail(SW_EINVAL, "sw_traceback: hit %lld: query index %lld out of range", h, qi);
@@ -83,32 +83,56 @@ extern "C" int sw_traceback(const sw_db *db, const uint8_t *queries, const int64
     x.toff = db_sorted_off(db, pos);
     x.n = db_sorted_len(db, pos);
     x.npad = db_sorted_npad(db, pos);
-    x.mrow = (int32_t)std::max<int64_t>(chunk, tr_round_up(x.m, chunk));
-    x.dir_off = dir_bytes;
-    x.strip_off = strip_entries;
+    x.nb = std::max(1, (x.m + band_rows - 1) / band_rows);
+    x.dir0 = dir_words;
     x.ops_off = ops_bytes;
-    strip_entries += tr_round_up(x.npad, 32);
-    dir_bytes += tr_round_up((int64_t)x.mrow * x.npad / 2, 256);
+    dir_words += (int64_t)x.nb * (x.npad + 32) * 32;
     ops_bytes += (int64_t)x.m + x.n;
-    max_chunks = std::max(max_chunks, x.mrow / chunk);
+    nbands += x.nb;
   }
+  if (nbands >= ((int64_t)1 << 31)) return tr_fail(SW_EINVAL, "sw_traceback: too many bands");
   if (ops_bytes > ops_capacity)
     return tr_fail(SW_EINVAL, "sw_traceback: ops buffer holds %lld bytes, the hits need %lld", ops_capacity,
                    ops_bytes);
   if (ops_bytes > 0 && !ops) return tr_fail(SW_EINVAL, "sw_traceback: null ops");
 
+  // the bands of all hits, the hits that take longest first
+  std::vector<int32_t> order((size_t)n_hits), band_hit((size_t)nbands);
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+    return (int64_t)th[x].npad + 64 * (int64_t)th[x].nb > (int64_t)th[y].npad + 64 * (int64_t)th[y].nb;
+  });
+  int32_t next_band = 0;
+  for (int32_t h : order) {
+    th[h].band0 = next_band;
+    for (int32_t b = 0; b < th[h].nb; ++b) band_hit[next_band++] = h;
+  }
+
   const int64_t b_q = tr_round_up(std::max<int64_t>(q_offsets[n_queries], 1), 256);
   const int64_t b_sub = 512, b_hits = tr_round_up((int64_t)sizeof(TraceHit) * n_hits, 256);
   const int64_t b_res = tr_round_up((int64_t)sizeof(TraceResult) * n_hits, 256);
   const int64_t b_ops = tr_round_up(std::max<int64_t>(ops_bytes, 1), 256);
-  const int64_t b_strip = tr_round_up(strip_entries * (int64_t)sizeof(uint2), 256);
-  const int64_t bytes = b_q + b_sub + b_hits + b_res + b_strip + b_ops + dir_bytes;
+  const int64_t b_bandhit = tr_round_up(4 * nbands, 256), b_best = tr_round_up((int64_t)sizeof(int4) * nbands, 256);
+  const int64_t b_words = 256;
+  const int64_t bytes = b_q + b_sub + b_hits + b_bandhit + b_best + b_res + b_words + b_ops + 4 * dir_words;
   cudaStream_t s = (cudaStream_t)stream;
   TraceScratch sc;
   sc.s = s;
   cudaError_t e = pool_alloc(&sc.block, (size_t)bytes, s);
   if (e != cudaSuccess) {
     sc.block = nullptr;
+    // (short hits take whole bands of 256 rows and 32 columns more: in two calls they need half at a time)
+    if (e == cudaErrorMemoryAllocation && n_hits > 1) {
+      cudaGetLastError();
+      const int64_t first = n_hits / 2, used = th[first].ops_off;
+      int rc = sw_traceback(db, queries, q_offsets, n_queries, hits, first, submat, gap_open, gap_extend, out, ops,
+                            ops_capacity, stream);
+      if (rc != SW_OK) return rc;
+      rc = sw_traceback(db, queries, q_offsets, n_queries, hits + first, n_hits - first, submat, gap_open, gap_extend,
+                        out + first, ops + used, ops_capacity - used, stream);
+      for (int64_t h = first; rc == SW_OK && h < n_hits; ++h) out[h].ops_offset += used;
+      return rc;
+    }
     return tr_cuda(e, "device allocation");
   }
   uint8_t *p = (uint8_t *)sc.block;
@@ -117,18 +141,25 @@ extern "C" int sw_traceback(const sw_db *db, const uint8_t *queries, const int64
   int8_t *d_sub = (int8_t *)(d_q + b_q);
   TraceHit *d_hits = (TraceHit *)((uint8_t *)d_sub + b_sub);
   TraceResult *d_res = (TraceResult *)((uint8_t *)d_hits + b_hits);
-  uint2 *d_strip = (uint2 *)((uint8_t *)d_res + b_res);
-  uint8_t *d_ops = (uint8_t *)d_strip + b_strip;
-  uint8_t *d_dirs = d_ops + b_ops;
+  int32_t *d_bandhit = (int32_t *)((uint8_t *)d_res + b_res);
+  int4 *d_best = (int4 *)((uint8_t *)d_bandhit + b_bandhit);
+  int32_t *d_words = (int32_t *)((uint8_t *)d_best + b_best);  // [0] band counter, [1] status
+  uint8_t *d_ops = (uint8_t *)d_words + b_words;
   a.qres = d_q;
   a.tres = db_view(db).res;
+  a.tres_bytes = db_view(db).res_bytes;
   a.submat = d_sub;
   a.hits = d_hits;
+  a.band_hit = d_bandhit;
   a.nhits = (int32_t)n_hits;
-  a.dirs = d_dirs;
+  a.nbands = (int32_t)nbands;
+  a.band_counter = d_words;
+  a.status = d_words + 1;
+  a.dirs = (uint32_t *)(d_ops + b_ops);
+  a.dir_words = dir_words;
+  a.best = d_best;
   a.ops = d_ops;
   a.results = d_res;
-  a.strips = d_strip;
   a.sc.go = gap_open + gap_extend;
   a.sc.ge = gap_extend;
   a.sc.pad = std::min(0, smin);
@@ -139,14 +170,21 @@ extern "C" int sw_traceback(const sw_db *db, const uint8_t *queries, const int64
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_sub, submat, 400, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_hits, th.data(), sizeof(TraceHit) * n_hits, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return tr_cuda(e, "upload");
-  if ((e = launch_trace(a, trace_warps(max_chunks), s)) != cudaSuccess) return tr_cuda(e, "traceback kernels");
+  if ((e = cudaMemcpyAsync(d_bandhit, band_hit.data(), 4 * (size_t)nbands, cudaMemcpyHostToDevice, s)) != cudaSuccess)
+    return tr_cuda(e, "upload");
+  int dev = 0, sms = 1;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return tr_cuda(e, "cudaGetDevice");
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if ((e = launch_trace(a, sms, s)) != cudaSuccess) return tr_cuda(e, "traceback kernels");
   std::vector<TraceResult> res((size_t)n_hits);
+  int32_t words[2] = {0, 0};
   e = cudaMemcpyAsync(res.data(), d_res, sizeof(TraceResult) * n_hits, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(words, d_words, sizeof words, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && ops_bytes > 0) e = cudaMemcpyAsync(ops, d_ops, ops_bytes, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return tr_cuda(e, "results");
-  for (int64_t h = 0; h < n_hits; ++h)
-    if (res[h].n_ops < 0) return tr_fail(SW_ETIMEOUT, "sw_traceback: hit %lld: a bounded device wait expired", h);
+  if (words[1] == SW_ETIMEOUT) return tr_fail(SW_ETIMEOUT, "sw_traceback: a bounded device wait expired");
+  if (words[1]) return tr_fail(SW_ECUDA, "sw_traceback: internal error: an index left its buffer (checked build)");
   for (int64_t h = 0; h < n_hits; ++h) {
     sw_alignment &o = out[h];
     o.score = res[h].score;
