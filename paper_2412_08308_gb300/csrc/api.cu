@@ -435,6 +435,9 @@ struct sw_queries {
   int64_t prof_bytes = 0;
   uint2 *d_gbuf = nullptr, *d_igbuf = nullptr;
   int32_t *d_words = nullptr;
+  // sw_search to host memory: the scores, directly after the words' b_words bytes and before the row tracks' rings
+  int32_t *d_scores = nullptr;
+  size_t b_words = 0, b_scores = 0;
   int32_t *d_flag_pos = nullptr, *d_iflag_pos = nullptr;
   // band-stream jobs (small batches): long queries against every unit, the
   // other queries against the long units
@@ -666,7 +669,9 @@ struct PlanScratch {
   std::vector<uint8_t> stage;  // the plan's upload, laid out like its device block
   std::vector<TW> tw;
   std::vector<Task> tasks;
+  std::vector<uint8_t> back;  // a search's words and scores on their way to the caller
 };
+constexpr int64_t kSearchStage = 64 << 10;
 
 PlanScratch &plan_scratch() {
   static thread_local PlanScratch ps;
@@ -684,9 +689,15 @@ PlanScratch &plan_scratch() {
 
 }  // namespace
 
-int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q_offsets, int64_t n_queries,
-                       const int8_t *submat, int32_t gap_open, int32_t gap_extend, int32_t mode,
-                       const sw_options *opts, void *stream, sw_queries **out) {
+// The plan of a batch, its device block and its upload.  one_search: for a
+// single search that reads its results back and frees the batch (sw_search):
+// the upload is not waited for (the caller's thread synchronises the stream
+// before it returns or plans again), and score_bytes of the block, if not 0,
+// hold its scores.
+static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_t *q_offsets, int64_t n_queries,
+                           const int8_t *submat, int32_t gap_open, int32_t gap_extend, int32_t mode,
+                           const sw_options *opts, void *stream, bool one_search, int64_t score_bytes,
+                           sw_queries **out) {
   g_err.clear();
   if (!out) return fail(SW_EINVAL, "sw_queries_prepare: null output handle");
   *out = nullptr;
@@ -1198,6 +1209,19 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
     }
     return 0.95 * std::max(thr, lat) + 0.15 * std::min(thr, lat);
   };
+  // A lower bound of the inter-task plan's modelled time: the longest query's
+  // chunks over the longest short unit, in the plan's rows or any of them,
+  // with the warp alone on its SM sub-partition.
+  auto inter_at_least = [&]() {
+    if (n_short <= 0) return 0.0;
+    double m = 1, best = 1e300;
+    for (int64_t q = 0; q < n_queries; ++q) m = std::max<double>(m, qlen(q));
+    for (int rows : {24, 16, 12, 8, 4})
+      if (!o.rows_per_lane || rows == o.rows_per_lane)
+        best = std::min(best, std::ceil(m / (32 * rows)) * max_short *
+                                  chain_step_cycles(packed ? kFormQPair : kFormInt32, rows, 1));
+    return best;
+  };
   // Which kernels: the small-batch ones (band-stream jobs for the long queries
   // and transposed ones for the others, or all transposed), or the inter- and
   // intra-task ones, by modelled time.  Above 16,384 sequences the inter-task
@@ -1213,19 +1237,6 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
       any_band |= band_q[q] != 0;
     }
     if (o.band_stream == 0 && n <= 16384) {
-      plan = best_plan();
-      double inter = plan.time;
-      if (n_long) {  // the intra-task kernel beside it: about 4.4 int32 cells per cycle and SM
-        double m_sum = 0, m_max = 0;
-        for (int64_t q = 0; q < n_queries; ++q) {
-          m_sum += qlen(q);
-          m_max = std::max<double>(m_max, qlen(q));
-        }
-        const double rate = packed && (int64_t)sc.maxp * max_long <= sc.thresh ? 9.6 : 4.4;
-        const double cols = (double)ust.prefix[(size_t)n_long] * (packed ? 2 : 1);
-        const double intra = std::max(m_max * max_long, m_sum * cols / sms) / rate;
-        inter = std::max(inter, intra) + 0.3 * std::min(inter, intra);
-      }
       const double tracks_a = rank_heights_of(), bands_a = any_band ? band_time() : 0.0;
       double best_small = std::max(tracks_a, bands_a) + 0.5 * std::min(tracks_a, bands_a);
       if (any_band) {  // all transposed?
@@ -1240,7 +1251,26 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
           track_q.swap(tq);
         }
       }
-      small = best_small < inter;
+      // (the plan is left out where its longest chain alone would take longer:
+      // one 144-residue query x 2,000 proteins, 7.6 of 130 us)
+      if (best_small < inter_at_least()) {
+        small = true;
+      } else {
+        plan = best_plan();
+        double inter = plan.time;
+        if (n_long) {  // the intra-task kernel beside it: about 4.4 int32 cells per cycle and SM
+          double m_sum = 0, m_max = 0;
+          for (int64_t q = 0; q < n_queries; ++q) {
+            m_sum += qlen(q);
+            m_max = std::max<double>(m_max, qlen(q));
+          }
+          const double rate = packed && (int64_t)sc.maxp * max_long <= sc.thresh ? 9.6 : 4.4;
+          const double cols = (double)ust.prefix[(size_t)n_long] * (packed ? 2 : 1);
+          const double intra = std::max(m_max * max_long, m_sum * cols / sms) / rate;
+          inter = std::max(inter, intra) + 0.3 * std::min(inter, intra);
+        }
+        small = best_small < inter;
+      }
     }
   }
   if (small) {
@@ -1723,7 +1753,8 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   const size_t b_qtoff = tmode ? round_up(8 * nqm, 256) : 0;
   const size_t b_qtnpad = tmode ? round_up(4 * nqm, 256) : 0;
   const size_t b_trings = tmode ? round_up(std::max<int64_t>(Q->track_ring_bytes, 8), 256) : 0;
-  Q->bytes = b_tjobs + b_tjobof + b_tlanes + b_qt + b_qtoff + b_qtnpad + b_trings + b_qres + b_sub + 2 * b_qd + b_tasks + b_itasks + b_itasks32 + b_ipos32 + b_rtasks + b_prof +
+  const size_t b_scores = round_up(score_bytes, 256);
+  Q->bytes = b_scores + b_tjobs + b_tjobof + b_tlanes + b_qt + b_qtoff + b_qtnpad + b_trings + b_qres + b_sub + 2 * b_qd + b_tasks + b_itasks + b_itasks32 + b_ipos32 + b_rtasks + b_prof +
              b_gbuf + b_igbuf + b_words + b_flag + b_iflag + b_qdp + b_ptasks + b_track + b_bjobs + b_bjobof +
              b_btpos + b_brings;
   cudaMemPool_t pool = nullptr;
@@ -1749,7 +1780,6 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   Q->d_itasks = (Task *)take(b_itasks);
   Q->d_itasks32 = (Task *)take(b_itasks32);
   Q->d_ipos32 = (int32_t *)take(b_ipos32);
-  Q->d_words = (int32_t *)take(b_words);
   Q->d_qdp = (QDesc *)take(b_qdp);
   Q->d_track = (TrackChunk *)take(b_track);
   Q->d_ptasks = (Task *)take(b_ptasks);
@@ -1764,8 +1794,13 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
     Q->d_qt_off = (int64_t *)take(b_qtoff);
     Q->d_qt_npad = (int32_t *)take(b_qtnpad);
   }
+  Q->d_words = (int32_t *)take(b_words);
+  Q->b_words = b_words;
   const size_t up_bytes = (size_t)(p - (uint8_t *)Q->block);
   // device-only regions
+  if (b_scores) Q->d_scores = (int32_t *)take(b_scores);
+  Q->b_scores = b_scores;
+  if (tmode) Q->d_trings = (unsigned long long *)take(b_trings);
   Q->d_rtasks = (Task *)take(b_rtasks);
   Q->d_prof = take(b_prof);
   Q->d_gbuf = (uint2 *)take(b_gbuf);
@@ -1773,7 +1808,6 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   Q->d_flag_pos = Q->inter_may_flag ? (int32_t *)take(b_flag) : nullptr;
   Q->d_iflag_pos = packed ? (int32_t *)take(b_iflag) : nullptr;
   Q->d_brings = Q->n_bjobs ? (unsigned long long *)take(b_brings) : nullptr;
-  if (tmode) Q->d_trings = (unsigned long long *)take(b_trings);
   Q->d_upos = const_cast<int32_t *>(db->d_ident) + s0;  // the short sequences, in sorted order
   Q->n_upos = n + 1 - s0;
 
@@ -1842,7 +1876,7 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(&Q->join2, cudaEventDisableTiming);
     }
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess && !one_search) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     free_queries(Q);
     return cuda_fail(e, "sw_queries_prepare: upload");
@@ -1851,13 +1885,21 @@ int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q
   return SW_OK;
 }
 
+int sw_queries_prepare(const sw_db *db, const uint8_t *queries, const int64_t *q_offsets, int64_t n_queries,
+                       const int8_t *submat, int32_t gap_open, int32_t gap_extend, int32_t mode,
+                       const sw_options *opts, void *stream, sw_queries **out) {
+  return prepare_queries(db, queries, q_offsets, n_queries, submat, gap_open, gap_extend, mode, opts, stream, false, 0,
+                         out);
+}
+
 int sw_queries_free(sw_queries *q) {
   g_err.clear();
   free_queries(q);
   return SW_OK;
 }
 
-int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev, void *stream) {
+// fresh: the batch has just been uploaded (its words are zero)
+static int search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev, void *stream, bool fresh) {
   g_err.clear();
   if (!db || !Q) return fail(SW_EINVAL, "sw_search_prepared: null handle");
   if (Q->db != db) return fail(SW_EINVAL, "sw_search_prepared: query batch prepared for another database");
@@ -1869,7 +1911,7 @@ int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev
   const int nq = (int)Q->nq;
   int32_t *w = Q->d_words;
 
-  SW_CUDA(cudaMemsetAsync(w, 0, 4 * Q->zero_words(), s), "memset");
+  if (!fresh) SW_CUDA(cudaMemsetAsync(w, 0, 4 * Q->zero_words(), s), "memset");
   std::unique_ptr<StageRange> stage(new StageRange("swgb: query profiles"));
   if (Q->n_solo)
     SW_CUDA(launch_build_profiles(Q->d_qres, Q->d_qd, nq, Q->d_submat, Q->sc.pad, Q->d_prof, s), "profile kernel");
@@ -1884,7 +1926,14 @@ int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev
   stage.reset(new StageRange("swgb: dynamic programming"));
   // band-stream and transposed jobs add their scores with atomicMax: every score starts at 0
   const bool small = Q->n_bjobs || Q->n_tjobs;
-  if (small) SW_CUDA(cudaMemsetAsync(scores_dev, 0, 4 * (size_t)Q->nq * (size_t)db->n, s), "memset");
+  // (the block's own scores lie before the row tracks' rings: one memset for both)
+  const bool with_rings = Q->n_tjobs && scores_dev == Q->d_scores;
+  if (small)
+    SW_CUDA(cudaMemsetAsync(scores_dev, 0,
+                            with_rings ? Q->b_scores + (size_t)Q->track_ring_bytes
+                                       : 4 * (size_t)Q->nq * (size_t)db->n,
+                            s),
+            "memset");
   const bool band_timing = Q->timing && small;
   if (band_timing) SW_CUDA(cudaEventRecord(Q->ev0, s), "event");
 
@@ -1963,7 +2012,7 @@ int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev
   }
 
   if (Q->n_tjobs) {  // transposed jobs, on the caller's stream beside the band-stream ones
-    SW_CUDA(cudaMemsetAsync(Q->d_trings, 0, (size_t)Q->track_ring_bytes, s), "memset");
+    if (!with_rings) SW_CUDA(cudaMemsetAsync(Q->d_trings, 0, (size_t)Q->track_ring_bytes, s), "memset");
     TrackArgs ta{};
     ta.db = db->view;
     ta.lanes = Q->d_tlanes;
@@ -2049,6 +2098,10 @@ int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev
   return SW_OK;
 }
 
+int sw_search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores_dev, void *stream) {
+  return search_prepared(db, Q, scores_dev, stream, false);
+}
+
 int sw_search_graph(const sw_db *db, sw_queries *Q, int32_t *scores_dev, void *stream) {
   g_err.clear();
   if (!db || !Q) return fail(SW_EINVAL, "sw_search_graph: null handle");
@@ -2085,13 +2138,8 @@ int sw_search_graph(const sw_db *db, sw_queries *Q, int32_t *scores_dev, void *s
   return SW_OK;
 }
 
-int sw_queries_status(const sw_queries *Q, void *stream, int64_t *rescued) {
-  g_err.clear();
-  if (!Q) return fail(SW_EINVAL, "sw_queries_status: null handle");
-  cudaStream_t s = (cudaStream_t)stream;
-  std::vector<int32_t> w(Q->zero_words());
-  SW_CUDA(cudaMemcpyAsync(w.data(), Q->d_words, 4 * w.size(), cudaMemcpyDeviceToHost, s), "status read");
-  SW_CUDA(cudaStreamSynchronize(s), "status sync");
+// what the words of a finished search say
+static int words_status(const sw_queries *Q, const int32_t *w, int64_t *rescued) {
   int64_t inter_flags = 0, intra_flags = 0;
   for (int64_t q = 0; q < Q->nq; ++q) {
     inter_flags += w[8 + q];
@@ -2103,6 +2151,16 @@ int sw_queries_status(const sw_queries *Q, void *stream, int64_t *rescued) {
   if (w[2] == kStatusBounds) return fail(SW_ECUDA, "internal error: an index left its buffer (checked build)");
   if (intra_flags) return fail(SW_ECUDA, "internal error: a packed intra-task lane passed its bound");
   return SW_OK;
+}
+
+int sw_queries_status(const sw_queries *Q, void *stream, int64_t *rescued) {
+  g_err.clear();
+  if (!Q) return fail(SW_EINVAL, "sw_queries_status: null handle");
+  cudaStream_t s = (cudaStream_t)stream;
+  std::vector<int32_t> w(Q->zero_words());
+  SW_CUDA(cudaMemcpyAsync(w.data(), Q->d_words, 4 * w.size(), cudaMemcpyDeviceToHost, s), "status read");
+  SW_CUDA(cudaStreamSynchronize(s), "status sync");
+  return words_status(Q, w.data(), rescued);
 }
 
 int sw_queries_set_timing(sw_queries *q, int32_t enable) {
@@ -2154,30 +2212,34 @@ int sw_search(const sw_db *db, const uint8_t *queries, const int64_t *q_offsets,
   g_err.clear();
   if (!db) return fail(SW_EINVAL, "sw_search: null database");
   if (n_queries > 0 && db->n > 0 && !scores_out) return fail(SW_EINVAL, "sw_search: null scores");
+  const int64_t count = n_queries > 0 && n_queries <= std::numeric_limits<int32_t>::max() ? n_queries * db->n : 0;
+  const bool host = count > 0 && !is_device_ptr(scores_out);
   sw_queries *Q = nullptr;
-  int rc = sw_queries_prepare(db, queries, q_offsets, n_queries, submat, gap_open, gap_extend, mode, nullptr, stream,
-                              &Q);
+  int rc = prepare_queries(db, queries, q_offsets, n_queries, submat, gap_open, gap_extend, mode, nullptr, stream, true,
+                           host ? 4 * count : 0, &Q);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t count = n_queries * db->n;
-  int32_t *dst = scores_out;
-  void *tmp = nullptr;
-  const bool dev = count > 0 && is_device_ptr(scores_out);
-  if (count > 0 && !dev) {
-    cudaError_t e = swgb::pool_alloc(&tmp, 4 * count, s);
-    if (e != cudaSuccess) {
-      free_queries(Q);
-      return cuda_fail(e, "sw_search: score buffer");
-    }
-    dst = (int32_t *)tmp;
-  }
-  rc = count > 0 ? sw_search_prepared(db, Q, dst, stream) : SW_OK;
-  if (rc == SW_OK && count > 0 && !dev) {
-    cudaError_t e = cudaMemcpyAsync(scores_out, dst, 4 * count, cudaMemcpyDeviceToHost, s);
+  if (count > 0) rc = search_prepared(db, Q, host ? Q->d_scores : scores_out, stream, true);
+  // The words (status, flag counts) and, up to 64 KB, the scores after them
+  // come back in one copy: a copy to pageable memory waits for the device and
+  // then for its own staging, 11 us each for a search of 130 us.
+  const size_t words = 4 * (size_t)Q->zero_words();
+  const bool together = host && 4 * count <= kSearchStage;
+  std::vector<uint8_t> &back = plan_scratch().back;
+  back.resize(together ? Q->b_words + 4 * (size_t)count : words);
+  if (rc == SW_OK && host && !together) {
+    cudaError_t e = cudaMemcpyAsync(scores_out, Q->d_scores, 4 * count, cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) rc = cuda_fail(e, "sw_search: score copy");
   }
-  if (rc == SW_OK) rc = sw_queries_status(Q, stream, nullptr);
-  if (tmp) cudaFreeAsync(tmp, s);
+  if (rc == SW_OK) {
+    cudaError_t e = cudaMemcpyAsync(back.data(), Q->d_words, back.size(), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) rc = cuda_fail(e, "sw_search: results");
+  }
+  if (rc == SW_OK) {
+    if (together) memcpy(scores_out, back.data() + Q->b_words, 4 * (size_t)count);
+    rc = words_status(Q, (const int32_t *)back.data(), nullptr);
+  }
   std::string keep = g_err;
   free_queries(Q);
   g_err = keep;
