@@ -38,23 +38,18 @@ WORKLOAD = "protein DB search: 20 queries (144-5478 aa) x 200,000 synthetic prot
 SM_COUNT_FALLBACK = 152
 # The integer ALU pipe of an sm_103 SMSP accepts one warp instruction every
 # second cycle (ncu: a stream of IMNMX / VIMNMX / IADD / PRMT runs the ALU pipe
-# at ~99% with issue at ~51%), i.e. 64 lanes per clock per SM.  Every max of
-# the recurrences runs there; the DP kernels are bound by it.  The FMA pipe is
-# a second integer pipe of the same width (it takes the per-half 16x2 adds).
+# at ~99% with issue at ~51%), i.e. 64 lanes per clock per SM.  Every maximum of
+# the recurrences runs there, whether it has two inputs, three, or an addition
+# fused to it; the DP kernels are bound by it.  Additions on their own (the
+# per-half 16x2 adds, the byte dot products) go to the FMA pipe.
 ALU_LANES_PER_SM_CLK = 64
-INT_PIPES = 2  # ALU + FMA: the lanes the paper's instruction model (Eqs. 4-6) can use for adds and maxima
-# Algorithmic integer operations per cell, the roofline's count:
-#  - packed s16x2: about 6 operations per 32-bit word of two cells (H - Go
-#    shared by E and F, the E and F max-adds, H_diag + SM, the three-way max
-#    with the zero floor, the running best), i.e. 3 per cell -- every one of
-#    them issues on the ALU pipe (adds fuse into the maxima that consume them);
-#  - int32: the 12 statements of Algorithm 1 (the paper's model, Eq. 6),
-#    against both integer pipes.
-# The maxima alone (the ALU pipe's irreducible work): 5 per word (2.5 per
-# cell) packed, 6 per cell int32.
-ALG_OPS_PER_CELL = {"packed": 3.0, "int32": 12.0}
-ALG_PIPES = {"packed": 1, "int32": INT_PIPES}
-ALU_MAX_OPS_PER_CELL = {"packed": 2.5, "int32": 6.0}
+# Instructions on that pipe that a cell (int32) or a word of two cells (packed
+# s16x2) cannot do without, the roofline's count: one three-input maximum for
+# H (the zero floor free in it), an add-maximum each for E and F, half a
+# three-input maximum for the running best: 3.5.
+ALG_OPS_PER_CELL = {"packed": 1.75, "int32": 3.5}
+ALG_PIPES = {"packed": 1, "int32": 1}
+ALU_MAX_OPS_PER_CELL = ALG_OPS_PER_CELL  # (all of them are maxima)
 
 
 def roofline_of(gcups, mode, n_sm, sm_mhz):

@@ -27,11 +27,11 @@
 //
 // Cell arithmetic
 // ---------------
-// int32 form: the twelve-instruction body of Algorithm 1, one cell per lane op.
+// int32 form: one cell per lane op (int_rows_of in dp_common.cuh).
 // packed forms: two cells per 32-bit word, each 16-bit half a signed cell
 // value (two database sequences, or two queries against one sequence);
 // additions are per-half (__vadd2 / __vsub2, no carry crosses the halves) and
-// maxima are per-half VIMNMX (__vmaxs2, __vimax_s16x2_relu for the zero floor).
+// maxima are per half, of three inputs (word_rows in dp_common.cuh).
 // E and F never fall below -Go, so no half wraps downward; a half whose final
 // score exceeds 32767 - max(SM) may have wrapped upward and is flagged and
 // recomputed exactly in int32 (rescue pass; query pairs are planned only where
