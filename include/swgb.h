@@ -246,8 +246,8 @@ int sw_queries_info(const sw_queries *q, int64_t *h2d_bytes, int64_t *device_byt
  *               owned by the caller
  *   stream      stream for the work
  *
- * The call allocates and frees its own scratch (the batch's block and, for
- * host scores, a device score buffer, both from the library's stream-ordered
+ * The call allocates and frees its own scratch (the batch's block, which for
+ * host scores holds the device scores too, from the library's stream-ordered
  * memory pool of the current device, which keeps up to 1 GiB of freed blocks
  * for the next call) and returns when the scores are in place.  Errors: as
  * sw_queries_prepare / sw_search_prepared, plus SW_ETIMEOUT.
