@@ -413,6 +413,23 @@ int sw_traceback(const sw_db *db, const uint8_t *queries, const int64_t *q_offse
 int sw_selftest_wait(int32_t which, int64_t budget_cycles, int32_t *status_out, void *stream);
 
 /*
+ * sw_selftest_trace -- check what sw_traceback's kernels leave behind when a
+ * wait between the bands of a hit expires.  Runs them on one made-up hit (a
+ * query of more bands than the GPU holds warps against 16 residues) in memory
+ * that holds the remains of other work, with budget_cycles for each wait.
+ *
+ *   budget_cycles  clock cycles, in (0, 2^36]; a few thousand always expire,
+ *                  2^33 (about 4 s) never does
+ *   status_out     host pointer: SW_ETIMEOUT when a wait expired, else SW_OK
+ *   score_out      host pointer: the alignment's score (16), or -1 when none
+ *                  was written
+ *   stream         stream for the work; the call returns when done
+ *
+ * Errors: SW_EINVAL, SW_ENOMEM, SW_ECUDA.
+ */
+int sw_selftest_trace(int64_t budget_cycles, int32_t *status_out, int32_t *score_out, void *stream);
+
+/*
  * sw_last_error -- the message of the last failed call on this thread, or ""
  * if it succeeded.  The paper has no error interface; the message names the
  * argument or CUDA call that failed (the status code of every entry point

@@ -35,6 +35,7 @@ SIGNATURES = {
     "sw_align_pair": (ctypes.c_int, [_p, _i64, _p, _i64, _p, _i32, _i32, _p, _p, _p, _p]),
     "sw_traceback": (ctypes.c_int, [_p, _p, _p, _i64, _p, _i64, _p, _i32, _i32, _p, _p, _i64, _p]),
     "sw_selftest_wait": (ctypes.c_int, [_i32, _i64, ctypes.POINTER(ctypes.c_int32), _p]),
+    "sw_selftest_trace": (ctypes.c_int, [_i64, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32), _p]),
     "sw_last_error": (ctypes.c_char_p, []),
 }
 
@@ -205,3 +206,10 @@ def sw_selftest_wait(which, budget_cycles, stream):
     st = ctypes.c_int32(-1)
     check(lib().sw_selftest_wait(int(which), int(budget_cycles), ctypes.byref(st), stream))
     return st.value
+
+
+def sw_selftest_trace(budget_cycles, stream):
+    """Returns (status, score)."""
+    st, score = ctypes.c_int32(-1), ctypes.c_int32(-1)
+    check(lib().sw_selftest_trace(int(budget_cycles), ctypes.byref(st), ctypes.byref(score), stream))
+    return st.value, score.value

@@ -427,6 +427,7 @@ struct OnceRing {
   bool prev, next;
   uint32_t lo_bias = 0x80000000u, hi_bias = 0u;
   unsigned long long pend = 0ull;
+  long long budget = kWaitBudgetCycles;  // of a wait
 
   __device__ __forceinline__ bool fresh() const { return (pend >> 31 & 1ull) != 0ull; }
   __device__ __forceinline__ void load() {
@@ -437,7 +438,7 @@ struct OnceRing {
     if (!__all_sync(0xffffffffu, ok)) {
       const long long t0 = clock64();
       do {
-        if (__any_sync(0xffffffffu, clock64() - t0 > kWaitBudgetCycles)) {
+        if (__any_sync(0xffffffffu, clock64() - t0 > budget)) {
           if (lane == 0) atomicExch(status, SW_ETIMEOUT);
           return false;
         }

@@ -272,6 +272,7 @@ struct TraceArgs {
   int32_t nhits, nbands;
   int32_t *band_counter;      // (cleared by launch_trace, as is the status)
   int32_t *status;            // SW_ETIMEOUT on an expired wait
+  long long wait_cycles;      // clock budget of a wait for the band above
   uint32_t *dirs;
   int4 *best;                 // [nbands] best score of each band and its cell
   uint8_t *ops;
@@ -280,6 +281,9 @@ struct TraceArgs {
   // buffer sizes, tested by the checked build (-DSW_CHECK) before every access
   int64_t tres_bytes, dir_words;
 };
+// Clock budget of a traceback's waits, ~60 s: the bands of a long hit wait on
+// one another as long as the longest of them takes.
+constexpr long long kTraceWaitCycles = 120000000000LL;
 int trace_rows_per_band();
 cudaError_t launch_trace(const TraceArgs &a, int sms, cudaStream_t s);
 

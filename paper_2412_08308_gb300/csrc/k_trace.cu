@@ -147,6 +147,8 @@ __global__ void __launch_bounds__(kTraceThreads, 4) trace_fill_kernel(const Trac
     if (lane == 0) g = atomicAdd(a.band_counter, 1);
     g = __shfl_sync(0xffffffffu, g, 0);
     if (g >= a.nbands) break;
+    // (a wait of another band has expired: the entries of its bands below never come)
+    if (*(const volatile int32_t *)a.status != 0) break;
     const TraceHit hit = a.hits[a.band_hit[g]];
     const int b = g - hit.band0;
     __syncwarp();  // (the band before this one has read its profile, residues and slots)
@@ -172,6 +174,7 @@ __global__ void __launch_bounds__(kTraceThreads, 4) trace_fill_kernel(const Trac
     OnceRing<kBlockWords / 2> x{ring, ring + band_words / 2, rgb, lane,
                                 reinterpret_cast<const unsigned long long *>(a.dirs), a.dir_words / 2, a.status, b > 0,
                                 b + 1 < hit.nb};
+    x.budget = a.wait_cycles;
     TraceLane ln{};
     ln.row0 = row0;
     ln.n = hit.n;
@@ -212,6 +215,7 @@ __global__ void __launch_bounds__(kTraceThreads, 4) trace_fill_kernel(const Trac
 // them (64 x 8: two runs, 302 against 265 us for 200 hits).
 constexpr int kWalkSteps = 144, kWalkLanes = 16;
 __global__ void __launch_bounds__(128) trace_walk_kernel(const TraceArgs a) {
+  if (*a.status != 0) return;  // the fill gave up: bands not taken have left no best cell
   __shared__ __align__(16) uint32_t tiles[4][kWalkSteps * kWalkLanes];
   __shared__ int8_t sm[kAlphabet * kAlphabet];
   for (int x = threadIdx.x; x < kAlphabet * kAlphabet; x += blockDim.x) sm[x] = a.submat[x];
@@ -240,6 +244,8 @@ __global__ void __launch_bounds__(128) trace_walk_kernel(const TraceArgs a) {
       bj = oj;
     }
   }
+  // (every index below follows from the cell)
+  if (!in_range(bi, (int64_t)hit.m + 1, a.status) || !in_range(bj, (int64_t)hit.n + 1, a.status)) return;
   const uint32_t *dirs = a.dirs + hit.dir0;
   const uint8_t *q = a.qres + hit.qoff, *t = a.tres + hit.toff;
   const int steps = hit.npad + 32;

@@ -155,6 +155,7 @@ extern "C" int sw_traceback(const sw_db *db, const uint8_t *queries, const int64
   a.nbands = (int32_t)nbands;
   a.band_counter = d_words;
   a.status = d_words + 1;
+  a.wait_cycles = kTraceWaitCycles;
   a.dirs = (uint32_t *)(d_ops + b_ops);
   a.dir_words = dir_words;
   a.best = d_best;
