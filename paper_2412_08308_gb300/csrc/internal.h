@@ -148,6 +148,7 @@ struct PairBandArgs {
   int32_t *best;           // max over all cells (atomicMax), zeroed before launch
   int32_t *status;         // SW_ETIMEOUT on an expired wait
   Scoring sc;
+  int64_t ring_entries;    // entries of `strips`, tested by the checked build (-DSW_CHECK) before every access
 };
 size_t pair_smem_bytes(int pbuf_bytes, int warps);
 int pair_max_warps();        // warps of a CTA, at most

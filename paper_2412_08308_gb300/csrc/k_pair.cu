@@ -66,6 +66,8 @@ struct WrapRing {
   int32_t go;
   uint2 *rgb;
   int lane;
+  const unsigned long long *base;  // the rings and their entries (checked build)
+  int64_t entries;
   bool prev, next;
   uint32_t lo_bias, hi_bias;     // this lap's tag in H's word; Go and the generation tag in F's
   // reading: ring position and lap parity of the next block, columns consumed
@@ -79,7 +81,7 @@ struct WrapRing {
     return ((uint32_t)pend >> 31) == rlap && (uint32_t)(pend >> 63) == gen_in;
   }
   __device__ __forceinline__ void load() {
-    if (lane < kColBlock) pend = ld_relaxed_u64(in + rpos + lane);
+    if (lane < kColBlock && in_range(in - base + rpos + lane, entries, status)) pend = ld_relaxed_u64(in + rpos + lane);
   }
   __device__ __forceinline__ bool land(int slot) {
     bool ok = lane >= kColBlock || fresh();
@@ -117,6 +119,8 @@ struct WrapRing {
     return true;
   }
   __device__ __forceinline__ bool room(int wblk) {
+    if (!in_range(own - base + wpos, entries, status) || !in_range(own - base + wpos + kColBlock - 1, entries, status))
+      return false;
     if ((wblk + 1) * kColBlock <= room_end) return true;
     const int need = (wblk + 1) * kColBlock - window;
     int seen = 0;
@@ -171,6 +175,8 @@ __global__ void __launch_bounds__(32 * kPairWarps, 1) pair_band_kernel(const Pai
     x.go = cs.go;
     x.rgb = rgb;
     x.lane = lane;
+    x.base = a.strips;
+    x.entries = a.ring_entries;
     x.prev = b > 0;
     x.next = b + 1 < a.nbands;
     x.lo_bias = 0u;

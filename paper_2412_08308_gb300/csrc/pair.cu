@@ -254,6 +254,7 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
   a.best = d_words;
   a.status = d_words + 1;
   a.sc = scr;
+  a.ring_entries = nslots * window;
   if (kernel_ms) {
     if ((e = cudaEventCreate(&sc.e0)) != cudaSuccess || (e = cudaEventCreate(&sc.e1)) != cudaSuccess)
       return pair_cuda(e, "cudaEventCreate");
@@ -267,6 +268,7 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return pair_cuda(e, "result");
   if (words[1] == SW_ETIMEOUT) return pair_fail(SW_ETIMEOUT, "sw_align_pair: a bounded device wait expired");
+  if (words[1]) return pair_fail(SW_ECUDA, "sw_align_pair: internal error: an index left its buffer (checked build)");
   if (kernel_ms) cudaEventElapsedTime(kernel_ms, sc.e0, sc.e1);
   *score = words[0];
   return SW_OK;
