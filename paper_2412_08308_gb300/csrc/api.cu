@@ -353,6 +353,9 @@ struct sw_db {
   };
   mutable std::mutex track_mu;
   mutable std::vector<std::unique_ptr<TrackLayout>> track_layouts;
+  // whether its row tracks can be kept at any lane height: at most one lane per
+  // row of the lowest one and one more per sequence
+  bool keeps_tracks() const { return (total / 8 + n) * (int64_t)sizeof(TrackLane) <= kTrackLayoutBytes; }
   // the layout for (tR, cut), built and uploaded on stream s on first use
   // (synchronising s), or nullptr: not kept (too large, too many, called on
   // another device, or a CUDA error) -- the caller then builds it itself
@@ -1222,12 +1225,38 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
                                   chain_step_cycles(packed ? kFormQPair : kFormInt32, rows, 1));
     return best;
   };
+  // Modelled time (cycles) of the intra-task launches, one CTA (and matrix) per
+  // SM: the longest matrix, or all of them over the SMs.  A chain sweeps a
+  // unit's columns one after the other, however few rows it has: 550 cycles a
+  // column for a query of one warp (500 with 32-bit cells), 1,000 + 32 per warp
+  // where its warps pass the rows on (60 to 5,000 residues against sequences of
+  // up to 35,000: 8.6 to 23 ms, within 6 %).
+  auto intra_time = [&]() {
+    double longest = 0, work = 0;
+    for (int64_t q = 0; q < n_queries; ++q) {
+      const int w = std::max(1, std::min(intra_threads() / 32, (qlen(q) + 32 * Ri - 1) / (32 * Ri)));
+      const double chunks = std::ceil(std::max(1, qlen(q)) / (32.0 * w * Ri));
+      const double column = chunks * (w > 1 ? 1000 + 32 * w : packed ? 550 : 500) * Ri / 16;
+      longest = std::max(longest, column * max_long);
+      // (pairs of sequences that could pass the 16-bit range run one by one)
+      work += column * (double)ust.prefix[(size_t)n_long] * (may_flag(q, max_long) ? 2 : 1);
+    }
+    return std::max(longest, work / sms);
+  };
   // Which kernels: the small-batch ones (band-stream jobs for the long queries
   // and transposed ones for the others, or all transposed), or the inter- and
-  // intra-task ones, by modelled time.  Above 16,384 sequences the inter-task
-  // kernel measures equal or faster (20,000 proteins, packed: 60 residues 177
-  // against 205 us, 144 336 / 302, 400 655 / 604, 1,000 1,318 / 1,318, 1,301
-  // 1,938 / 2,207), and a new database need not lay its row tracks first.
+  // intra-task ones, by modelled time.  Where the database has units past the
+  // cutover, at any size whose row tracks the database can keep: the intra-task
+  // kernel takes one such unit far longer than bands do (35,000 residues: 9.4
+  // against 0.78 ms for a 144-residue query, 18.1 against 2.1 ms for 1,301; the
+  // model picks within 5 % of the faster side up to 40,000 proteins, within 30 %
+  // at 80,000).  Without such units, up to 16,384 sequences: above, the sides
+  // differ by -23 to +85 % (17,000 to 40,000 proteins, packed: transposed jobs
+  // 0.78 to 1.2 of the inter-task time at 144 residues, 0.85 to 0.88 at 400,
+  // 0.95 to 1.0 at 1,000, 1.05 to 1.2 at 1,301, 1.0 to 1.6 at 60), the model
+  // misses by more where the sequences are short (40,000 of 10 to 60 residues x
+  // 1,301: 542 us inter-task, 986 as band-stream jobs), and a new database need
+  // not lay its row tracks first.
   bool small = o.band_stream == 2;
   if (n > 0 && n_queries > 0 && o.band_stream != 1) {
     bool any_band = false;
@@ -1236,7 +1265,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
       track_q[q] = !band_q[q];
       any_band |= band_q[q] != 0;
     }
-    if (o.band_stream == 0 && n <= 16384) {
+    if (o.band_stream == 0 && (n <= 16384 || (n_long && db->keeps_tracks()))) {
       const double tracks_a = rank_heights_of(), bands_a = any_band ? band_time() : 0.0;
       double best_small = std::max(tracks_a, bands_a) + 0.5 * std::min(tracks_a, bands_a);
       if (any_band) {  // all transposed?
@@ -1258,15 +1287,8 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
       } else {
         plan = best_plan();
         double inter = plan.time;
-        if (n_long) {  // the intra-task kernel beside it: about 4.4 int32 cells per cycle and SM
-          double m_sum = 0, m_max = 0;
-          for (int64_t q = 0; q < n_queries; ++q) {
-            m_sum += qlen(q);
-            m_max = std::max<double>(m_max, qlen(q));
-          }
-          const double rate = packed && (int64_t)sc.maxp * max_long <= sc.thresh ? 9.6 : 4.4;
-          const double cols = (double)ust.prefix[(size_t)n_long] * (packed ? 2 : 1);
-          const double intra = std::max(m_max * max_long, m_sum * cols / sms) / rate;
+        if (n_long) {  // the intra-task kernel beside it
+          const double intra = intra_time();
           inter = std::max(inter, intra) + 0.3 * std::min(inter, intra);
         }
         small = best_small < inter;
