@@ -450,8 +450,9 @@ struct sw_queries {
   // transposed jobs (small batches): database row tracks against each short query
   int64_t n_tjobs = 0, n_tbands = 0, n_tlanes = 0, track_ring_bytes = 0, qt_bytes = 16;
   int tgrid = 1, tR = 16;
+  int n_tgroups = 0;
   TrackJob *d_tjobs = nullptr;
-  int32_t *d_tjob_of = nullptr;
+  TrackGroup *d_tgroups = nullptr;
   TrackLane *d_tlanes = nullptr;
   bool tlanes_shared = false;  // d_tlanes is the database's kept lane table, not in the block
   uint8_t *d_qt = nullptr;
@@ -665,7 +666,7 @@ struct PlanScratch {
   std::vector<int32_t> bjob_of;
   std::vector<int2> btpos;
   std::vector<TrackJob> tjobs;
-  std::vector<int32_t> tjob_of;
+  std::vector<TrackGroup> tgroups;
   std::vector<TrackLane> tlanes;
   std::vector<TrackPipe> tpipes;
   TrackBins bins;
@@ -682,7 +683,7 @@ PlanScratch &plan_scratch() {
   ps.bjob_of.clear();
   ps.btpos.clear();
   ps.tjobs.clear();
-  ps.tjob_of.clear();
+  ps.tgroups.clear();
   ps.tlanes.clear();
   ps.tpipes.clear();
   ps.tw.clear();
@@ -1110,7 +1111,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   std::vector<int32_t> &bjob_of = scratch.bjob_of;
   std::vector<int2> &btpos = scratch.btpos;
   std::vector<TrackJob> &tjobs = scratch.tjobs;
-  std::vector<int32_t> &tjob_of = scratch.tjob_of;
+  std::vector<TrackGroup> &tgroups = scratch.tgroups;
   std::vector<TrackLane> &tlanes = scratch.tlanes;
   std::vector<int64_t> qt_off(std::max<int64_t>(n_queries, 1), 0);
   std::vector<int32_t> qt_npad(std::max<int64_t>(n_queries, 1), 16);
@@ -1423,12 +1424,22 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
       }
       Q->qt_bytes = std::max<int64_t>(qt, 16);
       const int32_t cut = track_cut();
-      // the jobs: each pipeline once per query (deeper pipelines first)
-      auto make_jobs = [&](const std::vector<TrackPipe> &pipes) {
+      // the jobs: each pipeline once per query, deeper pipelines first, and the
+      // order of their bands.  Job by job, the warps in flight hold a few
+      // pipelines, whose bands run about 50 steps apart and wait on one another;
+      // by level (bands with more of their job below them first) a band follows
+      // the one above it with the other jobs' bands of that depth between them.
+      // By level where those 50 steps a band outlast a band's own or the bands
+      // fill the warps twice (40 queries of 144 residues x 5 sequences of 30,000:
+      // 4.25 ms job by job, 0.72 by level; four of 100 to 400 x 1,200 of 2,500: 1.02
+      // and 0.73); else the hand-off to a neighbour on the same SM is the faster
+      // (400 residues x 4,000 proteins and 400 of 2,500: 301 and 321 us).
+      auto make_jobs = [&](const std::vector<TrackPipe> &pipes, int occ) {
         tjobs.clear();
-        tjob_of.clear();
+        tgroups.clear();
         tring = 0;
         tband = 0;
+        int32_t steps = 0;
         for (const TrackPipe &pp : pipes)
           for (int64_t q = 0; q < n_queries; ++q) {
             if (!track_q[q]) continue;
@@ -1437,14 +1448,30 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
             j.packed = pp.packed;
             j.nb = pp.nb;
             j.rows = pp.rows;
-            j.band0 = (int32_t)tband;
             j.lane0 = pp.lane0;
             j.ring0 = tring;
             tring += (int64_t)(pp.nb - 1) * qt_npad[q];
-            for (int32_t b = 0; b < pp.nb; ++b) tjob_of.push_back((int32_t)tjobs.size());
             tband += pp.nb;
+            steps = std::max(steps, (qt_npad[q] + 64) / 2);
             tjobs.push_back(j);
           }
+        if (tband >= ((int64_t)1 << 30)) return;  // (the plan is refused below)
+        const int32_t deepest = tjobs.empty() ? 0 : tjobs[0].nb;
+        int32_t start = 0;
+        if (deepest > 2 && (50 * (int64_t)(deepest - 1) > steps ||
+                            tband > 2 * (int64_t)sms * occ * (track_threads() / 32))) {
+          size_t k = 0;
+          for (int32_t below = deepest; below > 0; --below) {
+            while (k < tjobs.size() && tjobs[k].nb >= below) ++k;
+            tgroups.push_back({start, 0, 0, below});
+            start += (int32_t)k;
+          }
+        } else {
+          for (size_t k = 0; k < tjobs.size(); ++k) {
+            if (k == 0 || tjobs[k].nb != tjobs[k - 1].nb) tgroups.push_back({start, (int32_t)k, tjobs[k].nb, 0});
+            start += tjobs[k].nb;
+          }
+        }
       };
       if (any_track) {
         // the height with the least modelled time; one that its packed bands
@@ -1468,12 +1495,12 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
         const int tR = c.tR;
         tocc = c.occ;
         if (lay) {
-          make_jobs(lay->pipes);
+          make_jobs(lay->pipes, tocc);
           Q->d_tlanes = lay->d_lanes;  // the database's (not the batch's block)
           n_tlanes = lay->n_lanes;
         } else {
           lay_tracks(bins, tR, scratch.tpipes, tlanes);
-          make_jobs(scratch.tpipes);
+          make_jobs(scratch.tpipes, tocc);
           n_tlanes = (int64_t)tlanes.size();
         }
         Q->tR = tR;
@@ -1492,6 +1519,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
         Q->bone = bocc == 1 && bmax > 1;
         Q->n_tjobs = (int64_t)tjobs.size();
         Q->n_tbands = tband;
+        Q->n_tgroups = (int)tgroups.size();
         Q->n_tlanes = n_tlanes;
         Q->tlanes_shared = Q->d_tlanes != nullptr;
         Q->track_ring_bytes = 8 * tring;
@@ -1505,7 +1533,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
       bjob_of.clear();
       btpos.clear();
       tjobs.clear();
-      tjob_of.clear();
+      tgroups.clear();
       tlanes.clear();
       Q->d_tlanes = nullptr;
     }
@@ -1769,14 +1797,14 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   const size_t b_brings = Q->n_bjobs ? round_up(std::max<int64_t>(Q->band_ring_bytes, 8), 256) : 0;
   const bool tmode = Q->n_tjobs > 0;
   const size_t b_tjobs = tmode ? round_up((int64_t)sizeof(TrackJob) * Q->n_tjobs, 256) : 0;
-  const size_t b_tjobof = tmode ? round_up(4 * Q->n_tbands, 256) : 0;
+  const size_t b_tgroups = tmode ? round_up(sizeof(TrackGroup) * tgroups.size(), 256) : 0;
   const size_t b_tlanes = tmode && !Q->tlanes_shared ? round_up((int64_t)sizeof(TrackLane) * Q->n_tlanes, 256) : 0;
   const size_t b_qt = tmode ? round_up(Q->qt_bytes, 256) : 0;
   const size_t b_qtoff = tmode ? round_up(8 * nqm, 256) : 0;
   const size_t b_qtnpad = tmode ? round_up(4 * nqm, 256) : 0;
   const size_t b_trings = tmode ? round_up(std::max<int64_t>(Q->track_ring_bytes, 8), 256) : 0;
   const size_t b_scores = round_up(score_bytes, 256);
-  Q->bytes = b_scores + b_tjobs + b_tjobof + b_tlanes + b_qt + b_qtoff + b_qtnpad + b_trings + b_qres + b_sub + 2 * b_qd + b_tasks + b_itasks + b_itasks32 + b_ipos32 + b_rtasks + b_prof +
+  Q->bytes = b_scores + b_tjobs + b_tgroups + b_tlanes + b_qt + b_qtoff + b_qtnpad + b_trings + b_qres + b_sub + 2 * b_qd + b_tasks + b_itasks + b_itasks32 + b_ipos32 + b_rtasks + b_prof +
              b_gbuf + b_igbuf + b_words + b_flag + b_iflag + b_qdp + b_ptasks + b_track + b_bjobs + b_bjobof +
              b_btpos + b_brings;
   cudaMemPool_t pool = nullptr;
@@ -1810,7 +1838,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   Q->d_btpos = (int2 *)take(b_btpos);
   if (tmode) {
     Q->d_tjobs = (TrackJob *)take(b_tjobs);
-    Q->d_tjob_of = (int32_t *)take(b_tjobof);
+    Q->d_tgroups = (TrackGroup *)take(b_tgroups);
     if (!Q->tlanes_shared) Q->d_tlanes = (TrackLane *)take(b_tlanes);
     Q->d_qt = take(b_qt);
     Q->d_qt_off = (int64_t *)take(b_qtoff);
@@ -1846,7 +1874,8 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
                  (int64_t)sizeof(QDesc) * Q->npairs + (int64_t)sizeof(TrackChunk) * (int64_t)Q->track.size() +
                  (int64_t)sizeof(Task) * (Q->n_tasks + Q->n_itasks + Q->n_itasks32 + Q->n_ptasks) +
                  4 * (int64_t)ipos32.size() + 16 + (int64_t)sizeof(BandJob) * Q->n_bjobs + 4 * Q->n_bands +
-                 (int64_t)sizeof(int2) * Q->n_btargets + (int64_t)sizeof(TrackJob) * Q->n_tjobs + 4 * Q->n_tbands +
+                 (int64_t)sizeof(int2) * Q->n_btargets + (int64_t)sizeof(TrackJob) * Q->n_tjobs +
+                 (int64_t)(sizeof(TrackGroup) * tgroups.size()) +
                  (Q->tlanes_shared ? 0 : (int64_t)sizeof(TrackLane) * Q->n_tlanes) +
                  (tmode ? Q->qt_bytes + 12 * n_queries : 0);
   // stage the host tables at their offsets in the block (the rest zero:
@@ -1878,7 +1907,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   }
   if (tmode) {
     put(Q->d_tjobs, tjobs.data(), sizeof(TrackJob) * Q->n_tjobs);
-    put(Q->d_tjob_of, tjob_of.data(), 4 * Q->n_tbands);
+    put(Q->d_tgroups, tgroups.data(), sizeof(TrackGroup) * tgroups.size());
     if (!Q->tlanes_shared) put(Q->d_tlanes, tlanes.data(), sizeof(TrackLane) * Q->n_tlanes);
     uint8_t *qtp = stage.data() + (Q->d_qt - (uint8_t *)Q->block);
     memset(qtp, kPadCode, (size_t)Q->qt_bytes);
@@ -2039,7 +2068,8 @@ static int search_prepared(const sw_db *db, const sw_queries *Q, int32_t *scores
     ta.db = db->view;
     ta.lanes = Q->d_tlanes;
     ta.jobs = Q->d_tjobs;
-    ta.band_job = Q->d_tjob_of;
+    ta.groups = Q->d_tgroups;
+    ta.n_groups = Q->n_tgroups;
     ta.nbands = (int32_t)Q->n_tbands;
     ta.band_counter = w + 1;
     ta.qt = Q->d_qt;

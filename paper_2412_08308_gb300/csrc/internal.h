@@ -210,16 +210,25 @@ struct TrackJob {
   int32_t q;       // the query: the columns, and the row of scores written
   int32_t packed;  // 1: two row tracks in the 16-bit halves; 0: one track, int32 cells
   int32_t nb;      // bands
-  int32_t band0;   // global index of the job's band 0
   int32_t lane0;   // band b's lanes at TrackArgs::lanes[lane0 + 32 b ...]
   int32_t rows;    // rows per lane: the launch's, or track_long_rows() of it
   int64_t ring0;   // entry offset of ring 0 (between bands 0 and 1); rings are qt_npad[q] long
+};
+struct TrackGroup {
+  int32_t start;  // first band of the launch
+  int32_t job;    // first job
+  int32_t nb;     // bands of each job, all of them in the group; 0: by level
+  int32_t below;  // by level: bands of the job from this one on
 };
 struct TrackArgs {
   DbView db;                  // the rows' sequences
   const TrackLane *lanes;
   const TrackJob *jobs;
-  const int32_t *band_job;    // [nbands] job of each global band
+  // The bands in the order they are handed out (jobs: deeper ones first), in
+  // groups from band TrackGroup::start on: the jobs of one depth one after the
+  // other, or, by level, one band of each of the first jobs.
+  const TrackGroup *groups;
+  int32_t n_groups;
   int32_t nbands;
   int32_t *band_counter;      // (cleared by launch_trace, as is the status)
   const uint8_t *qt;          // queries padded to multiples of 16 with the pad code

@@ -271,6 +271,24 @@ __device__ __forceinline__ void track_scores(const TrackArgs &a, int32_t q, int3
   }
 }
 
+// The job of band g of the launch, and its band or (negative) how many of the
+// job's bands are left from it on.
+__device__ __forceinline__ int2 track_band_of(const TrackArgs &a, int g, int lane) {
+  int4 e = make_int4(0, 0, 1, 0);
+  for (int k = 0; k < a.n_groups; k += 32) {  // the last group that starts at or before g
+    const int4 v = k + lane < a.n_groups ? reinterpret_cast<const int4 *>(a.groups)[k + lane]
+                                         : make_int4(0x7fffffff, 0, 1, 0);
+    const uint32_t m = __ballot_sync(0xffffffffu, v.x <= g);
+    if (m == 0u) break;
+    const int src = 31 - __clz(m);
+    e = make_int4(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src),
+                  __shfl_sync(0xffffffffu, v.z, src), __shfl_sync(0xffffffffu, v.w, src));
+    if (m != 0xffffffffu) break;
+  }
+  const int i = g - e.x;
+  return e.z == 0 ? make_int2(e.y + i, -e.w) : make_int2(e.y + i / e.z, i % e.z);
+}
+
 // One band: its rows' profile, the sweep, and the scores of its sequences.
 template <int R, int UP, int UI>
 __device__ __forceinline__ bool track_band(const TrackArgs &a, uint8_t *prof, const uint8_t *score,
@@ -325,8 +343,9 @@ __global__ void __launch_bounds__(kTrackThreads, R <= 8 ? 4 : R <= 20 ? 2 : 1) b
     if (lane == 0) g = atomicAdd(a.band_counter, 1);
     g = __shfl_sync(0xffffffffu, g, 0);
     if (g >= a.nbands) break;
-    const TrackJob job = a.jobs[a.band_job[g]];
-    const int b = g - job.band0;
+    const int2 jb = track_band_of(a, g, lane);
+    const TrackJob job = a.jobs[jb.x];
+    const int b = jb.y < 0 ? job.nb + jb.y : jb.y;
     const bool packed = job.packed != 0;
     const int64_t li = (int64_t)job.lane0 + 32 * (int64_t)b + lane;
     const TrackLane L = in_range(li, a.n_lanes, a.status) ? a.lanes[li] : idle;
