@@ -202,6 +202,13 @@ struct TrackPipe {
   int32_t packed, nb, lane0, rows;  // rows per lane
 };
 
+// What the transposed jobs of one query cost a launch: bands over all
+// pipelines and the most bands of one, of the 16-bit [0] and int32 [1] tracks.
+struct TrackLoad {
+  double bands[2] = {0, 0};
+  int64_t deepest[2] = {1, 1};
+};
+
 void bin_tracks(const std::vector<int32_t> &len, int tR, int32_t cut, TrackBins &b) {
   const int tL = track_long_rows(tR);
   // tracks by the lanes free in their last band, per height
@@ -345,8 +352,7 @@ struct sw_db {
   // by every query batch that plans them
   struct TrackLayout {
     int32_t tR = 0, cut = 0;
-    int64_t bands = 0;    // bands of one query over all pipelines
-    int32_t deepest = 1;  // most bands of a pipeline
+    TrackLoad load;
     int64_t n_lanes = 0;
     std::vector<TrackPipe> pipes;
     TrackLane *d_lanes = nullptr;
@@ -379,8 +385,9 @@ struct sw_db {
     lay_tracks(b, tR, t->pipes, lanes);
     if ((int64_t)(lanes.size() * sizeof(TrackLane)) > kTrackLayoutBytes) return nullptr;
     for (const TrackPipe &p : t->pipes) {
-      t->bands += p.nb;
-      t->deepest = std::max(t->deepest, p.nb);
+      const int f = p.packed ? 0 : 1;
+      t->load.bands[f] += p.nb;
+      t->load.deepest[f] = std::max<int64_t>(t->load.deepest[f], p.nb);
     }
     t->n_lanes = (int64_t)lanes.size();
     if (!lanes.empty()) {
@@ -1116,47 +1123,56 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   std::vector<int64_t> qt_off(std::max<int64_t>(n_queries, 1), 0);
   std::vector<int32_t> qt_npad(std::max<int64_t>(n_queries, 1), 16);
   bool band_mode = false;
-  // Bands of one query in lanes of tR rows, and the most bands of one
-  // sequence, estimated from the length histogram.
-  auto track_estimate = [&](int tR, const sw_db::UnitStats &single, int32_t cut, double *bands, int64_t *deepest) {
+  // The load of one query in lanes of tR rows, estimated from the length
+  // histogram (lengths up to cut take the 16-bit tracks).
+  auto track_estimate = [&](int tR, const sw_db::UnitStats &single, int32_t cut) {
     const int tL = track_long_rows(tR);
-    double lanes = 0;
-    *bands = 0;
-    *deepest = 1;
+    TrackLoad e;
+    double lanes[2] = {0, 0};
     for (size_t h = 1; h < single.hist.size(); ++h) {
       if (!single.hist[h]) continue;
       const int64_t len = (int64_t)h * kColBlock - 7;  // (the middle of the bin)
+      const int f = len > cut ? 1 : 0;
       if (len <= 32 * tR) {
-        lanes += (double)single.hist[h] * (double)((len + tR - 1) / tR);
+        lanes[f] += (double)single.hist[h] * (double)((len + tR - 1) / tR);
       } else {
         const int64_t nb = (len + 32 * tL - 1) / (32 * tL);
-        // (two 16-bit tracks share a band; int32 ones, past the cut, do not)
-        *bands += (double)(single.hist[h] * nb) * (packed && len > cut ? 2 : 1);
-        *deepest = std::max(*deepest, nb);
+        e.bands[f] += (double)(single.hist[h] * nb);
+        e.deepest[f] = std::max(e.deepest[f], nb);
         // (short sequences fill most of what the last band leaves)
-        lanes -= 0.8 * (double)single.hist[h] * (double)(32 * tL * nb - len) / tR;
+        lanes[f] -= 0.8 * (double)single.hist[h] * (double)(32 * tL * nb - len) / tR;
       }
     }
-    *bands = std::ceil((*bands + std::max(0.0, lanes) / 32 / 0.98) * (packed ? 0.5 : 1.0));
+    for (int f = 0; f < 2; ++f)  // (two 16-bit tracks share a band)
+      e.bands[f] = std::ceil((e.bands[f] + std::max(0.0, lanes[f]) / 32 / 0.98) * (f == 0 ? 0.5 : 1.0));
+    return e;
   };
   // Modelled time (cycles) of the transposed jobs: their bands over the SM
   // sub-partitions, up to the launch's residency at a time; at least the
   // longest pipeline, whose bands start about 50 steps after one another.
-  auto track_time = [&](int tR, int occ, double bands, int64_t deepest) {
-    double work = 0, steps_max = 0, nb = 0;
+  auto track_time = [&](int tR, int occ, const TrackLoad &load) {
+    double steps_sum = 0, steps_max = 0, n_q = 0;
     for (int64_t q = 0; q < n_queries; ++q) {
       if (!track_q[q]) continue;
       const double steps = (double)(round_up(std::max(1, qlen(q)), kColBlock) + 64) / 2;
-      work += bands * steps;
+      steps_sum += steps;
       steps_max = std::max(steps_max, steps);
-      nb += bands;
+      ++n_q;
     }
-    const double parts = 4.0 * sms;
+    const double parts = 4.0 * sms, nb = n_q * (load.bands[0] + load.bands[1]);
     const int w = (int)std::max(1.0, std::min((double)occ, std::ceil(nb / parts)));
-    const double step = track_step_cycles(packed, tR, w);
-    const double all = nb > parts * w ? work * step / (parts * w) + 0.5 * steps_max * step : steps_max * step;
-    const double chain = (steps_max + 50.0 * (double)(deepest - 1)) * track_step_cycles(packed, track_long_rows(tR), w);
-    return deepest > 1 ? std::max(all, chain) : all;
+    double work = 0, step_max = 0, chain = 0;
+    for (int f = 0; f < 2; ++f) {
+      if (load.bands[f] <= 0) continue;
+      const double step = track_step_cycles(f == 0, tR, w);
+      work += load.bands[f] * steps_sum * step;
+      step_max = std::max(step_max, step);
+      if (load.deepest[f] > 1)
+        chain = std::max(chain, (steps_max + 50.0 * (double)(load.deepest[f] - 1)) *
+                                    track_step_cycles(f == 0, track_long_rows(tR), w));
+    }
+    const double all = nb > parts * w ? work / (parts * w) + 0.5 * steps_max * step_max : steps_max * step_max;
+    return std::max(all, chain);
   };
   // a sequence takes the 16-bit tracks (packed mode) unless its pair with the
   // longest of these queries could pass the 16-bit range: a length cut that
@@ -1169,10 +1185,17 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
            : (int64_t)sc.maxp * mtq <= sc.thresh ? std::numeric_limits<int32_t>::max()
                                                  : sc.thresh / sc.maxp;
   };
-  // rows per lane of the transposed jobs, in order of the modelled time
+  // rows per lane and cut of the transposed jobs, in order of the modelled
+  // time.  A deep pipeline's time is its bands' steps one after the other, and
+  // an int32 step is the shorter one (16 rows: 353 against 460 cycles), so
+  // sequences past kDeepCut may take int32 tracks where there are few of them
+  // (144 residues, packed, x one sequence of 35,000: 765 -> 605 us; x 4,000
+  // proteins and one of 9,000: 236 -> 203).
+  constexpr int32_t kDeepCut = 2048;
   struct TrackChoice {
     double time;
     int tR, occ;
+    int32_t cut;
   };
   std::vector<TrackChoice> heights;
   auto rank_heights = [&]() {
@@ -1182,13 +1205,20 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     for (const TrackHeight &h : kTrackHeights) {
       const int occ = cached_occupancy(2, h.rows, 0, gaps, 0, 0);
       if (occ <= 0) continue;
-      double bands = 0;
-      int64_t deepest = 1;
-      track_estimate(h.rows, single, cut, &bands, &deepest);
-      heights.push_back({track_time(h.rows, occ, bands, deepest), h.rows, occ});
+      heights.push_back({track_time(h.rows, occ, track_estimate(h.rows, single, cut)), h.rows, occ, cut});
+      if (cut > kDeepCut && db->max_npad > kDeepCut)
+        heights.push_back({track_time(h.rows, occ, track_estimate(h.rows, single, kDeepCut)), h.rows, occ, kDeepCut});
     }
-    std::sort(heights.begin(), heights.end(),
-              [](const TrackChoice &x, const TrackChoice &y) { return x.time < y.time; });
+    std::stable_sort(heights.begin(), heights.end(),
+                     [](const TrackChoice &x, const TrackChoice &y) { return x.time < y.time; });
+    // (the deep sequences in int32 only where that is clearly the faster: the
+    // chains' part of the model is within 20 %)
+    const auto plain = std::find_if(heights.begin(), heights.end(), [&](const TrackChoice &c) { return c.cut == cut; });
+    if (plain != heights.end()) {
+      const int32_t keep = heights[0].time < 0.8 * plain->time ? heights[0].cut : cut;
+      heights.erase(std::remove_if(heights.begin(), heights.end(), [&](const TrackChoice &c) { return c.cut != keep; }),
+                    heights.end());
+    }
     return heights.empty() ? 1e300 : heights[0].time;
   };
   auto rank_heights_of = [&]() {
@@ -1423,7 +1453,6 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
         qt += qt_npad[q];
       }
       Q->qt_bytes = std::max<int64_t>(qt, 16);
-      const int32_t cut = track_cut();
       // the jobs: each pipeline once per query, deeper pipelines first, and the
       // order of their bands.  Job by job, the warps in flight hold a few
       // pipelines, whose bands run about 50 steps apart and wait on one another;
@@ -1431,7 +1460,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
       // the one above it with the other jobs' bands of that depth between them.
       // By level where those 50 steps a band outlast a band's own or the bands
       // fill the warps twice (40 queries of 144 residues x 5 sequences of 30,000:
-      // 4.25 ms job by job, 0.72 by level; four of 100 to 400 x 1,200 of 2,500: 1.02
+      // 4.25 ms job by job, 0.69 by level; four of 100 to 400 x 1,200 of 2,500: 1.02
       // and 0.73); else the hand-off to a neighbour on the same SM is the faster
       // (400 residues x 4,000 proteins and 400 of 2,500: 301 and 321 us).
       auto make_jobs = [&](const std::vector<TrackPipe> &pipes, int occ) {
@@ -1480,18 +1509,19 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
         // that repeated searches skip the binning and the lane upload.
         TrackBins &bins = scratch.bins;
         TrackChoice c = heights[0];
-        const sw_db::TrackLayout *lay = db->track_layout(c.tR, cut, s);
-        if (lay) c.time = track_time(c.tR, c.occ, (double)lay->bands, lay->deepest);
+        const sw_db::TrackLayout *lay = db->track_layout(c.tR, c.cut, s);
+        if (lay) c.time = track_time(c.tR, c.occ, lay->load);
         for (size_t k = 1; lay && k < heights.size() && heights[k].time < c.time; ++k) {
-          const sw_db::TrackLayout *other = db->track_layout(heights[k].tR, cut, s);
+          const TrackChoice &h = heights[k];
+          const sw_db::TrackLayout *other = db->track_layout(h.tR, h.cut, s);
           if (!other) break;
-          const double t = track_time(heights[k].tR, heights[k].occ, (double)other->bands, other->deepest);
+          const double t = track_time(h.tR, h.occ, other->load);
           if (t < c.time) {
-            c = {t, heights[k].tR, heights[k].occ};
+            c = {t, h.tR, h.occ, h.cut};
             lay = other;
           }
         }
-        if (!lay) bin_tracks(db->h_len, c.tR, cut, bins);
+        if (!lay) bin_tracks(db->h_len, c.tR, c.cut, bins);
         const int tR = c.tR;
         tocc = c.occ;
         if (lay) {

@@ -61,3 +61,25 @@ def test_orders_agree(api, case, mode):
     finally:
         db.close()
     assert np.array_equal(got[0], got[1])
+
+
+# one or a few sequences past the length from which packed mode may take int32 tracks
+@pytest.mark.parametrize("lens", [[(1, 20000)], [(300, 300), (1, 2048), (1, 2049), (2, 9000)], [(300, 300), (1, 35000)],
+                                  [(40, 4000)], [(400, 2500)]])
+@pytest.mark.parametrize("q_len", [[60], [400], [144, 700], [1500]])
+def test_deep_sequences_in_either_width(api, lens, q_len):
+    rng = np.random.Generator(np.random.PCG64(len(lens) + len(q_len)))
+    seqs = [rng.integers(0, 20, size=L).astype(np.uint8) for n, L in lens for _ in range(n)]
+    qs = [rng.integers(0, 20, size=m).astype(np.uint8) for m in q_len]
+    seqs[-1][1000:1000 + len(qs[0])] = qs[0][:len(seqs[-1]) - 1000]
+    db, qs = api.Database.from_sequences(from_list(seqs)), from_list(qs)
+    try:
+        got = []
+        for opts in (None, api.options(band_stream="always"), api.options(band_stream="never")):
+            batch = api.PreparedQueries(db, qs.residues, qs.offsets, BLOSUM62, mode="packed", opts=opts)
+            got.append(batch.search().cpu().numpy())
+            batch.status()
+            batch.close()
+    finally:
+        db.close()
+    assert np.array_equal(got[0], got[2]) and np.array_equal(got[1], got[2])
