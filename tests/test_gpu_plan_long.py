@@ -47,3 +47,25 @@ def test_short_queries_leave_the_intra_task_kernel(api, n, long, mode, q_len):
     finally:
         db.close()
     assert np.array_equal(got[0], got[1])
+
+
+# more than 16,384 peptides: up to 2,500,000 residues the transposed jobs are weighed too
+@pytest.mark.parametrize("n,lo,hi", [(16384, 8, 30), (16385, 8, 30), (20000, 10, 60), (20000, 125, 125), (20001, 125, 125)])
+@pytest.mark.parametrize("mode", ["packed", "int32"])
+@pytest.mark.parametrize("q_len", [[255], [256], [1000], [30, 300]])
+def test_peptide_databases(api, n, lo, hi, mode, q_len):
+    rng = np.random.Generator(np.random.PCG64(n + hi))
+    lens = rng.integers(lo, hi + 1, size=n)
+    res = rng.integers(0, 20, size=int(lens.sum())).astype(np.uint8)
+    qs = from_list([rng.integers(0, 20, size=k).astype(np.uint8) for k in q_len])
+    db = api.Database(res, np.concatenate([[0], np.cumsum(lens)]))
+    try:
+        got = []
+        for opts in (None, api.options(band_stream="never")):
+            batch = api.PreparedQueries(db, qs.residues, qs.offsets, BLOSUM62, mode=mode, opts=opts)
+            got.append(batch.search().cpu().numpy())
+            batch.status()
+            batch.close()
+    finally:
+        db.close()
+    assert np.array_equal(got[0], got[1])
