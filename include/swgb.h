@@ -115,9 +115,11 @@ typedef struct sw_options {
                               into the two 16-bit halves where no lane can overflow (one
                               database sequence per chain), 1 = never pair (two database
                               sequences per chain for every query) */
-  int32_t band_stream;     /* 0 = auto: batches against up to 16,384 sequences run in the small-batch
-                              kernels instead of the inter- and intra-task kernels where their
-                              modelled time is less: a query of at least two bands (see
+  int32_t band_stream;     /* 0 = auto: batches run in the small-batch kernels instead of the inter-
+                              and intra-task kernels where their modelled time is less (weighed
+                              for up to 16,384 sequences, and above for databases with sequences
+                              past the cutover, up to 33 million residues, or of up to 2.5 million
+                              residues): a query of at least two bands (see
                               band_rows) against every database unit, its rows cut into bands,
                               one warp each, the bands of a query running as a pipeline over a
                               stream of units; every shorter query (or all of them, where that

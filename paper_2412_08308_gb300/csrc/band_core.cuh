@@ -167,7 +167,7 @@ struct BandLane {
   W S;                       // best so far
 
   __device__ __forceinline__ void reset(const Consts &cs) {
-    const W E0 = FORM != kFormInt32 ? (W)cs.E0W : (W)0;
+    const W E0 = FORM != kFormInt32 ? (W)cs.F0W : (W)0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       Hl[r] = (W)0;

@@ -66,8 +66,8 @@ __device__ __forceinline__ uint32_t checked_codes(uint32_t res, int32_t *status)
 }
 
 struct Consts {
-  // packed: (x, x) in both 16-bit halves
-  uint32_t goW, geW, F0W, E0W;
+  // packed: (x, x) in both 16-bit halves; F0W: E and F of the boundaries
+  uint32_t goW, geW, F0W;
   // int32
   int32_t go, ge;
 };
@@ -81,7 +81,6 @@ __device__ __forceinline__ Consts make_consts(const Scoring &sc) {
   c.geW = (uint32_t)ge * 0x10001u;
   const uint32_t ngo = (uint32_t)(-go) & 0xffffu;  // E, F start at -Go (any value <= 0 works)
   c.F0W = ngo | (ngo << 16);
-  c.E0W = c.F0W;
   c.go = go;
   c.ge = ge;
   return c;
@@ -99,13 +98,9 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 
 // Selectors.  pair(i) -> (byte i of a, its sign, byte i of b, its sign): the two
 // bytes sign-extended into the 16-bit halves (residue codes < 128 come out
-// zero-extended).  sext(i) -> byte i of a sign-extended to 32 bits.
-// one(i) -> byte i of a, zero-extended from b = 0.
+// zero-extended).  one(i) -> byte i of a, zero-extended from b = 0.
 __host__ __device__ constexpr uint32_t sel_pair(int i) {
   return (uint32_t)i | ((uint32_t)(i | 8) << 4) | ((uint32_t)(4 + i) << 8) | ((uint32_t)((4 + i) | 8) << 12);
-}
-__host__ __device__ constexpr uint32_t sel_sext(int i) {
-  return (uint32_t)i | ((uint32_t)(i | 8) << 4) | ((uint32_t)(i | 8) << 8) | ((uint32_t)(i | 8) << 12);
 }
 __host__ __device__ constexpr uint32_t sel_one(int i) { return 0x4440u | (uint32_t)i; }
 
@@ -246,7 +241,7 @@ template <int R, int FORM>
 __device__ __forceinline__ void lane_reset(LaneState<R, FORM> &st, const Consts &cs) {
   using W = Word<FORM>;
   constexpr bool PACKED = FORM != kFormInt32;
-  const W E0 = PACKED ? (W)cs.E0W : (W)0;
+  const W E0 = PACKED ? (W)cs.F0W : (W)0;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     st.Hl[r] = (W)0;

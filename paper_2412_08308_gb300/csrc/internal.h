@@ -230,7 +230,7 @@ struct TrackArgs {
   const TrackGroup *groups;
   int32_t n_groups;
   int32_t nbands;
-  int32_t *band_counter;      // (cleared by launch_trace, as is the status)
+  int32_t *band_counter;      // zeroed before the launch (a word of the batch, as is the status)
   const uint8_t *qt;          // queries padded to multiples of 16 with the pad code
   const int64_t *qt_off;      // [nq] offset of each padded query in qt
   const int32_t *qt_npad;     // [nq] padded length

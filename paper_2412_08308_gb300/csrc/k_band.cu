@@ -184,10 +184,10 @@ __global__ void __launch_bounds__(kBandStreamThreads, 1) band_stream_kernel(cons
 //
 // Two row tracks share a word in the 16-bit forms; their substitution scores
 // come from two byte tables, one per track (rows [0, 21) and [21, 42) of the
-// band's profile), paired into the two halves by a byte shuffle: the column's
-// residue code c is passed as the pair (c, c + 21) to the two-sequence cell
-// form.  (One table of query-pair words would save the shuffle but take
-// twice the shared memory, and so half the resident warps.)
+// band's profile), both read at the column's residue code and paired into the
+// two halves by a byte shuffle (TablePairProfile).  (One table of query-pair
+// words would save the shuffle but take twice the shared memory, and so half
+// the resident warps.)
 // ---------------------------------------------------------------------------
 
 // 4 warps, one per SM sub-partition: a small batch has few bands, and CTAs

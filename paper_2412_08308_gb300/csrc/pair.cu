@@ -194,8 +194,8 @@ extern "C" int sw_align_pair(const uint8_t *query, int64_t m, const uint8_t *tar
   // at least npad / (warps of the grid) columns, plus the hand-back interval
   // and the lead of a band over the one below.  32,768 columns by default:
   // shorter rings stall the last bands of a round while the band below waits
-  // for its warp (7M x 5M: 2,447 GCUPS at 8,192, 2,485 from 16,384 up; 3M x
-  // 3M: 2,281 and 2,325 from 32,768 up).
+  // for its warp (7M x 5M: 3,985 GCUPS at 8,192, 3,997 at 16,384, 4,008 at
+  // 32,768; 3M x 3M: 3,605, 3,839, 3,870 and no more above).
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = (size_t)1 << 30;
   int64_t window = o.ring_columns ? o.ring_columns : 32768;
