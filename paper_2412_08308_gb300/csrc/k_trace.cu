@@ -144,11 +144,13 @@ __global__ void __launch_bounds__(kTraceThreads, 4) trace_fill_kernel(const Trac
   const Consts cs = make_consts(a.sc);
   for (;;) {
     int g = 0;
-    if (lane == 0) g = atomicAdd(a.band_counter, 1);
+    if (lane == 0) {
+      const int32_t gave_up = *(const volatile int32_t *)a.status;
+      g = atomicAdd(a.band_counter, 1);
+      if (gave_up) g = a.nbands;  // (a wait has expired: the entries of the bands below it never come)
+    }
     g = __shfl_sync(0xffffffffu, g, 0);
     if (g >= a.nbands) break;
-    // (a wait of another band has expired: the entries of its bands below never come)
-    if (*(const volatile int32_t *)a.status != 0) break;
     const TraceHit hit = a.hits[a.band_hit[g]];
     const int b = g - hit.band0;
     __syncwarp();  // (the band before this one has read its profile, residues and slots)
