@@ -362,9 +362,9 @@ struct sw_db {
   mutable std::mutex track_mu;
   mutable std::vector<std::unique_ptr<TrackLayout>> track_layouts;
   mutable int64_t track_bytes = 0;  // of their lane tables
-  // whether its row tracks can be kept at any lane height: at most one lane per
-  // row of the lowest one and one more per sequence
-  bool keeps_tracks() const { return (total / 8 + n) * (int64_t)sizeof(TrackLane) <= kTrackLayoutBytes; }
+  // whether its row tracks can be kept in lanes of 16 rows or more (a large
+  // database's bands fill the GPU at those)
+  bool keeps_tracks() const { return (total / 16 + n) * (int64_t)sizeof(TrackLane) <= kTrackLayoutBytes; }
   // the layout for (tR, cut), built and uploaded on stream s on first use
   // (synchronising s), or nullptr: not kept (too large, too many, called on
   // another device, or a CUDA error) -- the caller then builds it itself
@@ -1207,11 +1207,13 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     heights.clear();
     const sw_db::UnitStats &single = db->units(false);
     const int32_t cut = track_cut();
+    // (beside band-stream jobs, which take longer, the fewer bands are the better)
+    const bool alone = std::find(band_q.begin(), band_q.end(), (char)1) == band_q.end();
     for (const TrackHeight &h : kTrackHeights) {
       const int occ = cached_occupancy(2, h.rows, 0, gaps, 0, 0);
       if (occ <= 0) continue;
       heights.push_back({track_time(h.rows, occ, track_estimate(h.rows, single, cut)), h.rows, occ, cut});
-      if (cut > kDeepCut && db->max_npad > kDeepCut)
+      if (alone && cut > kDeepCut && db->max_npad > kDeepCut)
         heights.push_back({track_time(h.rows, occ, track_estimate(h.rows, single, kDeepCut)), h.rows, occ, kDeepCut});
     }
     std::stable_sort(heights.begin(), heights.end(),
@@ -1281,22 +1283,25 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   };
   // Which kernels: the small-batch ones (band-stream jobs for the long queries
   // and transposed ones for the others, or all transposed), or the inter- and
-  // intra-task ones, by modelled time.  Where the database has units past the
-  // cutover, at any size whose row tracks the database can keep: the intra-task
-  // kernel takes one such unit far longer than bands do (35,000 residues: 9.4
-  // against 0.78 ms for a 144-residue query, 18.1 against 2.1 ms for 1,301; the
-  // model picks within 5 % of the faster side up to 40,000 proteins, within 30 %
-  // at 80,000).  Without such units, up to 16,384 sequences: above, the sides
-  // differ by -23 to +85 % (17,000 to 40,000 proteins, packed: transposed jobs
-  // 0.78 to 1.2 of the inter-task time at 144 residues, 0.85 to 0.88 at 400,
-  // 0.95 to 1.0 at 1,000, 1.05 to 1.2 at 1,301, 1.0 to 1.6 at 60), the model
-  // misses by more where the sequences are short (40,000 of 10 to 60 residues x
-  // 1,301: 542 us inter-task, 986 as band-stream jobs), and a new database need
-  // not lay its row tracks first.  Few residues are laid quickly, and ordinary
-  // queries against many peptides are a fifth to a third faster transposed
-  // (400 residues x 25,000 of 8 to 30: 98 us against 124; 1,000 residues, int32,
-  // x 80,000: 574 and 987; with more residues the model picks the slower side by
-  // up to 5 % at 1,000).
+  // intra-task ones, by modelled time.
+  //  - Where the database has units past the cutover, at any size whose row
+  //    tracks it can keep: the intra-task kernel takes one such unit far longer
+  //    than bands do (35,000 residues: 9.4 against 0.78 ms for a 144-residue
+  //    query, 18.1 against 2.1 ms for 1,301).  The model picks within 5 % of the
+  //    faster side up to 40,000 proteins; above 16,384 the small-batch kernels
+  //    have to be modelled a tenth faster (3,000 residues x 150,000 proteins,
+  //    less than that apart: 25.7 against 24.1 ms).
+  //  - Else up to 16,384 sequences.  Above, the sides differ by -23 to +85 %
+  //    (17,000 to 40,000 proteins, packed: transposed jobs 0.78 to 1.2 of the
+  //    inter-task time at 144 residues, 0.85 to 0.88 at 400, 0.95 to 1.0 at
+  //    1,000, 1.05 to 1.2 at 1,301, 1.0 to 1.6 at 60), the model misses by more
+  //    where the sequences are short (40,000 of 10 to 60 residues x 1,301: 542
+  //    us inter-task, 986 as band-stream jobs), and a new database need not lay
+  //    its row tracks first.
+  //  - But few residues are laid quickly, and ordinary queries against many
+  //    peptides are a fifth to a third faster transposed (400 residues x 25,000
+  //    of 8 to 30: 98 us against 124; 1,000, int32, x 80,000: 574 and 987; with
+  //    more residues the model picks the slower side by up to 5 % at 1,000).
   bool small = o.band_stream == 2;
   if (n > 0 && n_queries > 0 && o.band_stream != 1) {
     bool any_band = false;
@@ -1334,7 +1339,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
           const double intra = intra_time();
           inter = std::max(inter, intra) + 0.3 * std::min(inter, intra);
         }
-        small = best_small < inter;
+        small = best_small < (n_long && n > 16384 ? 0.9 : 1.0) * inter;
       }
     }
   }

@@ -69,3 +69,19 @@ def test_peptide_databases(api, n, lo, hi, mode, q_len):
     finally:
         db.close()
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("band", ["auto", "always", "never"])
+@pytest.mark.parametrize("mode", ["packed", "int32"])
+def test_empty_database_and_empty_batch(api, band, mode):
+    none = np.zeros(0, dtype=np.uint8)
+    q = np.arange(20, dtype=np.uint8)
+    for db_seqs, q_res, q_off in (([], q, [0, 20]), ([q, none], none, [0]), ([none, none], q, [0, 20]), ([], none, [0])):
+        db = api.Database(np.concatenate([none] + db_seqs), np.cumsum([0] + [len(s) for s in db_seqs]))
+        batch = api.PreparedQueries(db, q_res, np.array(q_off), BLOSUM62, mode=mode, opts=api.options(band_stream=band))
+        out = batch.search()
+        batch.status()
+        assert out.shape == (len(q_off) - 1, len(db_seqs)) and int(out.sum()) == (
+            0 if not any(len(s) for s in db_seqs) or len(q_off) == 1 else int(np.diag(BLOSUM62).sum()))
+        batch.close()
+        db.close()
