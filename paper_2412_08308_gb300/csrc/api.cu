@@ -299,13 +299,11 @@ void lay_tracks(const TrackBins &b, int tR, std::vector<TrackPipe> &pipes, std::
   std::stable_sort(pipes.begin(), pipes.end(), [](const TrackPipe &x, const TrackPipe &y) { return x.nb > y.nb; });
 }
 
-// Row-track layouts a database keeps (built on first use, the lane tables on
-// the device): as long as one has at most this many bytes of lanes and all of
-// them at most that many; other layouts are built for every plan.  (Five
-// heights, and per matrix up to four cuts: a count that searches in both modes
-// reach must not end the keeping.  2,000 proteins: 0.5 to 1.3 MB a layout.)
+// Row-track layouts a database keeps (built on first use, its lane table on
+// the device): at most this many, each with at most this many bytes of lanes;
+// other layouts are built for every plan.
+constexpr size_t kTrackLayouts = 8;
 constexpr int64_t kTrackLayoutBytes = (int64_t)64 << 20;
-constexpr int64_t kTrackLayoutsBytes = (int64_t)512 << 20;
 
 }  // namespace
 
@@ -361,7 +359,6 @@ struct sw_db {
   };
   mutable std::mutex track_mu;
   mutable std::vector<std::unique_ptr<TrackLayout>> track_layouts;
-  mutable int64_t track_bytes = 0;  // of their lane tables
   // whether its row tracks can be kept in lanes of 16 rows or more (a large
   // database's bands fill the GPU at those)
   bool keeps_tracks() const { return (total / 16 + n) * (int64_t)sizeof(TrackLane) <= kTrackLayoutBytes; }
@@ -373,13 +370,12 @@ struct sw_db {
     for (const std::unique_ptr<TrackLayout> &t : track_layouts)
       if (t->tR == tR && t->cut == cut) return t.get();
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev != device) {
+    if (track_layouts.size() >= kTrackLayouts || cudaGetDevice(&dev) != cudaSuccess || dev != device) {
       cudaGetLastError();
       return nullptr;
     }
     // at most one lane per track_long_rows(tR) residues and one more per sequence
-    const int64_t most = (total / track_long_rows(tR) + n) * (int64_t)sizeof(TrackLane);
-    if (most > kTrackLayoutBytes || track_bytes + most > kTrackLayoutsBytes) return nullptr;
+    if ((total / track_long_rows(tR) + n) * (int64_t)sizeof(TrackLane) > kTrackLayoutBytes) return nullptr;
     TrackBins b;
     bin_tracks(h_len, tR, cut, b);
     std::unique_ptr<TrackLayout> t(new TrackLayout());
@@ -406,7 +402,6 @@ struct sw_db {
       }
       t->d_lanes = (TrackLane *)d;
     }
-    track_bytes += t->n_lanes * (int64_t)sizeof(TrackLane);
     track_layouts.push_back(std::move(t));
     return track_layouts.back().get();
   }
