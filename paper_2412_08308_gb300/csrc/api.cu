@@ -492,18 +492,33 @@ namespace {
 // chunk for the boundary strip and the CTA barrier.  (Against the measured
 // time of the 20-query benchmark with L forced to 4..32, this model is
 // proportional to within 1.5 %.)  At least Lmin lanes.
-int choose_lanes(int m, int R, const double *fill, int Lmin = 4) {
+double lanes_cost(int m, int R, const double *fill, int L) {
+  const int LR = L * R;
+  const int C = std::max(1, (m + LR - 1) / LR);
+  const double rows = (double)C * LR;
+  const int G = 32 / L;
+  const double lane_eff = (double)(G * L) / 32.0;
+  return rows * fill[L] / lane_eff * (1.0 + 0.001 * C);
+}
+
+// The lanes with the least cost(L), at least Lmin of them.  Where the costs are
+// kept from one floor to the next (null: not), each is formed once.
+struct LaneCosts {
+  double c[33];
+  bool have = false;
+};
+template <class Cost>
+int choose_lanes(int Lmin, LaneCosts *kept, const Cost &cost) {
+  if (kept && !kept->have) {
+    for (int L = 4; L <= 32; ++L) kept->c[L] = cost(L);
+    kept->have = true;
+  }
   int bestL = Lmin;
   double best = 1e300;
   for (int L = Lmin; L <= 32; ++L) {
-    const int LR = L * R;
-    const int C = std::max(1, (m + LR - 1) / LR);
-    const double rows = (double)C * LR;
-    const int G = 32 / L;
-    const double lane_eff = (double)(G * L) / 32.0;
-    const double cost = rows * fill[L] / lane_eff * (1.0 + 0.001 * C);
-    if (cost < best - 1e-9) {
-      best = cost;
+    const double c = kept ? kept->c[L] : cost(L);
+    if (c < best - 1e-9) {
+      best = c;
       bestL = L;
     }
   }
@@ -844,6 +859,7 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     std::vector<int> plan_L;
     double time = 0;       // modelled cycles
     bool even = false;     // many tasks per CTA: no task sets the time
+    int floor_to = 32;     // up to this floor of lanes the plan stays the same
   };
   struct Part {
     int C, L;  // chunks and lanes per chain of a query's (a track plan's) chains
@@ -873,17 +889,21 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     if (work / slots < 8 * longest) {
       *even = false;
       // x: the largest length with more than j * slots tasks at least that long
+      auto longer = [&](double x) {  // tasks at least x long
+        double cnt = 0;
+        for (const Part &p : parts) {
+          const double len = x / p.C - inter_chain_lag(rows, form, p.L);
+          const size_t bin = len <= 0 ? 0 : (size_t)std::ceil(len / kColBlock);
+          cnt += bin < at_least.size() ? std::ceil((double)at_least[bin] / (W * (32 / p.L))) : 0.0;
+        }
+        return cnt;
+      };
       for (int j = 1; j <= 3 && tasks > j * slots; ++j) {
+        if (longer(bound / (j + 1)) <= j * slots) continue;  // (x is no more than that)
         double lo = 0, hi = longest;
         for (int it = 0; it < 10; ++it) {
           const double x = 0.5 * (lo + hi);
-          double cnt = 0;
-          for (const Part &p : parts) {
-            const double len = x / p.C - inter_chain_lag(rows, form, p.L);
-            const size_t bin = len <= 0 ? 0 : (size_t)std::ceil(len / kColBlock);
-            cnt += bin < at_least.size() ? std::ceil((double)at_least[bin] / (W * (32 / p.L))) : 0.0;
-          }
-          (cnt > j * slots ? lo : hi) = x;
+          (longer(x) > j * slots ? lo : hi) = x;
         }
         bound = std::max(bound, (j + 1) * lo);
       }
@@ -908,18 +928,34 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   // The plan at `rows` rows per lane with at least Lfloor lanes per chain
   // (where the query has that many): more lanes mean fewer chunks, so shorter
   // tasks, at the price of idle lanes and longer pipeline fill.
+  // (the same queries are planned at many floors: costs that do not depend on the
+  // floor are kept, and a floor that changes no choice is not planned.  31 queries
+  // of 19 to 674 residues x 266 sequences: preparing 397 -> 219 us; four of 56 to
+  // 68 x 615 95 -> 51)
+  auto floor_of_any = [](int m, int rows) { return std::min(32, std::max(4, (m + rows - 1) / rows)); };
+  std::vector<LaneCosts> kept_costs[7];  // by rows / 4: of each query, then of each group
   auto make_plan = [&](int rows, int Lfloor) {
     InterPlan P;
     P.R = rows;
+    std::vector<LaneCosts> &kept = kept_costs[rows / 4];
+    if (kept.empty() && n_queries <= 256) kept.resize((size_t)n_queries + 2 * elig.size());
+    auto kept_of = [&](size_t k) { return kept.empty() ? nullptr : &kept[k]; };
     const double *fl = fill_of(packed ? kFormPacked : kFormInt32, rows), *flq = fill_of(kFormQPair, rows);
-    auto floor_of = [&](int m) { return std::min({32, Lfloor, std::max(4, (m + rows - 1) / rows)}); };
+    auto floor_of = [&](int m) { return std::min(Lfloor, floor_of_any(m, rows)); };
     auto chunks_of = [&](int32_t q, int L) { return std::max(1, (qlen(q) + L * rows - 1) / (L * rows)); };
+    // (a choice of L stays while the floor is at most L, or is bound by the length)
+    auto chosen = [&](int m, int L) {
+      if (L < floor_of_any(m, rows)) P.floor_to = std::min(P.floor_to, L);
+      return L;
+    };
     P.L.resize((size_t)n_queries);
     for (int64_t q = 0; q < n_queries; ++q) {
       const int m = std::max(1, qlen(q));
       P.L[q] = forceL ? forceL
-               : q > 0 && qlen(q) == qlen(q - 1) ? P.L[q - 1]  // (batches of one length: chosen once)
-                                                 : choose_lanes(m, rows, fl, floor_of(m));
+               : q > 0 && qlen(q) == qlen(q - 1)
+                   ? P.L[q - 1]  // (batches of one length: chosen once)
+                   : chosen(m, choose_lanes(floor_of(m), kept_of((size_t)q),
+                                            [&](int L) { return lanes_cost(m, rows, fl, L); }));
     }
     P.in_track.assign((size_t)n_queries, 0);
     if (!elig.empty()) {
@@ -941,39 +977,29 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
       // best L for a group packed into two tracks, and its modelled cost
       int last_a = -1, last_b = -1, last_L = 4;
       double last_cost = 0;
-      auto plan_group = [&](const int32_t *g0, const int32_t *g1, std::vector<int32_t> *tr, int *Lout) {
-        auto pack = [&](int L, std::vector<int32_t> *out) {
-          int64_t load[2] = {0, 0};
-          for (const int32_t *q = g0; q < g1; ++q) {
-            const int t = load[1] < load[0] ? 1 : 0;
-            if (out) out[t].push_back(*q);
-            load[t] += chunks_of(*q, L);
-          }
-          return std::max(load[0], load[1]);
-        };
+      auto pack = [&](const int32_t *g0, const int32_t *g1, int L, std::vector<int32_t> *out) {
+        int64_t load[2] = {0, 0};
+        for (const int32_t *q = g0; q < g1; ++q) {
+          const int t = load[1] < load[0] ? 1 : 0;
+          if (out) out[t].push_back(*q);
+          load[t] += chunks_of(*q, L);
+        }
+        return std::max(load[0], load[1]);
+      };
+      auto plan_group = [&](const int32_t *g0, const int32_t *g1, size_t key, int *Lout) {
         auto cost_of = [&](int L) {
-          const double eff = (double)((32 / L) * L) / 32.0, chunks = (double)pack(L, nullptr);
+          const double eff = (double)((32 / L) * L) / 32.0, chunks = (double)pack(g0, g1, L, nullptr);
           return chunks * L * rows * flq[L] / eff * (1.0 + 0.002 * chunks / std::max<double>(1.0, (double)(g1 - g0)));
         };
         int Lp = forceL ? forceL : 4;
         // (neighbouring pairs of the same two lengths: chosen once)
         const bool again = g1 - g0 == 2 && last_a == qlen(g0[0]) && last_b == qlen(g0[1]);
         if (again) {
-          pack(last_L, tr);
           *Lout = last_L;
           return last_cost;
         }
-        if (!forceL) {
-          double best = 1e300;
-          for (int L = floor_of(qlen(*g0)); L <= 32; ++L) {
-            const double c = cost_of(L);
-            if (c < best - 1e-9) {
-              best = c;
-              Lp = L;
-            }
-          }
-        }
-        pack(Lp, tr);
+        if (!forceL)
+          Lp = chosen(qlen(*g0), choose_lanes(floor_of(qlen(*g0)), kept_of((size_t)n_queries + key), cost_of));
         *Lout = Lp;
         const double cost = cost_of(Lp);
         if (g1 - g0 == 2) {
@@ -991,27 +1017,30 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
       };
       const int64_t ne = (int64_t)elig.size();
       // grouped tracks
-      std::vector<std::vector<int32_t>> tA, tB;
-      std::vector<int> LA, LB;
+      struct Group {
+        int64_t i0, i1;  // of elig
+        int L;
+      };
+      std::vector<Group> gA, gB;
       double costA = 0, costB = 0;
       const int64_t tiles8 = std::max<int64_t>(1, (Q->n_single + 31) / 32);
       int64_t K = std::max<int64_t>((8 * 2 * (int64_t)sms + tiles8 - 1) / tiles8, std::min<int64_t>(8, ne / 8));
       K = std::max<int64_t>(1, std::min<int64_t>(K, ne / 2));
-      auto add = [&](int64_t i0, int64_t i1, std::vector<std::vector<int32_t>> &t, std::vector<int> &Ls) {
-        std::vector<int32_t> tr[2];
+      gA.reserve((size_t)K);
+      gB.reserve((size_t)(ne / 2));
+      // (key: groups from 0, pairs from the count of eligible queries)
+      auto add = [&](int64_t i0, int64_t i1, int64_t key, std::vector<Group> &g) {
         int Lp = 4;
-        const double c = plan_group(elig.data() + i0, elig.data() + i1, tr, &Lp);
-        t.push_back(std::move(tr[0]));
-        t.push_back(std::move(tr[1]));
-        Ls.push_back(Lp);
+        const double c = plan_group(elig.data() + i0, elig.data() + i1, (size_t)key, &Lp);
+        g.push_back({i0, i1, Lp});
         return c;
       };
-      for (int64_t k = 0; k < K; ++k) costA += add(ne * k / K, ne * (k + 1) / K, tA, LA);
+      for (int64_t k = 0; k < K; ++k) costA += add(ne * k / K, ne * (k + 1) / K, k, gA);
       // pairs
       std::vector<int32_t> soloB;
       for (int64_t i = 0; i < ne; ++i) {
         if (i + 1 < ne && 4 * (int64_t)qlen(elig[i + 1]) >= 3 * (int64_t)qlen(elig[i])) {
-          costB += add(i, i + 2, tB, LB);
+          costB += add(i, i + 2, ne + i, gB);
           ++i;
         } else {
           soloB.push_back(elig[i]);
@@ -1019,13 +1048,13 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
         }
       }
       for (int32_t q : elig) P.in_track[q] = 1;
-      if (costB < costA) {
-        P.tracks = std::move(tB);
-        P.plan_L = std::move(LB);
+      if (costB < costA)
         for (int32_t q : soloB) P.in_track[q] = 0;
-      } else {
-        P.tracks = std::move(tA);
-        P.plan_L = std::move(LA);
+      const std::vector<Group> &groups = costB < costA ? gB : gA;
+      P.tracks.resize(2 * groups.size());
+      for (size_t k = 0; k < groups.size(); ++k) {
+        pack(elig.data() + groups[k].i0, elig.data() + groups[k].i1, groups[k].L, &P.tracks[2 * k]);
+        P.plan_L.push_back(groups[k].L);
       }
     }
     std::vector<Part> solo, pairs;
@@ -1062,8 +1091,28 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     static const int kFloors[] = {5, 6, 8, 10, 12, 16, 20, 24, 32};
     InterPlan best;
     bool first = true;
+    int floor_to[7] = {0};  // by rows / 4: floors up to it give the plan seen last
+    int32_t m_max = 1;
+    for (int64_t q = 0; q < n_queries; ++q) m_max = std::max(m_max, qlen(q));
+    // the least a plan can take: the longest query's chunks over the longest
+    // short unit, in either form, with the warp alone on its SM sub-partition
+    auto at_least = [&](int rows, int Lfloor) {
+      double t = 1e300;
+      for (int form : {(int)kFormPacked, (int)kFormQPair, (int)kFormInt32}) {
+        if (packed == (form == kFormInt32)) continue;
+        double steps = 1e300;
+        for (int L = std::min(Lfloor, floor_of_any(m_max, rows)); L <= 32; ++L)
+          steps = std::min(steps, (double)((m_max + L * rows - 1) / (L * rows)) *
+                                      (double)round_up(max_short + inter_chain_lag(rows, form, L), kColBlock));
+        t = std::min(t, steps * chain_step_cycles(form, rows, 1));
+      }
+      return t;
+    };
     auto consider = [&](int rows, int Lfloor) {
+      if (Lfloor <= floor_to[rows / 4]) return false;
+      if (!first && !forceL && n_queries > 1 && n_short > 0 && at_least(rows, Lfloor) >= best.time) return false;
       InterPlan P = make_plan(rows, Lfloor);
+      floor_to[rows / 4] = P.floor_to;
       const bool even = P.even;
       if (first || P.time < best.time * (1 - 1e-9)) best = std::move(P);
       first = false;
