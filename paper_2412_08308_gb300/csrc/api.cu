@@ -1278,18 +1278,22 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     return 0.0;
   };
   // Modelled time (cycles) of the band-stream jobs of the queries in band_q:
-  // padded cells at the kernel's rate, or one stream's columns and the bands'
+  // cells at the kernel's rate, or one stream's columns and the bands'
   // hand-offs one after another (from timings of one query of 1,301 to 6,000
-  // residues x 500 to 40,000 proteins, within 20 %).
+  // residues x 500 to 40,000 proteins, within 20 %).  A band's last lane ends a
+  // unit 31 columns after its first, which is a tenth of a protein and more
+  // than a peptide: 4,852 residues x 58,000 of about 20, int32, 7.3 ms (2.5 by the
+  // sequences' own cells; 3.4 inter-task, 2.2 transposed).
   auto band_time = [&]() {
     double thr = 0, lat = 0;
     const int brows = 32 * bR;
+    const double columns = (double)db->units(false).prefix[(size_t)n] + 32.0 * (double)n;
     const double widest = Q->n_units > 0 ? (double)unit_len(0) : 0.0;
     for (int64_t q = 0; q < n_queries; ++q) {
       if (!band_q[q]) continue;
       const double nb = (double)((qlen(q) + brows - 1) / brows), rows = nb * brows;
       const bool i32 = !packed || may_flag(q, (int32_t)widest);  // (some units in int32: their columns set the pace)
-      thr += rows * (double)db->total / (packed ? 2246 : 1329);
+      thr += rows * columns / (packed ? 2510 : 1485);
       lat = std::max(lat, packed && !i32 ? 528 * widest + 24800 * nb : (packed ? 180 : 310) * widest + 27000 * nb);
     }
     return 0.95 * std::max(thr, lat) + 0.15 * std::min(thr, lat);
