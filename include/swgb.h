@@ -118,9 +118,9 @@ typedef struct sw_options {
   int32_t band_stream;     /* 0 = auto: batches run in the small-batch kernels instead of the inter-
                               and intra-task kernels where their modelled time is less (weighed
                               for up to 16,384 sequences, and above for databases with sequences
-                              past the cutover, up to 60 million residues, or of up to 2.5 million
-                              residues): a query of at least two bands (see
-                              band_rows) against every database unit, its rows cut into bands,
+                              past the cutover, up to 60 million residues, or of at most 200
+                              residues on average, up to 10 million): a query of at least two bands
+                              (see band_rows) against every database unit, its rows cut into bands,
                               one warp each, the bands of a query running as a pipeline over a
                               stream of units; every shorter query (or all of them, where that
                               takes less) transposed, the database sequences stacked as rows in

@@ -1339,17 +1339,18 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   //    faster side up to 40,000 proteins; above 16,384 the small-batch kernels
   //    have to be modelled a tenth faster (3,000 residues x 150,000 proteins,
   //    less than that apart: 25.7 against 24.1 ms).
-  //  - Else up to 16,384 sequences.  Above, the sides differ by -23 to +85 %
-  //    (17,000 to 40,000 proteins, packed: transposed jobs 0.78 to 1.2 of the
-  //    inter-task time at 144 residues, 0.85 to 0.88 at 400, 0.95 to 1.0 at
-  //    1,000, 1.05 to 1.2 at 1,301, 1.0 to 1.6 at 60), the model misses by more
-  //    where the sequences are short (40,000 of 10 to 60 residues x 1,301: 542
-  //    us inter-task, 986 as band-stream jobs), and a new database need not lay
-  //    its row tracks first.
-  //  - But few residues are laid quickly, and ordinary queries against many
-  //    peptides are a fifth to a third faster transposed (400 residues x 25,000
-  //    of 8 to 30: 98 us against 124; 1,000, int32, x 80,000: 574 and 987; with
-  //    more residues the model picks the slower side by up to 5 % at 1,000).
+  //  - Else up to 16,384 sequences, or of 200 residues on average at most (and
+  //    10 million together): longer ones are laid in row tracks too slowly for a
+  //    new database, for sides that differ little (17,000 to 40,000 proteins,
+  //    packed: transposed jobs 0.78 to 1.2 of the inter-task time at 144
+  //    residues, 0.85 to 0.88 at 400, 0.95 to 1.0 at 1,000, 1.05 to 1.2 at
+  //    1,301, 1.0 to 1.6 at 60), but the shorter the sequences the more of the
+  //    inter-task kernel's steps are fill (144 residues, packed, x 17,000 of
+  //    about 60: 102 us transposed, 172 inter-task; 1,000 x 60,000 of about 20
+  //    449 and 945).  Its model is low there by up to a half where the sequences
+  //    are the shortest or the query has 200 residues or more, and the transposed
+  //    jobs' is for a query of 60 or less: a factor weighs them (17,000 to 80,000
+  //    sequences of 10 to 200 on average x 40 to 1,000 residues, both modes).
   bool small = o.band_stream == 2;
   if (n > 0 && n_queries > 0 && o.band_stream != 1) {
     bool any_band = false;
@@ -1360,7 +1361,10 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     }
     int32_t m_max = 0;
     for (int64_t q = 0; q < n_queries; ++q) m_max = std::max(m_max, qlen(q));
-    const bool peptides = !n_long && !any_band && m_max >= 256 && db->total <= 2500000;
+    const bool peptides = !n_long && n > 16384 && db->total <= std::min<int64_t>(200 * n, 10000000);
+    const auto ramp = [](double x, double lo, double hi) { return std::min(1.0, std::max(0.0, (x - lo) / (hi - lo))); };
+    const double peptide_factor =
+        (0.75 + 0.4 * ramp(m_max, 60, 300)) * (1.2 - 0.2 * ramp((double)db->total / (double)n, 30, 100));
     if (o.band_stream == 0 && (n <= 16384 || (n_long && db->keeps_tracks()) || peptides)) {
       const double tracks_a = rank_heights_of(), bands_a = any_band ? band_time() : 0.0;
       double best_small = std::max(tracks_a, bands_a) + 0.5 * std::min(tracks_a, bands_a);
@@ -1387,7 +1391,8 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
           const double intra = intra_time();
           inter = std::max(inter, intra) + 0.3 * std::min(inter, intra);
         }
-        small = best_small < (n_long && n > 16384 ? 0.9 : 1.0) * inter;
+        const bool bands = std::find(band_q.begin(), band_q.end(), (char)1) != band_q.end();
+        small = best_small < (peptides && !bands ? peptide_factor : n_long && n > 16384 ? 0.9 : 1.0) * inter;
       }
     }
   }

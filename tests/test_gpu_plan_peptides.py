@@ -62,3 +62,19 @@ def _compare(api, n, lo, hi, q_len, mode, long=()):
 def test_long_queries_against_peptides(api, n, q_len, mode, long):
     auto, never, always = _compare(api, n, 10, 40, q_len, mode, long)
     assert auto < 1.5 * min(never, always), (auto, never, always)
+
+
+# more than 16,384 short sequences (inter-task alone: 1.7 to 2.1 times the transposed jobs' time)
+@pytest.mark.parametrize("n,lo,hi,q_len", [(17000, 1, 200, [300]), (60000, 1, 60, [800]), (60000, 1, 60, [1000])])
+@pytest.mark.parametrize("mode", ["packed", "int32"])
+def test_many_short_sequences(api, n, lo, hi, q_len, mode):
+    auto, never, always = _compare(api, n, lo, hi, q_len, mode, [1000])
+    assert auto < 1.4 * min(never, always), (auto, never, always)
+
+
+# the edges of the rule: 16,384 sequences, 200 residues on average, 10 million together
+@pytest.mark.parametrize("n,length", [(16384, 200), (16385, 200), (16385, 201), (50000, 200), (50001, 200)])
+@pytest.mark.parametrize("q_len", [[1], [59, 61], [300], [1024]])
+@pytest.mark.parametrize("mode", ["packed", "int32"])
+def test_edges_of_the_rule(api, n, length, q_len, mode):
+    _compare(api, n, length, length, q_len, mode)
