@@ -1350,7 +1350,9 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
   //    449 and 945).  Its model is low there by up to a half where the sequences
   //    are the shortest or the query has 200 residues or more, and the transposed
   //    jobs' is for a query of 60 or less: a factor weighs them (17,000 to 80,000
-  //    sequences of 10 to 200 on average x 40 to 1,000 residues, both modes).
+  //    sequences of 10 to 200 on average x 40 to 1,000 residues, both modes).  Not
+  //    above 1 for packed batches that fill the query tracks (256 queries of 30 to
+  //    285 x 60,000 of about 30: 20.0 ms inter-task, 23.9 transposed).
   bool small = o.band_stream == 2;
   if (n > 0 && n_queries > 0 && o.band_stream != 1) {
     bool any_band = false;
@@ -1363,8 +1365,9 @@ static int prepare_queries(const sw_db *db, const uint8_t *queries, const int64_
     for (int64_t q = 0; q < n_queries; ++q) m_max = std::max(m_max, qlen(q));
     const bool peptides = !n_long && n > 16384 && db->total <= std::min<int64_t>(200 * n, 10000000);
     const auto ramp = [](double x, double lo, double hi) { return std::min(1.0, std::max(0.0, (x - lo) / (hi - lo))); };
-    const double peptide_factor =
+    double peptide_factor =
         (0.75 + 0.4 * ramp(m_max, 60, 300)) * (1.2 - 0.2 * ramp((double)db->total / (double)n, 30, 100));
+    if (packed && n_queries >= 16) peptide_factor = std::min(1.0, peptide_factor);
     if (o.band_stream == 0 && (n <= 16384 || (n_long && db->keeps_tracks()) || peptides)) {
       const double tracks_a = rank_heights_of(), bands_a = any_band ? band_time() : 0.0;
       double best_small = std::max(tracks_a, bands_a) + 0.5 * std::min(tracks_a, bands_a);
